@@ -18,7 +18,9 @@ __device__ __forceinline__ void add_ll(long long *p, long long v) {
 
 // ---------------------------------------------------------------- int8 lattices
 // E = -sum_{i,d} J_{i,d} s_i s_{i+d}, M = sum_i s_i; integer sums, so the
-// atomic accumulation order does not matter.
+// atomic accumulation order does not matter.  Any even L, with or without
+// couplings; site indices are 32-bit (spin_init bounds the lattices) and the
+// coordinates come from multiply-high divisions.
 __global__ void measure_i8_kernel(const int8_t *__restrict__ s, const int8_t *__restrict__ J,
                                   Geom g, long long *__restrict__ E, long long *__restrict__ M) {
   griddep_wait();
@@ -26,18 +28,19 @@ __global__ void measure_i8_kernel(const int8_t *__restrict__ s, const int8_t *__
   const int64_t lat = blockIdx.y;
   const int8_t *sl = s + lat * g.N;
   const int8_t *Jr = J ? J + (lat % g.n_real) * (int64_t)g.dim * g.N : nullptr;
-  const int L = g.L;
-  const int64_t LL = (int64_t)L * L;
+  const uint32_t L = (uint32_t)g.L, LL = L * L, N = (uint32_t)g.N;
   long long e = 0, m = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % L), y = (int)((i / L) % L), z = g.dim == 3 ? (int)(i / LL) : 0;
+  for (uint64_t i64 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i64 < N;
+       i64 += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = (uint32_t)i64;
+    const uint32_t row = fdiv(i, g.fL), x = i - row * L;
+    const uint32_t z = g.dim == 3 ? fdiv(row, g.fL) : 0u, y = row - z * L;
     const int si = sl[i];
-    const int64_t ixp = i - x + (x == L - 1 ? 0 : x + 1);
-    const int64_t iyp = y == L - 1 ? i - (int64_t)(L - 1) * L : i + L;
+    const uint32_t ixp = x == L - 1 ? i - x : i + 1;
+    const uint32_t iyp = y == L - 1 ? i - (L - 1) * L : i + L;
     int bonds = (Jr ? Jr[i] : 1) * sl[ixp] + (Jr ? Jr[g.N + i] : 1) * sl[iyp];
     if (g.dim == 3) {
-      const int64_t izp = z == L - 1 ? i - (int64_t)(L - 1) * LL : i + LL;
+      const uint32_t izp = z == L - 1 ? i - (L - 1) * LL : i + LL;
       bonds += (Jr ? Jr[2 * g.N + i] : 1) * sl[izp];
     }
     e -= si * bonds;
@@ -51,48 +54,69 @@ __global__ void measure_i8_kernel(const int8_t *__restrict__ s, const int8_t *__
   }
 }
 
-// 2D ferromagnet, L % 16 == 0: one thread per 16-byte row segment.  For +-1
-// bytes bit 1 is set iff s = -1, so antiparallel bonds to the right and
-// downward neighbours are popcounts of (a ^ b) & 0x02..; E = 2 n_anti - 2N,
-// M = N - 2 n_down.
-__global__ void measure2d_i8_kernel(const int8_t *__restrict__ s, int L, long long *__restrict__ E,
-                                    long long *__restrict__ M) {
+// Ferromagnets with L % 8 == 0: a thread counts the 8-byte chunk m of a row
+// through len planes (3D; row y of planes z0 .. ) or len rows (2D; rows
+// y0 .. ), keeping the next plane's (row's) chunk for its next step, so each
+// byte is fetched from memory about once: antiparallel bonds to x + 1, to
+// y + 1 and, in 3D, to z + 1 by popcounts of (a ^ b) & 0x02.. (bit 1 of a
+// +-1 byte is set for -1), E = 2 n_anti - dim N, M = N - 2 n_down.  Bound by
+// memory: the per-site form above with its three divisions and byte loads
+// took 1276 us for one 3D lattice of L = 512, where 134 MB need 20 us at the
+// measured copy rate; a call of four sweeps and one measurement there went
+// from 2067 to 859 us.  Grid: (tiles of chunks x rows, segments, lattices);
+// the blocks of segment 0 and tile 0 add the constants.
+template <int kDim>
+__global__ void __launch_bounds__(256) measure_chunks_i8_kernel(const int8_t *__restrict__ s, int L, int tiles_x,
+                                                                int len, long long *__restrict__ E,
+                                                                long long *__restrict__ M) {
+  __shared__ int red[8][2];
   griddep_wait();
   griddep_release();
-  const int64_t lat = blockIdx.y;
-  const int8_t *sl = s + lat * (int64_t)L * L;
-  const uint32_t segs = (uint32_t)(L >> 4);
-  const uint32_t total = segs * (uint32_t)L;
-  const uint64_t B1 = 0x0202020202020202ull;
-  long long anti = 0, down = 0;
-  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
-    const uint32_t y = k / segs, sg = k - y * segs;
-    const int8_t *row = sl + (int64_t)y * L;
-    const int8_t *nrow = sl + (int64_t)(y == (uint32_t)L - 1 ? 0 : y + 1) * L;
-    const uint4 c = *reinterpret_cast<const uint4 *>(row + 16 * sg);
-    const uint4 d = *reinterpret_cast<const uint4 *>(nrow + 16 * sg);
-    const uint64_t c0 = (uint64_t)c.x | ((uint64_t)c.y << 32), c1 = (uint64_t)c.z | ((uint64_t)c.w << 32);
-    const uint64_t d0 = (uint64_t)d.x | ((uint64_t)d.y << 32), d1 = (uint64_t)d.z | ((uint64_t)d.w << 32);
-    const uint64_t nb = (uint8_t)row[sg == segs - 1 ? 0 : 16 * sg + 16];
-    const uint64_t r0 = (c0 >> 8) | (c1 << 56), r1 = (c1 >> 8) | (nb << 56);
-    anti += __popcll((c0 ^ r0) & B1) + __popcll((c1 ^ r1) & B1) + __popcll((c0 ^ d0) & B1) +
-            __popcll((c1 ^ d1) & B1);
-    down += __popcll(c0 & B1) + __popcll(c1 & B1);
+  constexpr uint64_t kBit1 = 0x0202020202020202ull;
+  const int chunks = L >> 3;
+  const int tile_y = blockIdx.x / tiles_x, tile_x = blockIdx.x - tile_y * tiles_x;
+  const int m = tile_x * blockDim.x + threadIdx.x;
+  // 3D: row y of the planes z0 ..; 2D: the rows z0 .. of the one plane
+  const int ty = tile_y * blockDim.y + threadIdx.y;
+  const int y = kDim == 3 ? ty : 0;
+  const int z0 = kDim == 3 ? blockIdx.y * len : ty * len;
+  const int64_t LL = (int64_t)L * L, N = kDim == 3 ? LL * L : LL;
+  const int64_t zs = kDim == 3 ? LL >> 3 : chunks;  // words from one step to the next
+  const int64_t lat = blockIdx.z;
+  int anti = 0, down = 0;
+  if (m < chunks && y < L && z0 < L) {
+    const int z1 = min(z0 + len, L);
+    const uint64_t *col = reinterpret_cast<const uint64_t *>(s + lat * N + (int64_t)y * L) + m;
+    const int64_t dd = (int64_t)((y == L - 1 ? 0 : y + 1) - y) * chunks;  // to row y + 1
+    const int64_t dx = m == chunks - 1 ? 1 - chunks : 1;                  // to the next chunk of the row
+    const uint64_t *cz = col + (int64_t)z0 * zs;
+    uint64_t C = *cz;
+#pragma unroll 4
+    for (int z = z0; z < z1; ++z) {
+      const uint64_t Bk = z == L - 1 ? col[0] : cz[zs];
+      const uint64_t nb = *reinterpret_cast<const uint8_t *>(cz + dx);
+      const uint64_t R = (C >> 8) | (nb << 56);
+      anti += __popcll((C ^ R) & kBit1) + __popcll((C ^ Bk) & kBit1);
+      if (kDim == 3) anti += __popcll((C ^ cz[dd]) & kBit1);
+      down += __popcll(C & kBit1);
+      C = Bk;
+      cz += zs;
+    }
   }
-  anti = warp_sum(anti);
-  down = warp_sum(down);
-  if ((threadIdx.x & 31) == 0) {
-    if (E) add_ll(&E[lat], 2 * anti);
-    if (M) add_ll(&M[lat], -2 * down);
+  anti = __reduce_add_sync(0xffffffffu, anti);
+  down = __reduce_add_sync(0xffffffffu, down);
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, warps = (blockDim.x * blockDim.y + 31) >> 5;
+  if ((tid & 31) == 0) {
+    red[tid >> 5][0] = anti;
+    red[tid >> 5][1] = down;
   }
-}
-
-__global__ void add_per_lattice_kernel(long long *__restrict__ v, int64_t n, long long c) {
-  griddep_wait();
-  griddep_release();
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    v[k] += c;
+  __syncthreads();
+  if (tid != 0) return;
+  long long a = 0, d = 0;
+  for (int k = 0; k < warps; ++k) a += red[k][0], d += red[k][1];
+  const bool first = blockIdx.x == 0 && blockIdx.y == 0;
+  if (E) add_ll(&E[lat], 2 * a - (first ? kDim * (long long)N : 0));
+  if (M) add_ll(&M[lat], (first ? (long long)N : 0) - 2 * d);
 }
 
 // q_{t,r} = sum_i s_i^(0) s_i^(1) between sets 0 and 1.
@@ -605,16 +629,21 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
   }
   cudaError_t e = cudaSuccess;
   if (h->d.layout == SPIN_I8) {
-    if ((E || M) && !J && g.dim == 2 && g.L % 16 == 0) {
-      const int64_t segs = (int64_t)g.L * (g.L / 16);
-      e = launch_dependent(measure2d_i8_kernel, dim3(capped(segs, 2048), (unsigned)nl), dim3(256), 0, st,
-                           (const int8_t *)h->spins, g.L, (long long *)E, (long long *)M);
-      if (e == cudaSuccess && E)
-        e = launch_dependent(add_per_lattice_kernel, dim3(capped(nl, 4096)), dim3(256), 0, st, (long long *)E, nl,
-                             -2 * (long long)g.N);
-      if (e == cudaSuccess && M)
-        e = launch_dependent(add_per_lattice_kernel, dim3(capped(nl, 4096)), dim3(256), 0, st, (long long *)M, nl,
-                             (long long)g.N);
+    if ((E || M) && !J && g.L % 8 == 0) {
+      // full warps (the block is 256 threads); len steps per thread: few
+      // enough blocks that their atomics do not queue, enough to fill the GPU
+      const int chunks = g.L / 8;
+      int bx = 1;
+      while (bx < chunks && bx < 64) bx *= 2;
+      const int by = 256 / bx, tiles_x = (chunks + bx - 1) / bx;
+      int len = 16;
+      while (len > 1 && nl * (g.N / 8) / len < 152 * 1024) len /= 2;
+      const int segs = (g.L + len - 1) / len;
+      const dim3 grid((unsigned)(tiles_x * (((g.dim == 3 ? g.L : segs) + by - 1) / by)),
+                      g.dim == 3 ? (unsigned)segs : 1u, (unsigned)nl);
+      e = launch_dependent(g.dim == 3 ? measure_chunks_i8_kernel<3> : measure_chunks_i8_kernel<2>, grid,
+                           dim3(bx, by), 0, st, (const int8_t *)h->spins, g.L, tiles_x, len, (long long *)E,
+                           (long long *)M);
     } else if (E || M) {
       e = launch_dependent(measure_i8_kernel, dim3(capped(g.N, 1024), (unsigned)nl), dim3(256), 0, st,
                            (const int8_t *)h->spins, (const int8_t *)J, g, (long long *)E, (long long *)M);
