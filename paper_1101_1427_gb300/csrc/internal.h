@@ -111,21 +111,33 @@ cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, in
                            const int64_t *energies);
 
 // Launches kernel k as a programmatic dependent of the previous work in
-// stream s (the kernel must call griddep_wait() before touching memory).
+// stream s (the kernel must call griddep_wait() before touching memory), in
+// clusters of `cluster` CTAs along x.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_dependent(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                             Args... args) {
-  cudaLaunchAttribute attr[1];
+cudaError_t launch_clusters(void (*k)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t s,
+                            Args... args) {
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
+
+// The same without clusters.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             Args... args) {
+  return launch_clusters(k, grid, block, 1, smem, s, args...);
 }
 
 // rng.cu

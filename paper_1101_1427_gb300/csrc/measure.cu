@@ -462,24 +462,22 @@ __global__ void __launch_bounds__(kRowThreads, 14) measure_msc_rows_kernel(const
 // ---------------------------------------------------------------- Heisenberg
 // Per-block partial sums in double, then a fixed-order second pass, so the
 // result does not depend on scheduling.
-constexpr int kHeisBlocks = 64;
-
+template <int kC>
 __global__ void measure_heis_kernel(const float4 *__restrict__ s, Geom g,
                                     double *__restrict__ partial) {
   griddep_wait();
   griddep_release();
   const int64_t lat = blockIdx.y;
-  heis_block_partials(s + lat * g.N, g.L, g.dim, g.N, blockIdx.x, gridDim.x,
-                      partial + (lat * gridDim.x + blockIdx.x) * 4);
+  heis_block_partials<kC>(s + lat * g.N, (uint32_t)g.L, g.fL, g.dim, (uint32_t)g.N, blockIdx.x, gridDim.x,
+                          partial + lat * kHeisParts * 4);
 }
 
-__global__ void finish_heis_kernel(const double *__restrict__ partial, int64_t n_lat, int nb,
+__global__ void finish_heis_kernel(const double *__restrict__ partial, int64_t n_lat,
                                    double *__restrict__ Ef, double *__restrict__ Mf) {
   griddep_wait();
   griddep_release();
-  const int64_t lat = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (lat >= n_lat) return;
-  heis_finish_lattice(partial, nb, lat, Ef, Mf);
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k < 4 * n_lat) heis_finish_component(partial, k, Ef, Mf);
 }
 
 // ---------------------------------------------------------------- replica exchange
@@ -604,11 +602,15 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
   if (h->d.model == SPIN_HEISENBERG) {
     if (!Ef && !Mf) return cudaSuccess;
     double *partial = (double *)h->d_scratch64;
-    cudaError_t e = launch_dependent(measure_heis_kernel, dim3(kHeisBlocks, (unsigned)nl), dim3(256), 0, st,
-                                     (const float4 *)h->spins, g, partial);
+    const int c = heis_measure_cluster(g.N);
+    const dim3 grid((unsigned)(kHeisParts * c), (unsigned)nl);
+    cudaError_t e = c == 1 ? launch_dependent(measure_heis_kernel<1>, grid, dim3(256), 0, st,
+                                              (const float4 *)h->spins, g, partial)
+                           : launch_clusters(measure_heis_kernel<kHeisCluster>, grid, dim3(256), c, 0, st,
+                                             (const float4 *)h->spins, g, partial);
     if (e != cudaSuccess) return e;
-    return launch_dependent(finish_heis_kernel, dim3(grid_for(nl, 128)), dim3(128), 0, st,
-                            (const double *)partial, nl, kHeisBlocks, Ef, Mf);
+    return launch_dependent(finish_heis_kernel, dim3(grid_for(4 * nl, 128)), dim3(128), 0, st,
+                            (const double *)partial, nl, Ef, Mf);
   }
   if (h->d.layout == SPIN_MSC1 && h->d.model == SPIN_ISING) {
     if (Q) cudaMemsetAsync(Q, 0, sizeof(int64_t) * g.n_temps * g.n_real, st);

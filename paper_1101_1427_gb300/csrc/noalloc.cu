@@ -8,7 +8,7 @@
 // that must not stall the device, since cudaFree and often cudaMalloc
 // synchronise it.  This variant takes the spins and the outputs from the
 // caller and keeps its partial sums in one fixed array compiled into the
-// library (kMaxLattices lattices x 64 blocks x 4 doubles = 512 KiB per
+// library (kMaxLattices lattices x 64 partials x 4 doubles = 512 KiB per
 // device, held from library load until process exit).
 #include <mutex>
 
@@ -17,31 +17,30 @@
 
 namespace {
 
-constexpr int kBlocks = 64;         // partial sums per lattice
+constexpr int kParts = spin::kHeisParts;  // partial sums per lattice
 constexpr int kMaxLattices = 256;   // capacity of the fixed scratch
 constexpr int kMaxDevices = 64;
 
-// Fixed scratch: [lattice][block][E, Mx, My, Mz].  Every call overwrites the
+// Fixed scratch: [lattice][partial][E, Mx, My, Mz].  Every call overwrites the
 // entries it uses before reading them, so nothing has to start at zero.
-static __device__ __align__(256) double g_partials[kMaxLattices * kBlocks * 4];
+static __device__ __align__(256) double g_partials[kMaxLattices * kParts * 4];
 
 std::mutex g_setup_mutex;
 double *g_partials_addr[kMaxDevices] = {};  // device address of g_partials, per device
 
 // The arithmetic and order of the reduction behind spin_measure (one shared
 // device function), so both give bit-identical sums.
-__global__ void heis_partials_kernel(const float4 *__restrict__ s, int dim, int L, int64_t N,
+template <int kC>
+__global__ void heis_partials_kernel(const float4 *__restrict__ s, int dim, uint32_t L, spin::FastDiv fL, int64_t N,
                                      double *__restrict__ part) {
   const int64_t lat = blockIdx.y;
-  spin::heis_block_partials(s + lat * N, L, dim, N, blockIdx.x, gridDim.x,
-                            part + (lat * gridDim.x + blockIdx.x) * 4);
+  spin::heis_block_partials<kC>(s + lat * N, L, fL, dim, (uint32_t)N, blockIdx.x, gridDim.x, part + lat * kParts * 4);
 }
 
 __global__ void heis_finish_kernel(const double *__restrict__ part, int64_t n_lat, double *__restrict__ Ef,
                                    double *__restrict__ Mf) {
-  const int64_t lat = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (lat >= n_lat) return;
-  spin::heis_finish_lattice(part, kBlocks, lat, Ef, Mf);
+  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (k < 4 * n_lat) spin::heis_finish_component(part, k, Ef, Mf);
 }
 
 // Device address of the fixed scratch for the current device, looked up
@@ -75,7 +74,24 @@ extern "C" int spin_heis_measure_noalloc(const float *spins, int32_t dim, int32_
   const int rc = partials_for_current_device(&part);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  heis_partials_kernel<<<dim3(kBlocks, (unsigned)n_lat), 256, 0, st>>>((const float4 *)spins, dim, L, N, part);
-  heis_finish_kernel<<<(n_lat + 127) / 128, 128, 0, st>>>(part, n_lat, Ef, Mf);
+  const int c = spin::heis_measure_cluster(N);
+  const dim3 grid((unsigned)(kParts * c), (unsigned)n_lat);
+  const spin::FastDiv fL = spin::make_fastdiv((uint32_t)L);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, c == 1 ? heis_partials_kernel<1> : heis_partials_kernel<spin::kHeisCluster>,
+                         (const float4 *)spins, (int)dim, (uint32_t)L, fL, N, part);
+  if (e != cudaSuccess) return SPIN_ECUDA;
+  heis_finish_kernel<<<(4 * n_lat + 127) / 128, 128, 0, st>>>(part, n_lat, Ef, Mf);
   return cudaGetLastError() == cudaSuccess ? SPIN_OK : SPIN_ECUDA;
 }
