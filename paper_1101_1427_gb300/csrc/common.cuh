@@ -99,6 +99,70 @@ __device__ __forceinline__ uint4 philox_x1(const PhiloxX1 &q, uint32_t x1, const
   return c;
 }
 
+// Philox4x32-10 for counters (x0, x1, x2, x3) with x0 running in a thread and
+// (x1, x2) one of a few fixed pairs (sweep number and lattice) per thread:
+// the products of words x0 and of round-1 word 2 depend on neither x1 nor x2
+// and serve every pair (PhiloxX0Shared), those of x1 and x2 are formed once
+// per pair (PhiloxX0), which leaves 2 + 16 n of the 20 n multiplies for n
+// pairs.  Equal to philox() word for word.
+struct PhiloxX0 {
+  uint32_t y;  // lo(M1 x2) ^ k0[1]
+  uint32_t z;  // hi(M0 (hi(M1 x2) ^ x1 ^ k0[0])) ^ k1[1]
+  uint32_t w;  // lo of the same product
+};
+
+struct PhiloxX0Shared {
+  uint32_t lo0, hi1, lo1;
+};
+
+__device__ __forceinline__ PhiloxX0 philox_x0_setup(uint32_t x1, uint32_t x2, const RoundKeys &rk) {
+  const uint64_t p1 = mul_wide(0xCD9E8D57u, x2);
+  const uint64_t p0 = mul_wide(0xD2511F53u, (uint32_t)(p1 >> 32) ^ x1 ^ rk.k0[0]);
+  PhiloxX0 q;
+  q.y = (uint32_t)p1 ^ rk.k0[1];
+  q.z = (uint32_t)(p0 >> 32) ^ rk.k1[1];
+  q.w = (uint32_t)p0;
+  return q;
+}
+
+__device__ __forceinline__ PhiloxX0Shared philox_x0_shared(uint32_t x0, uint32_t x3, const RoundKeys &rk) {
+  const uint64_t p0 = mul_wide(0xD2511F53u, x0);
+  const uint64_t p1 = mul_wide(0xCD9E8D57u, (uint32_t)(p0 >> 32) ^ x3 ^ rk.k1[0]);
+  PhiloxX0Shared s;
+  s.lo0 = (uint32_t)p0;
+  s.hi1 = (uint32_t)(p1 >> 32);
+  s.lo1 = (uint32_t)p1;
+  return s;
+}
+
+__device__ __forceinline__ uint4 philox_x0(const PhiloxX0 &q, const PhiloxX0Shared &s, const RoundKeys &rk) {
+  uint4 c = make_uint4(s.hi1 ^ q.y, s.lo1, s.lo0 ^ q.z, q.w);
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+    const uint64_t m0 = mul_wide(0xD2511F53u, c.x);
+    const uint64_t m1 = mul_wide(0xCD9E8D57u, c.z);
+    c = make_uint4((uint32_t)(m1 >> 32) ^ c.y ^ rk.k0[r], (uint32_t)m1, (uint32_t)(m0 >> 32) ^ c.w ^ rk.k1[r],
+                   (uint32_t)m0);
+  }
+  return c;
+}
+
+// Acceptance masks of 32 words built one bit at a time: push() shifts in the
+// bit r >= thr (the carry of r + (2^32 - thr), thr >= 1) from the right, so
+// that the word pushed last ends in bit 0; mask() returns the bits r < thr.
+// Two ALU instructions per word and threshold; a compare and a warp ballot
+// are two as well, but ballots issue at a fraction of the ALU rate (2^24
+// sites x 32 sweeps of masks: 400 us with ballots, 297 us with carries, 243
+// us for the generator alone).
+struct MaskBits {
+  uint32_t neg;  // 2^32 - thr, 0 for thr = 0
+  __device__ __forceinline__ explicit MaskBits(uint32_t thr) : neg(0u - thr) {}
+  __device__ __forceinline__ void push(uint32_t &acc, uint32_t r) const {
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %0, %0;\n\t}" : "+r"(acc) : "r"(r), "r"(neg));
+  }
+  __device__ __forceinline__ uint32_t mask(uint32_t acc) const { return neg ? ~acc : 0u; }
+};
+
 __host__ __device__ __forceinline__ uint32_t ctr_w(uint32_t tag, uint32_t colour, uint32_t extra) {
   return (tag << 28) | (colour << 27) | extra;
 }

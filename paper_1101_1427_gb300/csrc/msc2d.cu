@@ -6,10 +6,10 @@
 //
 // Every site keeps its own uniform (sites of one lattice must not share
 // random numbers), drawn exactly as in the int8 layout: for k = 128 B + 4 l + q
-// the colour index is j = y L/2 + k, so lane l of a warp computes the Philox
-// call j >> 2 = y L/8 + 32 B + l and its word q belongs to word 4 B + q,
-// bit l.  The comparisons with the two thresholds become masks through
-// warp ballots; the neighbour count and the flip decision are bit-sliced.
+// the colour index is j = y L/2 + k, so the Philox call j >> 2 = y L/8 + 32 B
+// + l serves bit l of the four words 4 B + q, word q of the call for word q.
+// The comparisons with the two thresholds become acceptance masks; the
+// neighbour count and the flip decision are bit-sliced.
 #include "internal.h"
 #include "msc2d_block.cuh"
 
@@ -27,61 +27,71 @@ __device__ __forceinline__ int64_t row_word(const Msc2d &m, int64_t lat, int c, 
   return lat * m.lat_words + ((int64_t)c * m.L + y) * m.wpr;
 }
 
-// One colour phase.  Each warp owns 32 consecutive blocks of the global
-// block list (lattice, row, block).  Stage 1: for each of those blocks in
-// turn, lane l draws the Philox call of sites k = 128 B + 4 l + q (q = 0..3)
-// and the warp ballots (r < thr4) and (r < thr8): bit l of the ballot for q
-// is exactly bit l of word 4 B + q, so the two ballots are the acceptance
-// masks of the block's four words; lane 0 parks them in shared memory.
-// Stage 2: lane b updates block b with bit-sliced logic.
-constexpr int kWarps = 8;
-
-__global__ void __launch_bounds__(256) msc2d_phase_kernel(uint32_t *__restrict__ w, Msc2d m,
-                                                          Geom g, uint32_t total_blocks,
-                                                          const uint32_t *__restrict__ thr,
-                                                          RoundKeys rk, uint32_t sweep,
-                                                          int colour) {
-  __shared__ uint4 masks[kWarps][32][2];
-  griddep_wait();
+// One colour phase, one thread per block of 128 sites and kN lattices: the
+// thread draws the block's 32 Philox calls, last call first, shifts every
+// word's two comparisons into the block's masks (MaskBits), and updates the
+// block from registers.  The kN lattices share the part of each call that
+// depends only on the site.  Bound by the wide multiplies (16.7 to 18 per
+// call, at about 26 per clock and SM with the rest of the generator around
+// them), the ALU pipe close behind.
+//
+// The masks depend on no spin, so they are drawn before griddep_wait(): the
+// generator of a phase fills the SMs while the previous phase drains, and
+// only the update waits for it.  Measured per phase, against one warp per 32
+// blocks with ballots for masks, all of it after the wait (us): 3 x L = 16384
+// 300 -> 242, 16 x L = 1024 9.1 -> 5.4, 20 x L = 512 7.5 -> 2.4, one L = 1024
+// 5.8 -> 2.0.  Grid: (blocks of a lattice / 256, groups of kN lattices).
+template <int kN>
+__global__ void __launch_bounds__(256) msc2d_phase_kernel(uint32_t *__restrict__ w, Msc2d m, Geom g,
+                                                                 uint32_t n_lat, uint32_t per_lat,
+                                                                 const uint32_t *__restrict__ thr, RoundKeys rk,
+                                                                 uint32_t sweep, int colour) {
   griddep_release();
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const uint32_t first = (blockIdx.x * kWarps + wib) * 32u;
-  if (first >= total_blocks) return;
-  // L^2/256 blocks per lattice is a multiple of 32, so all 32 blocks of a
-  // warp lie in one lattice, and the Philox counter of lane l in block b is
-  // 32 b + l (rows are consecutive in the colour index)
-  const uint32_t per_lat = (uint32_t)m.L * (uint32_t)m.bpr;
-  const uint32_t lat = first / per_lat;
-  const uint32_t lid = lattice_id32(g, lat);
-  const uint32_t t = slot_of32(g, lat);
-  const uint32_t thr4 = __ldg(thr + 4 * t + 1), thr8 = __ldg(thr + 4 * t + 2);
+  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= per_lat) return;
+  const uint32_t lat0 = blockIdx.y * kN;
+  PhiloxX0 pre[kN];
+  uint32_t thr4[kN], thr8[kN], A[kN][4], E[kN][4];
+#pragma unroll
+  for (int n = 0; n < kN; ++n) {
+    const uint32_t lat = min(lat0 + n, n_lat - 1);  // (a last group that is not full draws one lattice twice)
+    const uint32_t t = slot_of32(g, lat);
+    pre[n] = philox_x0_setup(sweep, lattice_id32(g, lat), rk);
+    thr4[n] = __ldg(thr + 4 * t + 1);
+    thr8[n] = __ldg(thr + 4 * t + 2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) A[n][q] = E[n][q] = 0u;
+  }
   const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
-  uint32_t j4 = 32u * (first - lat * per_lat) + (uint32_t)lane;
-  uint4 *mk = &masks[wib][0][0];
-#pragma unroll  // 32 independent generator calls: full unrolling lets them interleave
-  for (uint32_t b = 0; b < 32u; ++b, j4 += 32u) {
-    const uint4 r = philox(make_uint4(j4, sweep, lid, wctr), rk);
-    const uint32_t a0 = __ballot_sync(0xffffffffu, r.x < thr4);
-    const uint32_t a1 = __ballot_sync(0xffffffffu, r.y < thr4);
-    const uint32_t a2 = __ballot_sync(0xffffffffu, r.z < thr4);
-    const uint32_t a3 = __ballot_sync(0xffffffffu, r.w < thr4);
-    const uint32_t e0 = __ballot_sync(0xffffffffu, r.x < thr8);
-    const uint32_t e1 = __ballot_sync(0xffffffffu, r.y < thr8);
-    const uint32_t e2 = __ballot_sync(0xffffffffu, r.z < thr8);
-    const uint32_t e3 = __ballot_sync(0xffffffffu, r.w < thr8);
-    if (lane == 0) {
-      mk[2 * b] = make_uint4(a0, a1, a2, a3);
-      mk[2 * b + 1] = make_uint4(e0, e1, e2, e3);
+#pragma unroll(kN == 1 ? 4 : 2)
+  for (int i = 31; i >= 0; --i) {
+    const PhiloxX0Shared sh = philox_x0_shared(32u * b + (uint32_t)i, wctr, rk);
+#pragma unroll
+    for (int n = 0; n < kN; ++n) {
+      const uint4 r = philox_x0(pre[n], sh, rk);
+      const MaskBits m4(thr4[n]), m8(thr8[n]);
+      m4.push(A[n][0], r.x);
+      m4.push(A[n][1], r.y);
+      m4.push(A[n][2], r.z);
+      m4.push(A[n][3], r.w);
+      m8.push(E[n][0], r.x);
+      m8.push(E[n][1], r.y);
+      m8.push(E[n][2], r.z);
+      m8.push(E[n][3], r.w);
     }
   }
-  __syncwarp();
-  const uint32_t gb = first + (uint32_t)lane;
-  const uint32_t rem = gb - lat * per_lat;
-  const uint32_t y = rem / (uint32_t)m.bpr;
-  const uint32_t B = rem - y * (uint32_t)m.bpr;
+  griddep_wait();  // the masks depend on no spin
+  const uint32_t y = b / (uint32_t)m.bpr, B = b - y * (uint32_t)m.bpr;
   long long unused_a = 0, unused_d = 0;
-  msc2d_block<0>(w + (int64_t)lat * m.lat_words, m.L, m.wpr, m.bpr, colour, (int)y, B, mk[2 * lane],
-                 mk[2 * lane + 1], unused_a, unused_d);
+#pragma unroll
+  for (int n = 0; n < kN; ++n) {
+    if (lat0 + n >= n_lat) break;
+    const MaskBits m4(thr4[n]), m8(thr8[n]);
+    msc2d_block<0>(w + (int64_t)(lat0 + n) * m.lat_words, m.L, m.wpr, m.bpr, colour, (int)y, B,
+                   make_uint4(m4.mask(A[n][0]), m4.mask(A[n][1]), m4.mask(A[n][2]), m4.mask(A[n][3])),
+                   make_uint4(m8.mask(E[n][0]), m8.mask(E[n][1]), m8.mask(E[n][2]), m8.mask(E[n][3])), unused_a,
+                   unused_d);
+  }
 }
 
 // Hot start: bit 0 of the INIT word of each site, as in the int8 layout.
@@ -271,17 +281,38 @@ cudaError_t launch_init_msc2d(spin_lattice *h) {
 }
 
 namespace {
+// Lattices per thread: the count with the best rate (1547, 1631, 1665
+// flips/ns for 1, 2, 3 when the GPU and every group are full) after the idle
+// places of the last group, among those that leave 2^15 threads, about half
+// the threads of the GPU at this kernel's registers (20 x L = 512, 20480
+// blocks, us per phase for 1, 2, 3: 2.42, 2.79, 3.16; 16 x L = 1024, 65536
+// blocks: 5.62, 5.42, 5.98; 12 x L = 2048, 196608 blocks: 16.5, 15.6, 15.4).
+int lattices_per_thread(int64_t n_lat, int64_t blocks) {
+  const double rate[4] = {0.0, 1547.0, 1631.0, 1665.0};
+  int best = 1;
+  double most = 0.0;
+  for (int k = 1; k <= 3; ++k) {
+    if (k > 1 && blocks / k < (1 << 15)) break;
+    const double r = rate[k] * (double)n_lat / (double)((n_lat + k - 1) / k * k);
+    if (r > most) most = r, best = k;
+  }
+  return best;
+}
+
 // n_sweeps coded sweeps of the handle's lattices held in the words w.
 cudaError_t sweeps_msc2d_words(spin_lattice *h, uint32_t *w, int64_t n_sweeps) {
   const Msc2d m = geom2d(h);
   const RoundKeys rk = make_round_keys(h->d.seed);
-  const int64_t blocks = h->n_lat * m.L * m.bpr;  // < 2^31, checked by spin_init
-  const unsigned grid = (unsigned)((blocks + 32 * kWarps - 1) / (32 * kWarps));
+  const uint32_t per_lat = (uint32_t)(m.L * m.bpr);
+  const int kn = lattices_per_thread(h->n_lat, h->n_lat * per_lat);
+  const auto kern = kn == 3 ? msc2d_phase_kernel<3> : kn == 2 ? msc2d_phase_kernel<2> : msc2d_phase_kernel<1>;
+  const dim3 grid((per_lat + 255) / 256, (unsigned)((h->n_lat + kn - 1) / kn));
   for (int64_t k = 0; k < n_sweeps; ++k) {
     const uint32_t sweep = (uint32_t)(h->sweeps_done + k);
     for (int colour = 0; colour < 2; ++colour) {
-      const cudaError_t e = launch_dependent(msc2d_phase_kernel, dim3(grid), dim3(32 * kWarps), 0, h->stream, w, m,
-                                             h->g, (uint32_t)blocks, (const uint32_t *)h->d_thr, rk, sweep, colour);
+      const cudaError_t e =
+          launch_dependent(kern, grid, dim3(256), 0, h->stream, w, m, h->g, (uint32_t)h->n_lat, per_lat,
+                           (const uint32_t *)h->d_thr, rk, sweep, colour);
       if (e != cudaSuccess) return e;
     }
   }
