@@ -243,6 +243,8 @@ cudaError_t launch_sweeps_dcb(spin_lattice *h, int64_t n_sweeps) {
         e = launch_heis_dcb_tiles(h, coarse, sweep0);
       } else if (h->g.dim == 3) {
         e = h->order_tile == 8 ? launch_tiles3<8>(h, coarse, sweep0) : launch_tiles3<16>(h, coarse, sweep0);
+      } else if (dcb_bits_preferred(h)) {
+        e = launch_dcb_bits(h, coarse, sweep0);
       } else {
         switch (h->order_tile) {
           case 8: e = launch_tiles<8>(h, coarse, sweep0); break;

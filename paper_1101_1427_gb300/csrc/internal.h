@@ -167,6 +167,11 @@ cudaError_t launch_resident(spin_lattice *h, int64_t n_sweeps, int64_t *E, int64
 bool dcb_supported(const spin_lattice *h, int tile);
 cudaError_t launch_sweeps_dcb(spin_lattice *h, int64_t n_sweeps);
 
+// dcb_bits.cu: one coarse colour of the 2D int8 double checkerboard with the
+// tiles as bits in registers, and the rule for when that is the faster form
+bool dcb_bits_preferred(const spin_lattice *h);
+cudaError_t launch_dcb_bits(spin_lattice *h, int coarse, uint32_t sweep0);
+
 // batch.cu: load the batch kernel's device counters from the host counters
 int sync_device_counters(spin_lattice *h, cudaStream_t st);
 
