@@ -37,7 +37,8 @@ struct spin_lattice {
   int64_t n_lat;         // n_sets * n_temps * n_real lattices
   int64_t sweeps_done;
   int64_t pt_steps_done;
-  int variant;           // 2D int8 sweep: 0 phases, 1 fused
+  int variant;           // int8 sweep: 0 phases, 1 fused, 3 resident, 4 coded
+  int auto_form;         // no variant was asked for: longer int8 calls may take the bit planes
   int msc_width;         // EA coded: realisations sharing one uniform (32 or 64)
   int order;             // spin_update_order
   int order_tile;        // double checkerboard: tile edge T
@@ -107,8 +108,9 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
 // energies: the lattices' current energies if the caller has them (device,
 // [n_lat]), else NULL to compute them
 // labels: configuration labels moved with accepted exchanges (device, [n_lat], or NULL)
+// planes: the lattices are in the handle's bit planes (planes.cu)
 cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, int32_t *labels,
-                           const int64_t *energies);
+                           const int64_t *energies, bool planes = false);
 
 // Launches kernel k as a programmatic dependent of the previous work in
 // stream s (the kernel must call griddep_wait() before touching memory), in
@@ -139,6 +141,21 @@ cudaError_t launch_dependent(void (*k)(KArgs...), dim3 grid, dim3 block, size_t 
                              Args... args) {
   return launch_clusters(k, grid, block, 1, smem, s, args...);
 }
+
+// planes.cu: longer calls of int8 ferromagnets on bit planes in the handle's
+// working buffer
+bool planes_supported(const spin_lattice *h);
+bool planes_reserve(spin_lattice *h);  // false: no memory, or a capture that must not allocate
+size_t planes_lattice_bytes(const spin_lattice *h);
+cudaError_t planes_pack(spin_lattice *h);
+cudaError_t planes_unpack(spin_lattice *h);
+cudaError_t planes_sweeps(spin_lattice *h, int64_t n_sweeps);
+cudaError_t planes_measure(spin_lattice *h, int64_t *E, int64_t *M);
+// whether a call of n sweeps takes them (ising_i8.cu)
+bool planes_wanted(const spin_lattice *h, int64_t n_sweeps);
+
+// msc2d.cu: lattices per thread of the coded phase kernels
+int lattices_per_thread(int64_t n_lat, int64_t blocks);
 
 // rng.cu
 cudaError_t launch_rng_fill(uint64_t seed, uint32_t w, uint32_t lattice_id, uint32_t sweep,

@@ -668,11 +668,12 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
 }
 
 cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, int32_t *labels,
-                           const int64_t *energies) {
+                           const int64_t *energies, bool planes) {
   const Geom &g = h->g;
   cudaStream_t st = h->stream;
   if (!energies) {
-    cudaError_t e = launch_measure(h, J, h->d_energy, nullptr, nullptr, nullptr, nullptr);
+    cudaError_t e = planes ? planes_measure(h, h->d_energy, nullptr)
+                           : launch_measure(h, J, h->d_energy, nullptr, nullptr, nullptr, nullptr);
     if (e != cudaSuccess) return e;
     energies = h->d_energy;
   }
@@ -695,12 +696,12 @@ cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, in
   } else {
     int64_t lat_bytes = g.N;  // int8
     if (h->d.layout == SPIN_MSC1) lat_bytes = g.N / 8;
-    if (h->d.layout == SPIN_F32X4) lat_bytes = g.N * 16;
+    if (planes) lat_bytes = (int64_t)planes_lattice_bytes(h);
     const int64_t units = (lat_bytes & 15) == 0 ? lat_bytes / 16 : lat_bytes;
     return launch_dependent(pt_swap_bytes_kernel, dim3(capped(units, 1024), (unsigned)h->n_lat), dim3(256), 0, st,
-                            (uint8_t *)h->spins, (const uint8_t *)decision, g, parity, lat_bytes);
+                            (uint8_t *)(planes ? h->d_pingpong : h->spins), (const uint8_t *)decision, g, parity,
+                            lat_bytes);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace spin

@@ -281,7 +281,6 @@ cudaError_t launch_init_msc2d(spin_lattice *h) {
   return cudaGetLastError();
 }
 
-namespace {
 // Lattices per thread: the count with the best rate (1547, 1631, 1665
 // flips/ns for 1, 2, 3 when the GPU and every group are full) after the idle
 // places of the last group, among those that leave 2^15 threads, about half
@@ -300,8 +299,7 @@ int lattices_per_thread(int64_t n_lat, int64_t blocks) {
   return best;
 }
 
-// n_sweeps coded sweeps of the handle's lattices held in the words w.
-cudaError_t sweeps_msc2d_words(spin_lattice *h, uint32_t *w, int64_t n_sweeps) {
+cudaError_t launch_sweeps_msc2d(spin_lattice *h, int64_t n_sweeps) {
   const Msc2d m = geom2d(h);
   const RoundKeys rk = make_round_keys(h->d.seed);
   const uint32_t per_lat = (uint32_t)(m.L * m.bpr);
@@ -312,23 +310,16 @@ cudaError_t sweeps_msc2d_words(spin_lattice *h, uint32_t *w, int64_t n_sweeps) {
     const uint32_t sweep = (uint32_t)(h->sweeps_done + k);
     for (int colour = 0; colour < 2; ++colour) {
       const cudaError_t e =
-          launch_dependent(kern, grid, dim3(256), 0, h->stream, w, m, h->g, (uint32_t)h->n_lat, per_lat,
+          launch_dependent(kern, grid, dim3(256), 0, h->stream, (uint32_t *)h->spins, m, h->g, (uint32_t)h->n_lat, per_lat,
                            (const uint32_t *)h->d_thr, rk, sweep, colour);
       if (e != cudaSuccess) return e;
     }
   }
   return cudaSuccess;
 }
-}  // namespace
 
-cudaError_t launch_sweeps_msc2d(spin_lattice *h, int64_t n_sweeps) {
-  return sweeps_msc2d_words(h, (uint32_t *)h->spins, n_sweeps);
-}
-
-// Sweeps of 2D int8 ferromagnets through the coded layout: the lattices are
-// packed into a handle-owned word buffer (L^2 / 8 bytes per lattice), swept
-// with the bit-sliced coded kernel -- the same random words and the same
-// decisions as every int8 kernel -- and unpacked into the caller's buffer.
+// Whether int8 lattices may ask for the coded form of their sweeps (variant 4,
+// planes.cu).
 bool coded_i8_supported(const spin_lattice *h) {
   return h->d.model == SPIN_ISING && h->d.layout == SPIN_I8 && h->d.dim == 2 && h->g.L % 256 == 0 &&
          h->n_lat * (int64_t)h->g.L * (h->g.L / 256) < ((int64_t)1 << 31);
@@ -338,7 +329,7 @@ namespace {
 // Conversion of all lattices of the handle between bytes and the words w.
 // The warp kernels read and write 8 bytes per lane; a byte buffer that is
 // not 8-byte aligned takes the per-site kernels (16 x L = 1024: pack 17.6 us
-// and unpack 90 us per site, 6.7 and 5.4 us by warps).
+// and unpack 90 us per site, 7 and 5 us by warps).
 cudaError_t transcode(spin_lattice *h, const int8_t *in, int8_t *out, uint32_t *words) {
   const Msc2d m = geom2d(h);
   const uint32_t n_blocks = (uint32_t)(h->n_lat * (int64_t)m.L * m.bpr);  // < 2^31, checked by spin_init
@@ -357,24 +348,6 @@ cudaError_t transcode(spin_lattice *h, const int8_t *in, int8_t *out, uint32_t *
   return cudaGetLastError();
 }
 }  // namespace
-
-cudaError_t launch_sweeps_i8_coded(spin_lattice *h, int64_t n_sweeps) {
-  const Msc2d m = geom2d(h);
-  const size_t bytes = (size_t)h->n_lat * (size_t)m.lat_words * 4;
-  if (!h->d_pingpong || h->pingpong_bytes < bytes) {
-    if (h->d_pingpong) cudaFree(h->d_pingpong);
-    h->d_pingpong = nullptr;
-    cudaError_t e = cudaMalloc(&h->d_pingpong, bytes);
-    if (e != cudaSuccess) return e;
-    h->pingpong_bytes = bytes;
-  }
-  uint32_t *words = (uint32_t *)h->d_pingpong;
-  cudaError_t e = transcode(h, (const int8_t *)h->spins, nullptr, words);
-  if (e != cudaSuccess) return e;
-  e = sweeps_msc2d_words(h, words, n_sweeps);
-  if (e != cudaSuccess) return e;
-  return transcode(h, nullptr, (int8_t *)h->spins, words);
-}
 
 cudaError_t launch_unpack_msc2d(spin_lattice *h, int8_t *out) {
   return transcode(h, nullptr, out, (uint32_t *)h->spins);

@@ -1,0 +1,279 @@
+// Longer calls on int8 ferromagnets (L % 8 == 0): the lattices are packed into
+// bit planes (planes.cuh) in a handle-owned buffer, swept, measured and
+// exchanged there, and unpacked at the end.  The random words and decisions
+// are those of every int8 kernel, so the results are the same bit for bit.
+//
+// The byte kernels spend 22 to 25 lane instructions per flip, most of them on
+// bytes; on planes the generator and its two or three comparisons per word
+// are nearly all that is left.  Measured against them (us per call of the
+// byte kernels -> here): one 3D L = 512, 4 sweeps and a measurement, 859 ->
+// 535; three L = 1000, 20 sweeps and 2 measurements, 164 -> 111; 20 x L = 512,
+// 20 sweeps and 2 exchanges, 135 -> 113 (packed once instead of per exchange).
+#include "internal.h"
+#include "planes.cuh"
+
+namespace spin {
+namespace {
+
+// One colour phase, one thread per block and kN lattices, in the manner of
+// msc2d_phase_kernel (msc2d.cu): the thread draws the block's calls, last one
+// first, and shifts the comparisons into its masks (MaskBits) before
+// griddep_wait(), since they depend on no spin; only the update waits for the
+// previous phase.  Blocks with fewer bits than their colour's longest draw a
+// few calls they do not use, so that a warp's loops end together.
+template <int kDim, bool kNarrow, int kN>
+__global__ void __launch_bounds__(256) planes_phase_kernel(uint4 *__restrict__ w, Planes m, Geom g, uint32_t n_lat,
+                                                           const uint32_t *__restrict__ thr, RoundKeys rk,
+                                                           uint32_t sweep, int colour) {
+  griddep_release();
+  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= m.blocks) return;
+  const PlaneBlock k = plane_block<kNarrow>(m, b);
+  const uint32_t lat0 = blockIdx.y * kN;
+  constexpr int kT = kDim;  // thresholds: dE = 4, 8 and, in 3D, 12
+  PhiloxX0 pre[kN];
+  uint32_t t[kN][kT], A[kN][kT][4];
+#pragma unroll
+  for (int n = 0; n < kN; ++n) {
+    const uint32_t lat = min(lat0 + n, n_lat - 1);  // (a last group that is not full draws one lattice twice)
+    const uint32_t slot = slot_of32(g, lat);
+    pre[n] = philox_x0_setup(sweep, lattice_id32(g, lat), rk);
+#pragma unroll
+    for (int e = 0; e < kT; ++e) {
+      t[n][e] = __ldg(thr + 4 * slot + 1 + e);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) A[n][e][q] = 0u;
+    }
+  }
+  const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
+#pragma unroll(kN == 1 ? 4 : 2)
+  for (int i = (int)(kNarrow ? m.R * m.nb : m.w) - 1; i >= 0; --i) {
+    const PhiloxX0Shared sh = philox_x0_shared(k.j4 + (uint32_t)i, wctr, rk);
+#pragma unroll
+    for (int n = 0; n < kN; ++n) {
+      const uint4 r = philox_x0(pre[n], sh, rk);
+#pragma unroll
+      for (int e = 0; e < kT; ++e) {
+        const MaskBits mb(t[n][e]);
+        mb.push(A[n][e][0], r.x);
+        mb.push(A[n][e][1], r.y);
+        mb.push(A[n][e][2], r.z);
+        mb.push(A[n][e][3], r.w);
+      }
+    }
+  }
+  griddep_wait();
+  const uint32_t valid = low_bits(k.bits);
+#pragma unroll
+  for (int n = 0; n < kN; ++n) {
+    if (lat0 + n >= n_lat) break;
+    uint4 *S = w + ((size_t)(lat0 + n) * 2 + colour) * m.blocks;
+    const uint4 *O = w + ((size_t)(lat0 + n) * 2 + (colour ^ 1)) * m.blocks;
+    PlaneNbrs<kDim> nb;
+    plane_nbrs<kDim, kNarrow>(m, O, b, k, colour, nb);
+    uint32_t s[4];
+    put4(s, S[b]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t m4 = MaskBits(t[n][0]).mask(A[n][0][q]), m8 = MaskBits(t[n][1]).mask(A[n][1][q]);
+      const uint32_t m12 = kDim == 3 ? MaskBits(t[n][kT - 1]).mask(A[n][kT - 1][q]) : 0u;
+      s[q] ^= plane_flips<kDim>(s[q], nb, q, m4, m8, m12) & valid;
+    }
+    S[b] = make_uint4(s[0], s[1], s[2], s[3]);
+  }
+}
+
+// int8 <-> planes, one warp per block place (both colours): lane l holds the
+// 8-byte chunk of call l of the block (the chunks of a block are contiguous
+// in the row-major lattice), whose byte 2 q + p is the site of colour
+// (p + y + z) & 1 in plane q, and one ballot per byte position builds a word.
+template <bool kNarrow>
+__device__ __forceinline__ size_t chunk_index(const Planes &m, const PlaneBlock &k, uint32_t lat, int lane) {
+  (void)kNarrow;
+  return (size_t)lat * ((size_t)m.L * (m.dim == 3 ? m.L : 1) * m.nb) + k.j4 + lane;
+}
+
+template <bool kNarrow, bool kPack>
+__global__ void __launch_bounds__(256) planes_bytes_kernel(uint64_t *__restrict__ bytes, uint4 *__restrict__ w,
+                                                           Planes m, uint32_t total, FastDiv fblocks) {
+  griddep_wait();
+  griddep_release();
+  const int lane = threadIdx.x & 31;
+  constexpr int kPer = 2;  // blocks a warp has in flight
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (uint32_t first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPer; first < total; first += nwarps * kPer) {
+    PlaneBlock k[kPer];
+    uint32_t lat[kPer], b[kPer], par[kPer];
+    uint64_t v[kPer];
+    uint4 w0[kPer], w1[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      if (first + u >= total) break;  // uniform across the warp
+      lat[u] = fdiv(first + u, fblocks);
+      b[u] = first + u - lat[u] * m.blocks;
+      k[u] = plane_block<kNarrow>(m, b[u]);
+      // parity of the lane's row
+      par[u] = kNarrow ? (k[u].par + (uint32_t)lane / m.nb) & 1u : k[u].par;
+      if (kPack) {
+        v[u] = (uint32_t)lane < k[u].bits ? bytes[chunk_index<kNarrow>(m, k[u], lat[u], lane)] : 0ull;
+      } else {
+        w0[u] = w[(size_t)lat[u] * 2 * m.blocks + b[u]];
+        w1[u] = w[((size_t)lat[u] * 2 + 1) * m.blocks + b[u]];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      if (first + u >= total) break;
+      const bool mine = (uint32_t)lane < k[u].bits;
+      if (kPack) {
+        uint32_t lo = (uint32_t)v[u], hi = (uint32_t)(v[u] >> 32);
+        if (par[u]) {  // byte 2 q + c to the site of colour c
+          lo = __byte_perm(lo, 0u, 0x2301);
+          hi = __byte_perm(hi, 0u, 0x2301);
+        }
+        uint32_t word[8];
+#pragma unroll
+        for (int o = 0; o < 8; ++o)  // bit 1 of a +-1 byte is set for -1
+          word[o] = __ballot_sync(0xffffffffu, mine && ((o < 4 ? lo : hi) >> (8 * (o & 3) + 1) & 1u));
+        if (lane < 2)
+          w[((size_t)lat[u] * 2 + lane) * m.blocks + b[u]] =
+              lane ? make_uint4(word[1], word[3], word[5], word[7]) : make_uint4(word[0], word[2], word[4], word[6]);
+      } else if (mine) {
+        const uint32_t a[8] = {w0[u].x, w1[u].x, w0[u].y, w1[u].y, w0[u].z, w1[u].z, w0[u].w, w1[u].w};
+        uint32_t lo = 0x01010101u, hi = 0x01010101u;
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+          const uint32_t f = (a[o] >> lane & 1u) * (0xFEu << (8 * (o & 3)));  // 0x01 | 0xFE = -1
+          if (o < 4) lo |= f;
+          else hi |= f;
+        }
+        if (par[u]) {
+          lo = __byte_perm(lo, 0u, 0x2301);
+          hi = __byte_perm(hi, 0u, 0x2301);
+        }
+        bytes[chunk_index<kNarrow>(m, k[u], lat[u], lane)] = ((uint64_t)hi << 32) | lo;
+      }
+    }
+  }
+}
+
+// Energy and magnetisation: every bond joins the two colours, so the
+// antiparallel neighbours of the colour-0 sites count each once;
+// E = 2 n_anti - dim N, M = N - 2 n_down.  Adds to outputs the host zeroed.
+template <int kDim, bool kNarrow>
+__global__ void __launch_bounds__(256) planes_measure_kernel(const uint4 *__restrict__ w, Planes m, long long N,
+                                                             long long *__restrict__ E, long long *__restrict__ M) {
+  __shared__ int red[8][2];
+  griddep_wait();
+  griddep_release();
+  const uint32_t lat = blockIdx.y;
+  const uint4 *S = w + (size_t)lat * 2 * m.blocks, *O = S + m.blocks;
+  int anti = 0, down = 0;
+  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < m.blocks; b += gridDim.x * blockDim.x) {
+    const PlaneBlock k = plane_block<kNarrow>(m, b);
+    PlaneNbrs<kDim> nb;
+    plane_nbrs<kDim, kNarrow>(m, O, b, k, 0, nb);
+    uint32_t s[4];
+    put4(s, S[b]);
+    const uint32_t valid = low_bits(k.bits);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      anti += __popc((s[q] ^ nb.u[q]) & valid) + __popc((s[q] ^ nb.d[q]) & valid) + __popc(s[q] ^ nb.o[q]) +
+              __popc((s[q] ^ nb.s[q]) & valid);
+      if (kDim == 3) anti += __popc(s[q] ^ nb.f[q]) + __popc(s[q] ^ nb.b[q]);
+      down += __popc(s[q]) + __popc(nb.o[q]);
+    }
+  }
+  anti = __reduce_add_sync(0xffffffffu, anti);
+  down = __reduce_add_sync(0xffffffffu, down);
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5][0] = anti;
+    red[threadIdx.x >> 5][1] = down;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  long long a = 0, d = 0;
+  for (int i = 0; i < 8; ++i) a += red[i][0], d += red[i][1];
+  const bool first = blockIdx.x == 0;
+  if (E) atomicAdd((unsigned long long *)&E[lat], (unsigned long long)(2 * a - (first ? kDim * N : 0)));
+  if (M) atomicAdd((unsigned long long *)&M[lat], (unsigned long long)((first ? N : 0) - 2 * d));
+}
+
+bool narrow(const Planes &m) { return m.nb <= 16; }
+
+template <int kN>
+auto phase_kernel(const Planes &m) {
+  return m.dim == 3 ? (narrow(m) ? planes_phase_kernel<3, true, kN> : planes_phase_kernel<3, false, kN>)
+                    : (narrow(m) ? planes_phase_kernel<2, true, kN> : planes_phase_kernel<2, false, kN>);
+}
+
+cudaError_t transcode(spin_lattice *h, bool pack) {
+  const Planes m = make_planes(h->g.dim, h->g.L);
+  const uint32_t total = (uint32_t)(h->n_lat * m.blocks);  // < 2^32: a block has at least 8 sites
+  const auto kern = pack ? (narrow(m) ? planes_bytes_kernel<true, true> : planes_bytes_kernel<false, true>)
+                         : (narrow(m) ? planes_bytes_kernel<true, false> : planes_bytes_kernel<false, false>);
+  unsigned grid = grid_for(total, 16);  // 8 warps of 2 blocks
+  if (grid > 152 * 64) grid = 152 * 64;
+  return launch_dependent(kern, dim3(grid), dim3(256), 0, h->stream, (uint64_t *)h->spins, (uint4 *)h->d_pingpong, m,
+                          total, make_fastdiv(m.blocks));
+}
+
+}  // namespace
+
+bool planes_supported(const spin_lattice *h) {
+  return h->d.model == SPIN_ISING && h->d.layout == SPIN_I8 && h->g.L % 8 == 0;
+}
+
+size_t planes_lattice_bytes(const spin_lattice *h) {
+  return (size_t)make_planes(h->g.dim, h->g.L).blocks * 2 * sizeof(uint4);
+}
+
+cudaError_t planes_pack(spin_lattice *h) { return transcode(h, true); }
+cudaError_t planes_unpack(spin_lattice *h) { return transcode(h, false); }
+
+bool planes_reserve(spin_lattice *h) {
+  const size_t bytes = (size_t)h->n_lat * planes_lattice_bytes(h);
+  if (h->d_pingpong && h->pingpong_bytes >= bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  void *p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (h->d_pingpong) cudaFree(h->d_pingpong);
+  h->d_pingpong = p;
+  h->pingpong_bytes = bytes;
+  return true;
+}
+
+cudaError_t planes_sweeps(spin_lattice *h, int64_t n_sweeps) {
+  const Planes m = make_planes(h->g.dim, h->g.L);
+  const RoundKeys rk = make_round_keys(h->d.seed);
+  const int kn = lattices_per_thread(h->n_lat, h->n_lat * m.blocks);
+  const auto kern = kn == 3 ? phase_kernel<3>(m) : kn == 2 ? phase_kernel<2>(m) : phase_kernel<1>(m);
+  const dim3 grid((m.blocks + 255) / 256, (unsigned)((h->n_lat + kn - 1) / kn));
+  for (int64_t k = 0; k < n_sweeps; ++k)
+    for (int colour = 0; colour < 2; ++colour) {
+      const cudaError_t e = launch_dependent(kern, grid, dim3(256), 0, h->stream, (uint4 *)h->d_pingpong, m, h->g,
+                                             (uint32_t)h->n_lat, (const uint32_t *)h->d_thr, rk,
+                                             (uint32_t)(h->sweeps_done + k), colour);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
+}
+
+cudaError_t planes_measure(spin_lattice *h, int64_t *E, int64_t *M) {
+  if (!E && !M) return cudaSuccess;
+  const Planes m = make_planes(h->g.dim, h->g.L);
+  if (E) cudaMemsetAsync(E, 0, sizeof(int64_t) * h->n_lat, h->stream);
+  if (M) cudaMemsetAsync(M, 0, sizeof(int64_t) * h->n_lat, h->stream);
+  const auto kern = m.dim == 3 ? (narrow(m) ? planes_measure_kernel<3, true> : planes_measure_kernel<3, false>)
+                               : (narrow(m) ? planes_measure_kernel<2, true> : planes_measure_kernel<2, false>);
+  unsigned gx = grid_for(m.blocks, 256);
+  if (gx > 1024) gx = 1024;
+  return launch_dependent(kern, dim3(gx, (unsigned)h->n_lat), dim3(256), 0, h->stream, (const uint4 *)h->d_pingpong, m,
+                          (long long)h->g.N, (long long *)E, (long long *)M);
+}
+
+}  // namespace spin

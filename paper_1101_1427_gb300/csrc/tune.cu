@@ -48,23 +48,31 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
   const bool dcb = h->order != SPIN_ORDER_CHECKERBOARD;
   if (dcb && n_sweeps % h->order_hits != 0) return SPIN_EINVAL;
   const bool i8_ferro = h->d.model == SPIN_ISING && h->d.layout == SPIN_I8;
-  // candidate (variant, tile) pairs that give the handle's chain
+  // candidate (variant, tile) pairs that give the handle's chain; kAuto marks
+  // the default form of a handle whose variant was never set
+  constexpr int kAuto = 16;
+  auto apply = [h](const std::pair<int, int> &c) {
+    h->variant = c.first & (kAuto - 1);
+    h->auto_form = c.first / kAuto;
+    h->order_tile = c.second;
+  };
+  const std::pair<int, int> start(h->variant + kAuto * h->auto_form, h->order_tile);
   std::vector<std::pair<int, int>> cand;
   if (dcb) {
     if (h->order_tile == 0) {
       for (int t : {8, 16, 32, 64, 128})
-        if (spin::dcb_supported(h, t)) cand.emplace_back(h->variant, t);
+        if (spin::dcb_supported(h, t)) cand.emplace_back(start.first, t);
     } else {
-      cand.emplace_back(h->variant, h->order_tile);
+      cand.push_back(start);
     }
   } else if (i8_ferro) {
     for (int v : {0, 1, 3, 4}) {
-      const int old = h->variant;
       if (spin_set_variant(h, v) == SPIN_OK) cand.emplace_back(v, h->order_tile);
-      h->variant = old;
+      apply(start);
     }
+    if (h->auto_form && spin::planes_wanted(h, n_sweeps)) cand.push_back(start);
   } else {
-    cand.emplace_back(h->variant, h->order_tile);
+    cand.push_back(start);
   }
   if (cand.empty()) return SPIN_EINVAL;
   const Key key = key_of(h, n_sweeps);
@@ -72,8 +80,7 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tuned.find(key);
     if (it != g_tuned.end()) {
-      h->variant = it->second.first;
-      h->order_tile = it->second.second;
+      apply(it->second);
       if (best_variant) *best_variant = h->variant;
       if (best_tile) *best_tile = h->order_tile;
       return SPIN_OK;
@@ -88,7 +95,6 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
   cudaStream_t st = h->stream;
   cudaMemcpyAsync(backup, h->spins, (size_t)bytes, cudaMemcpyDeviceToDevice, st);
   const int64_t sweeps0 = h->sweeps_done, pt0 = h->pt_steps_done;
-  const int variant0 = h->variant, tile0 = h->order_tile;
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
@@ -96,8 +102,7 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
   std::pair<int, int> best = cand[0];
   int rc = SPIN_OK;
   for (const auto &c : cand) {
-    h->variant = c.first;
-    h->order_tile = c.second;
+    apply(c);
     float ms_c = 1e30f;
     for (int rep = 0; rep < 3 && rc == SPIN_OK; ++rep) {  // first run warms up, best of the other two
       cudaMemcpyAsync(h->spins, backup, (size_t)bytes, cudaMemcpyDeviceToDevice, st);
@@ -124,12 +129,10 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
   h->sweeps_done = sweeps0;
   h->pt_steps_done = pt0;
   if (rc != SPIN_OK) {
-    h->variant = variant0;
-    h->order_tile = tile0;
+    apply(start);
     return rc;
   }
-  h->variant = best.first;
-  h->order_tile = best.second;
+  apply(best);
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tuned[key] = best;
