@@ -266,6 +266,8 @@ int spin_sweep(spin_lattice *h, const void *couplings, const double *betas, int6
     return SPIN_EINVAL;  // whole compound moves only, and a tile edge chosen
   int rc = upload_thresholds(h, betas);
   if (rc) return rc;
+  if (planes_wanted(h, n_sweeps, 0) && planes_ready(h, n_sweeps))
+    return planes_run(h, betas, n_sweeps, 0, 0, nullptr, nullptr, nullptr, nullptr);
   cudaError_t e = h->order != SPIN_ORDER_CHECKERBOARD ? launch_sweeps_dcb(h, n_sweeps)
                                                       : do_sweeps(h, ea(h) ? couplings : nullptr, n_sweeps);
   if (e != cudaSuccess) return SPIN_ECUDA;
@@ -286,55 +288,16 @@ namespace {
 // One exchange step; `energies` (device, [n_lat]) are the lattices' current
 // energies when the caller has just measured them, else NULL.
 int pt_swap(spin_lattice *h, const void *couplings, const double *betas, uint64_t seed,
-            int64_t *accepted, int32_t *labels, const int64_t *energies, bool planes = false) {
+            int64_t *accepted, int32_t *labels, const int64_t *energies) {
   if (!h || seed != h->d.seed || !betas) return SPIN_EINVAL;
   if (h->d.model == SPIN_HEISENBERG) return SPIN_EINVAL;
   if (ea(h) && !couplings) return SPIN_EINVAL;
   int rc = upload_pt_tables(h, betas);
   if (rc) return rc;
-  cudaError_t e = launch_pt_swap(h, ea(h) ? couplings : nullptr, accepted, labels, energies, planes);
+  cudaError_t e = launch_pt_swap(h, ea(h) ? couplings : nullptr, accepted, labels, energies);
   if (e != cudaSuccess) return SPIN_ECUDA;
   h->pt_steps_done += 1;
   return SPIN_OK;
-}
-
-// spin_run on the handle's bit planes: packed once, swept, measured and
-// exchanged there, and unpacked at the end, also when an argument turns out
-// to be bad on the way (the sweeps done by then stand, as in spin_run).
-int run_planes(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
-               int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels) {
-  int rc = upload_thresholds(h, betas);
-  if (rc) return rc;
-  if (planes_pack(h) != cudaSuccess) return SPIN_ECUDA;
-  const int64_t nl = h->n_lat;
-  const bool measuring = measure_every > 0 && (E_series || M_series);
-  int64_t done = 0, k_meas = 0;
-  while (done < n_sweeps && rc == SPIN_OK) {
-    const int64_t cur = h->sweeps_done;
-    int64_t next = n_sweeps - done;
-    if (measuring) next = std::min(next, measure_every - cur % measure_every);
-    if (pt_every > 0) next = std::min(next, pt_every - cur % pt_every);
-    if (cur + next > (int64_t)0xFFFFFFFFll) {
-      rc = SPIN_EINVAL;
-      break;
-    }
-    if (planes_sweeps(h, next) != cudaSuccess) return SPIN_ECUDA;
-    h->sweeps_done += next;
-    done += next;
-    const int64_t now = h->sweeps_done;
-    const int64_t *energies = nullptr;  // energies measured at this sweep, if any
-    if (measuring && now % measure_every == 0) {
-      if (planes_measure(h, E_series ? E_series + k_meas * nl : nullptr,
-                         M_series ? M_series + k_meas * nl : nullptr) != cudaSuccess)
-        return SPIN_ECUDA;
-      if (E_series) energies = E_series + k_meas * nl;
-      ++k_meas;
-    }
-    if (pt_every > 0 && now % pt_every == 0)
-      rc = pt_swap(h, nullptr, betas, h->d.seed, accepted, labels, energies, true);
-  }
-  if (rc == SPIN_ECUDA) return rc;
-  return planes_unpack(h) == cudaSuccess ? rc : SPIN_ECUDA;
 }
 }  // namespace
 
@@ -352,9 +315,12 @@ int spin_run(spin_lattice *h, const void *couplings, const double *betas, int64_
   if (!h || n_sweeps < 0) return SPIN_EINVAL;
   if (pt_every > 0 && h->d.model == SPIN_HEISENBERG) return SPIN_EINVAL;
   const bool measuring = measure_every > 0 && (E_series || M_series || Q_series || Ef_series || Mf_series);
-  if ((measuring || pt_every > 0) && !Q_series && !Ef_series && !Mf_series && planes_wanted(h, n_sweeps) &&
-      planes_reserve(h))
-    return run_planes(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
+  if (!Q_series && !Ef_series && !Mf_series && planes_wanted(h, n_sweeps, pt_every)) {
+    const int rc = upload_thresholds(h, betas);
+    if (rc) return rc;
+    if (planes_ready(h, n_sweeps))
+      return planes_run(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
+  }
   int64_t done = 0, k_meas = 0;
   // small int8 ferromagnets: the resident kernel measures E and M itself,
   // so a call is one launch per exchange interval

@@ -9,6 +9,7 @@
 
 #include "../../include/spin.h"
 #include "common.cuh"
+#include "pt.cuh"
 
 // NVTX range over one ABI call, so that a profiler's timeline shows which
 // entry point enqueued which kernels (no cost when no tool is attached).
@@ -56,8 +57,9 @@ struct spin_lattice {
   int64_t *d_energy;     // [n_lat] scratch energies for the exchange step
   int64_t *d_scratch64;  // small reduction scratch
   int *d_err;            // device error word
-  void *d_pingpong;      // lattice-sized buffer of the fused 2D sweep (lazy)
+  void *d_pingpong;      // working buffer of the sweeps that need one (lazy)
   size_t pingpong_bytes;
+  int tape_half;         // half of the tape in it that was drawn last (planes_res.cu)
   // batched launches (options set with spin_set_batch_options)
   uint64_t batch_timeout_ns;  // bound on every team-barrier wait (0: 2 s)
   int batch_ctas_per_sm;      // 0: autotuned / default
@@ -108,9 +110,9 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
 // energies: the lattices' current energies if the caller has them (device,
 // [n_lat]), else NULL to compute them
 // labels: configuration labels moved with accepted exchanges (device, [n_lat], or NULL)
-// planes: the lattices are in the handle's bit planes (planes.cu)
+// planes: the lattices are bit planes in this buffer (planes.cu), not NULL
 cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, int32_t *labels,
-                           const int64_t *energies, bool planes = false);
+                           const int64_t *energies, void *planes = nullptr);
 
 // Launches kernel k as a programmatic dependent of the previous work in
 // stream s (the kernel must call griddep_wait() before touching memory), in
@@ -142,17 +144,43 @@ cudaError_t launch_dependent(void (*k)(KArgs...), dim3 grid, dim3 block, size_t 
   return launch_clusters(k, grid, block, 1, smem, s, args...);
 }
 
+inline PtTables pt_tables(const spin_lattice *h) {
+  PtTables p;
+  p.dbeta = h->d_pt_dbeta;
+  p.tab = h->d_pt_thr;
+  p.off = h->d_pt_off;
+  p.len = h->d_pt_len;
+  return p;
+}
+
 // planes.cu: longer calls of int8 ferromagnets on bit planes in the handle's
 // working buffer
 bool planes_supported(const spin_lattice *h);
-bool planes_reserve(spin_lattice *h);  // false: no memory, or a capture that must not allocate
 size_t planes_lattice_bytes(const spin_lattice *h);
-cudaError_t planes_pack(spin_lattice *h);
-cudaError_t planes_unpack(spin_lattice *h);
-cudaError_t planes_sweeps(spin_lattice *h, int64_t n_sweeps);
 cudaError_t planes_measure(spin_lattice *h, int64_t *E, int64_t *M);
 // whether a call of n sweeps takes them (ising_i8.cu)
-bool planes_wanted(const spin_lattice *h, int64_t n_sweeps);
+bool planes_wanted(const spin_lattice *h, int64_t n_sweeps, int32_t pt_every);
+// makes the buffers ready; false: no memory, or a capture that must not allocate
+bool planes_ready(spin_lattice *h, int64_t n_sweeps);
+// the call (SPIN_* status), spin_run without Q; counters advanced
+int planes_run(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
+               int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels);
+
+// planes_res.cu: the same for lattices small enough for one CTA each
+struct PlanesResCall {
+  int64_t *E, *M;         // series rows (NULL: none) after sweeps first, first + every, ... (1-based)
+  int every, first;
+  int64_t *E_last;        // energies after the last sweep (NULL: not wanted)
+  const int64_t *E_prev;  // energies that decide exchange `step` before the first sweep (NULL: none)
+  uint32_t step;
+  int64_t *accepted;
+  int32_t *labels;
+  bool bytes_in, bytes_out;  // from or to the caller's bytes instead of the planes
+};
+bool planes_res_supported(const spin_lattice *h);
+bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps);
+int64_t planes_res_draw(spin_lattice *h, int64_t sweep0, int64_t n, cudaError_t *err);
+cudaError_t planes_res_sweeps(spin_lattice *h, int64_t at, int64_t n, int from, const PlanesResCall &call);
 
 // msc2d.cu: lattices per thread of the coded phase kernels
 int lattices_per_thread(int64_t n_lat, int64_t blocks);

@@ -422,10 +422,20 @@ bool fused2d_supported(int L);                                     // fused2d.cu
 // the byte kernels, least against the fused pass.
 constexpr int64_t kCodedMinSweeps = 4;   // variant 4, shorter calls take the fused pass
 constexpr int64_t kPlanesMinSweeps = 2;  // against the colour phases
-bool planes_wanted(const spin_lattice *h, int64_t n_sweeps) {
-  if (!planes_supported(h) || h->order != SPIN_ORDER_CHECKERBOARD) return false;
+bool planes_wanted(const spin_lattice *h, int64_t n_sweeps, int32_t pt_every) {
+  if (!planes_supported(h) || h->order != SPIN_ORDER_CHECKERBOARD || n_sweeps < 1) return false;
   if (h->variant == 4) return n_sweeps >= kCodedMinSweeps;
-  if (!h->auto_form || h->variant == 3) return false;
+  // Small lattices: the launch that draws the masks ahead costs what the
+  // sweeps must win back from the kernel with the lattice as bytes, about
+  // 0.14 us + 0.13 ns per site and sweep, and 12 us per exchange (us per call
+  // of 4 / 8 / 16 / 64 sweeps, bytes against planes: L = 16 5.1 / 5.5 / 8.1 /
+  // 24 against 7.3 / 7.6 / 7.7 / 16, L = 64 5.5 / 8.7 / 14 / 51 against 8.1 /
+  // 8.9 / 10 / 20, L = 128 14 / 25 / 45 / 171 against 8.7 / 9.7 / 12 / 25).
+  if (h->variant == 3)
+    return (double)n_sweeps * (0.14 + 0.00013 * (double)h->g.N) +
+               (pt_every > 0 ? 12.0 * (double)(n_sweeps / pt_every) : 0.0) >=
+           5.5;
+  if (!h->auto_form) return false;
   return n_sweeps >= (h->variant == 1 ? kCodedMinSweeps : kPlanesMinSweeps);
 }
 
@@ -474,11 +484,6 @@ cudaError_t launch_sweeps_i8(spin_lattice *h, const int8_t *J, int64_t n_sweeps)
   const RoundKeys rk = make_round_keys(h->d.seed);
   const bool fast2d = g.dim == 2 && J == nullptr && (g.L % 8) == 0 && h->n_lat <= 65535;
   const bool fast3d = g.dim == 3 && J == nullptr && (g.L % 8) == 0 && h->n_lat <= 65535;
-  if (J == nullptr && planes_wanted(h, n_sweeps) && planes_reserve(h)) {
-    cudaError_t e = planes_pack(h);
-    if (e == cudaSuccess) e = planes_sweeps(h, n_sweeps);
-    return e == cudaSuccess ? planes_unpack(h) : e;
-  }
   if (fast2d && (h->variant == 1 || h->variant == 4) && fused2d_supported(g.L)) return launch_fused2d_i8(h, n_sweeps);
   if ((fast2d || fast3d) && h->variant == 3 && resident_supported(g.dim, g.L))
     return launch_resident(h, n_sweeps, nullptr, nullptr, 1, 1);

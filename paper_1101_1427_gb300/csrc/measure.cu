@@ -482,12 +482,8 @@ __global__ void finish_heis_kernel(const double *__restrict__ partial, int64_t n
 
 // ---------------------------------------------------------------- replica exchange
 // Thread per (set a, realisation r, pair t) of the step's parity.
-// Delta = dbeta_t (E_{t+1} - E_t); accept iff Delta >= 0 or the PT word of
-// (a, t, step, r) is below the tabulated threshold of exp(Delta).
 __global__ void pt_decide_kernel(const long long *__restrict__ E, Geom g,
-                                 const double *__restrict__ dbeta,
-                                 const uint32_t *__restrict__ tab, const int32_t *__restrict__ off,
-                                 const int32_t *__restrict__ len, RoundKeys rk, uint32_t step,
+                                 PtTables tables, RoundKeys rk, uint32_t step,
                                  uint8_t *__restrict__ decision, long long *__restrict__ accepted,
                                  int *__restrict__ labels) {
   griddep_wait();
@@ -503,17 +499,7 @@ __global__ void pt_decide_kernel(const long long *__restrict__ E, Geom g,
   const int t = parity + 2 * pk;
   const int64_t lat0 = ((int64_t)a * g.n_temps + t) * g.n_real + r;
   const int64_t lat1 = lat0 + g.n_real;
-  const long long dE = E[lat1] - E[lat0];
-  const double db = dbeta[t];
-  bool acc;
-  if (db * (double)dE >= 0.0) {
-    acc = true;
-  } else {
-    const long long m = (dE < 0 ? -dE : dE) / 4;
-    const uint32_t thr = m < len[t] ? tab[off[t] + m] : 0u;
-    const uint4 w = philox(make_uint4((uint32_t)r >> 2, step, lattice_id(a, 0, t), ctr_w(TAG_PT, 0, 0)), rk);
-    acc = word_of(w, (uint32_t)r & 3u) < thr;
-  }
+  const bool acc = pt_accept(pt_pair(tables, a, t, r, step, rk), E[lat0], E[lat1]);
   decision[lat0] = acc ? 1 : 0;
   if (labels && acc) {  // one thread per pair: no other thread touches these two
     const int l0 = labels[lat0];
@@ -668,7 +654,7 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
 }
 
 cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, int32_t *labels,
-                           const int64_t *energies, bool planes) {
+                           const int64_t *energies, void *planes) {
   const Geom &g = h->g;
   cudaStream_t st = h->stream;
   if (!energies) {
@@ -684,9 +670,8 @@ cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, in
   if (n_pairs <= 0) return cudaSuccess;
   const int64_t total = (int64_t)g.n_sets * n_pairs * g.n_real;
   cudaError_t e = launch_dependent(pt_decide_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st,
-                                   (const long long *)energies, g, (const double *)h->d_pt_dbeta,
-                                   (const uint32_t *)h->d_pt_thr, (const int32_t *)h->d_pt_off,
-                                   (const int32_t *)h->d_pt_len, make_round_keys(h->d.seed), step, decision,
+                                   (const long long *)energies, g, pt_tables(h), make_round_keys(h->d.seed), step,
+                                   decision,
                                    (long long *)accepted, (int *)labels);
   if (e != cudaSuccess) return e;
   if (h->d.layout == SPIN_MSC1 && h->d.model == SPIN_EA) {
@@ -699,7 +684,7 @@ cudaError_t launch_pt_swap(spin_lattice *h, const void *J, int64_t *accepted, in
     if (planes) lat_bytes = (int64_t)planes_lattice_bytes(h);
     const int64_t units = (lat_bytes & 15) == 0 ? lat_bytes / 16 : lat_bytes;
     return launch_dependent(pt_swap_bytes_kernel, dim3(capped(units, 1024), (unsigned)h->n_lat), dim3(256), 0, st,
-                            (uint8_t *)(planes ? h->d_pingpong : h->spins), (const uint8_t *)decision, g, parity,
+                            (uint8_t *)(planes ? planes : h->spins), (const uint8_t *)decision, g, parity,
                             lat_bytes);
   }
 }

@@ -9,10 +9,13 @@
 // byte kernels -> here): one 3D L = 512, 4 sweeps and a measurement, 859 ->
 // 535; three L = 1000, 20 sweeps and 2 measurements, 164 -> 111; 20 x L = 512,
 // 20 sweeps and 2 exchanges, 135 -> 113 (packed once instead of per exchange).
+#include <algorithm>
+
 #include "internal.h"
 #include "planes.cuh"
 
 namespace spin {
+int upload_pt_tables_for_batch(spin_lattice *h, const double *betas);  // api.cu
 namespace {
 
 // One colour phase, one thread per block and kN lattices, in the manner of
@@ -87,9 +90,7 @@ __global__ void __launch_bounds__(256) planes_phase_kernel(uint4 *__restrict__ w
 // 8-byte chunk of call l of the block (the chunks of a block are contiguous
 // in the row-major lattice), whose byte 2 q + p is the site of colour
 // (p + y + z) & 1 in plane q, and one ballot per byte position builds a word.
-template <bool kNarrow>
 __device__ __forceinline__ size_t chunk_index(const Planes &m, const PlaneBlock &k, uint32_t lat, int lane) {
-  (void)kNarrow;
   return (size_t)lat * ((size_t)m.L * (m.dim == 3 ? m.L : 1) * m.nb) + k.j4 + lane;
 }
 
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(256) planes_bytes_kernel(uint64_t *__restrict_
       // parity of the lane's row
       par[u] = kNarrow ? (k[u].par + (uint32_t)lane / m.nb) & 1u : k[u].par;
       if (kPack) {
-        v[u] = (uint32_t)lane < k[u].bits ? bytes[chunk_index<kNarrow>(m, k[u], lat[u], lane)] : 0ull;
+        v[u] = (uint32_t)lane < k[u].bits ? bytes[chunk_index(m, k[u], lat[u], lane)] : 0ull;
       } else {
         w0[u] = w[(size_t)lat[u] * 2 * m.blocks + b[u]];
         w1[u] = w[((size_t)lat[u] * 2 + 1) * m.blocks + b[u]];
@@ -126,32 +127,16 @@ __global__ void __launch_bounds__(256) planes_bytes_kernel(uint64_t *__restrict_
       if (first + u >= total) break;
       const bool mine = (uint32_t)lane < k[u].bits;
       if (kPack) {
-        uint32_t lo = (uint32_t)v[u], hi = (uint32_t)(v[u] >> 32);
-        if (par[u]) {  // byte 2 q + c to the site of colour c
-          lo = __byte_perm(lo, 0u, 0x2301);
-          hi = __byte_perm(hi, 0u, 0x2301);
-        }
+        const uint2 x = chunk_words(v[u], par[u]);
         uint32_t word[8];
 #pragma unroll
         for (int o = 0; o < 8; ++o)  // bit 1 of a +-1 byte is set for -1
-          word[o] = __ballot_sync(0xffffffffu, mine && ((o < 4 ? lo : hi) >> (8 * (o & 3) + 1) & 1u));
+          word[o] = __ballot_sync(0xffffffffu, mine && ((o < 4 ? x.x : x.y) >> (8 * (o & 3) + 1) & 1u));
         if (lane < 2)
           w[((size_t)lat[u] * 2 + lane) * m.blocks + b[u]] =
               lane ? make_uint4(word[1], word[3], word[5], word[7]) : make_uint4(word[0], word[2], word[4], word[6]);
       } else if (mine) {
-        const uint32_t a[8] = {w0[u].x, w1[u].x, w0[u].y, w1[u].y, w0[u].z, w1[u].z, w0[u].w, w1[u].w};
-        uint32_t lo = 0x01010101u, hi = 0x01010101u;
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          const uint32_t f = (a[o] >> lane & 1u) * (0xFEu << (8 * (o & 3)));  // 0x01 | 0xFE = -1
-          if (o < 4) lo |= f;
-          else hi |= f;
-        }
-        if (par[u]) {
-          lo = __byte_perm(lo, 0u, 0x2301);
-          hi = __byte_perm(hi, 0u, 0x2301);
-        }
-        bytes[chunk_index<kNarrow>(m, k[u], lat[u], lane)] = ((uint64_t)hi << 32) | lo;
+        bytes[chunk_index(m, k[u], lat[u], lane)] = chunk_of(w0[u], w1[u], lane, par[u]);
       }
     }
   }
@@ -214,37 +199,8 @@ cudaError_t transcode(spin_lattice *h, bool pack) {
                          : (narrow(m) ? planes_bytes_kernel<true, false> : planes_bytes_kernel<false, false>);
   unsigned grid = grid_for(total, 16);  // 8 warps of 2 blocks
   if (grid > 152 * 64) grid = 152 * 64;
-  return launch_dependent(kern, dim3(grid), dim3(256), 0, h->stream, (uint64_t *)h->spins, (uint4 *)h->d_pingpong, m,
-                          total, make_fastdiv(m.blocks));
-}
-
-}  // namespace
-
-bool planes_supported(const spin_lattice *h) {
-  return h->d.model == SPIN_ISING && h->d.layout == SPIN_I8 && h->g.L % 8 == 0;
-}
-
-size_t planes_lattice_bytes(const spin_lattice *h) {
-  return (size_t)make_planes(h->g.dim, h->g.L).blocks * 2 * sizeof(uint4);
-}
-
-cudaError_t planes_pack(spin_lattice *h) { return transcode(h, true); }
-cudaError_t planes_unpack(spin_lattice *h) { return transcode(h, false); }
-
-bool planes_reserve(spin_lattice *h) {
-  const size_t bytes = (size_t)h->n_lat * planes_lattice_bytes(h);
-  if (h->d_pingpong && h->pingpong_bytes >= bytes) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-  void *p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (h->d_pingpong) cudaFree(h->d_pingpong);
-  h->d_pingpong = p;
-  h->pingpong_bytes = bytes;
-  return true;
+  return launch_dependent(kern, dim3(grid), dim3(256), 0, h->stream, (uint64_t *)h->spins, (uint4 *)h->d_pingpong, m, total,
+                          make_fastdiv(m.blocks));
 }
 
 cudaError_t planes_sweeps(spin_lattice *h, int64_t n_sweeps) {
@@ -261,6 +217,156 @@ cudaError_t planes_sweeps(spin_lattice *h, int64_t n_sweeps) {
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
+}
+
+// One CTA per lattice with the masks drawn ahead (planes_res.cu) for lattices
+// that fit, unless there are so many that one sweep of masks is large (the
+// phases of so many sites fill the GPU anyway).
+bool resident(const spin_lattice *h) {
+  return planes_res_supported(h) && h->n_lat * h->g.N <= ((int64_t)1 << 26);
+}
+
+// Sweeps, measurements and exchanges of a call.  Its first launch takes the
+// caller's bytes and its last one leaves them there; in between the lattices
+// alternate between two buffers of planes.  An exchange is decided and carried
+// out by the launch that follows it, the call's last one on the bytes.
+int run_resident(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
+                 int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels) {
+  const int64_t nl = h->n_lat;
+  const bool measuring = measure_every > 0 && (E_series || M_series);
+  int64_t done = 0, rows = 0, tape_at = 0, tape_left = 0;
+  int64_t *energies[2] = {h->d_energy, h->d_energy + nl};
+  int which = 0;
+  bool pending = false;  // an exchange with energies[which ^ 1] is due
+  int rc = SPIN_OK, cur = 0;
+  while (done < n_sweeps && rc == SPIN_OK) {
+    const int64_t at = h->sweeps_done;
+    if (tape_left == 0) {
+      cudaError_t e;
+      tape_left = planes_res_draw(h, at, n_sweeps - done, &e);
+      tape_at = 0;
+      if (e != cudaSuccess) return SPIN_ECUDA;
+    }
+    int64_t next = n_sweeps - done;
+    if (pt_every > 0) next = std::min(next, pt_every - at % pt_every);
+    next = std::min(next, tape_left);
+    const bool exchange = pt_every > 0 && (at + next) % pt_every == 0;
+    PlanesResCall call = {};
+    call.every = call.first = 1;
+    if (measuring) {
+      call.E = E_series ? E_series + rows * nl : nullptr;
+      call.M = M_series ? M_series + rows * nl : nullptr;
+      call.every = measure_every;
+      call.first = (int)(measure_every - at % measure_every);
+      rows += (at + next) / measure_every - at / measure_every;
+    }
+    if (exchange) {
+      call.E_last = energies[which];
+      rc = upload_pt_tables_for_batch(h, betas);  // refused: the sweeps up to the exchange still run
+    }
+    call.bytes_in = done == 0;
+    call.bytes_out = rc != SPIN_OK || done + next == n_sweeps;
+    if (pending) {
+      call.E_prev = energies[which ^ 1];
+      call.step = (uint32_t)(h->pt_steps_done - 1);
+      call.accepted = accepted;
+      call.labels = labels;
+    }
+    if (planes_res_sweeps(h, tape_at, next, cur, call) != cudaSuccess) return SPIN_ECUDA;
+    cur ^= 1;
+    pending = false;
+    h->sweeps_done += next;
+    done += next;
+    tape_at += next;
+    tape_left -= next;
+    if (exchange && rc == SPIN_OK) {
+      pending = true;
+      which ^= 1;
+      h->pt_steps_done += 1;
+    }
+  }
+  if (pending) {
+    h->pt_steps_done -= 1;
+    const cudaError_t e = launch_pt_swap(h, nullptr, accepted, labels, energies[which ^ 1]);
+    h->pt_steps_done += 1;
+    if (e != cudaSuccess) return SPIN_ECUDA;
+  }
+  return rc;
+}
+
+// The same with a launch per colour phase, in one buffer.
+int run_phases(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
+               int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels) {
+  const int64_t nl = h->n_lat;
+  const bool measuring = measure_every > 0 && (E_series || M_series);
+  int64_t done = 0, rows = 0;
+  int rc = SPIN_OK;
+  while (done < n_sweeps && rc == SPIN_OK) {
+    const int64_t at = h->sweeps_done;
+    int64_t next = n_sweeps - done;
+    if (measuring) next = std::min(next, measure_every - at % measure_every);
+    if (pt_every > 0) next = std::min(next, pt_every - at % pt_every);
+    if (planes_sweeps(h, next) != cudaSuccess) return SPIN_ECUDA;
+    h->sweeps_done += next;
+    done += next;
+    const int64_t now = h->sweeps_done;
+    const int64_t *energies = nullptr;  // energies measured at this sweep, if any
+    if (measuring && now % measure_every == 0) {
+      if (planes_measure(h, E_series ? E_series + rows * nl : nullptr, M_series ? M_series + rows * nl : nullptr) !=
+          cudaSuccess)
+        return SPIN_ECUDA;
+      if (E_series) energies = E_series + rows * nl;
+      ++rows;
+    }
+    if (pt_every > 0 && now % pt_every == 0) {
+      rc = upload_pt_tables_for_batch(h, betas);
+      if (rc == SPIN_OK && launch_pt_swap(h, nullptr, accepted, labels, energies, h->d_pingpong) != cudaSuccess)
+        return SPIN_ECUDA;
+      if (rc == SPIN_OK) h->pt_steps_done += 1;
+    }
+  }
+  return rc;
+}
+
+}  // namespace
+
+bool planes_supported(const spin_lattice *h) {
+  return h->d.model == SPIN_ISING && h->d.layout == SPIN_I8 && h->g.L % 8 == 0;
+}
+
+size_t planes_lattice_bytes(const spin_lattice *h) {
+  return (size_t)make_planes(h->g.dim, h->g.L).blocks * 2 * sizeof(uint4);
+}
+
+bool planes_ready(spin_lattice *h, int64_t n_sweeps) {
+  if (h->sweeps_done + n_sweeps > (int64_t)0xFFFFFFFFll) return false;  // (refused by the other paths)
+  if (resident(h) && planes_res_reserve(h, n_sweeps)) return true;
+  if (h->variant == 3) return false;
+  const size_t bytes = (size_t)h->n_lat * planes_lattice_bytes(h);
+  if (h->d_pingpong && h->pingpong_bytes >= bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+  void *p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (h->d_pingpong) cudaFree(h->d_pingpong);
+  h->d_pingpong = p;
+  h->pingpong_bytes = bytes;
+  return true;
+}
+
+int planes_run(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
+               int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels) {
+  // (the same test as planes_ready: what it reserved is what runs)
+  const bool res = resident(h) && planes_res_reserve(h, n_sweeps);
+  if (res) return run_resident(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
+  if (transcode(h, true) != cudaSuccess) return SPIN_ECUDA;
+  const int rc = run_phases(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
+  if (rc == SPIN_ECUDA) return rc;
+  // also after a refused exchange: the sweeps up to it stand
+  return transcode(h, false) == cudaSuccess ? rc : SPIN_ECUDA;
 }
 
 cudaError_t planes_measure(spin_lattice *h, int64_t *E, int64_t *M) {

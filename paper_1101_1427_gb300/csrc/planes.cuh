@@ -67,6 +67,34 @@ __device__ __forceinline__ PlaneBlock plane_block(const Planes &m, uint32_t b) {
 
 __device__ __forceinline__ uint32_t low_bits(uint32_t n) { return n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
 
+// The 8-byte chunk v of a call's sites as two words whose byte 2 q + c (of the
+// eight) is the site of colour c in plane q; par: parity of y + z of its row.
+__device__ __forceinline__ uint2 chunk_words(uint64_t v, uint32_t par) {
+  uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
+  if (par) {
+    lo = __byte_perm(lo, 0u, 0x2301);
+    hi = __byte_perm(hi, 0u, 0x2301);
+  }
+  return make_uint2(lo, hi);
+}
+
+// The chunk of bit `lane` of a block's planes w0, w1 (colours 0 and 1).
+__device__ __forceinline__ uint64_t chunk_of(const uint4 &w0, const uint4 &w1, int lane, uint32_t par) {
+  const uint32_t a[8] = {w0.x, w1.x, w0.y, w1.y, w0.z, w1.z, w0.w, w1.w};
+  uint32_t lo = 0x01010101u, hi = 0x01010101u;
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    const uint32_t f = (a[o] >> lane & 1u) * (0xFEu << (8 * (o & 3)));  // 0x01 | 0xFE = -1
+    if (o < 4) lo |= f;
+    else hi |= f;
+  }
+  if (par) {
+    lo = __byte_perm(lo, 0u, 0x2301);
+    hi = __byte_perm(hi, 0u, 0x2301);
+  }
+  return ((uint64_t)hi << 32) | lo;
+}
+
 // The neighbours of the sites of block k of colour c in the other colour's
 // blocks O: per plane the sites above and below (y -+ 1), the two beside
 // (x -+ 1; which is which does not matter) and, in 3D, in front and behind.

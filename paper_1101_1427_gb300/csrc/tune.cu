@@ -70,7 +70,7 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
       if (spin_set_variant(h, v) == SPIN_OK) cand.emplace_back(v, h->order_tile);
       apply(start);
     }
-    if (h->auto_form && spin::planes_wanted(h, n_sweeps)) cand.push_back(start);
+    if (h->auto_form && spin::planes_wanted(h, n_sweeps, 0)) cand.push_back(start);
   } else {
     cand.push_back(start);
   }
