@@ -141,24 +141,6 @@ __device__ bool team_barrier(Sync &sy) {
   return s_ok != 0;
 }
 
-// counter planes += 3-bit value (x0, x1, x2)
-__device__ __forceinline__ void add3(uint32_t (&C)[kPl], uint32_t x0, uint32_t x1, uint32_t x2) {
-  uint32_t c = C[0] & x0;
-  C[0] ^= x0;
-  uint32_t t = C[1] ^ x1 ^ c;
-  c = (C[1] & x1) | (c & (C[1] ^ x1));
-  C[1] = t;
-  t = C[2] ^ x2 ^ c;
-  c = (C[2] & x2) | (c & (C[2] ^ x2));
-  C[2] = t;
-#pragma unroll
-  for (int k = 3; k < kPl; ++k) {
-    const uint32_t n = C[k] & c;
-    C[k] ^= c;
-    c = n;
-  }
-}
-
 // Harley-Seal counting of 1-bit planes: eight planes go through seven
 // carry-save adders into (ones, twos, fours) and one plane of weight 8,
 // which is rippled into the counter; flush() adds the remainders.
@@ -279,16 +261,26 @@ __device__ __forceinline__ void ea_phase_warp(uint32_t *__restrict__ s, const ui
                                               uint32_t lid, int colour, uint32_t t4, uint32_t t8,
                                               uint32_t t12, uint32_t first, uint32_t stride,
                                               uint32_t (&C)[kPl]) {
-  const uint32_t quads = (U.N / 2 + 3) / 4;
-  const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
   uint32_t buf[4][3];
   int n = 0;
+  if ((U.L & 7) != 0) {  // whole warps: lanes take consecutive sites
+    ea_sites_phase(s, Jg, colour, (uint32_t)U.L, U.N, U.fL, rk, sweep, lid, t4, t8, t12, first >> 5, stride >> 5,
+                   [&](const Flip &f, bool on) {
+                     if (!kCount) return;
+                     uint32_t a0 = 0, a1 = 0, a2 = 0;
+                     if (on) ea_after(f, a0, a1, a2);
+                     AddTo{C, buf, n}(a0, a1, a2);  // four sites per 128: the buffer is empty at the end
+                   });
+    return;
+  }
+  const uint32_t quads = U.N / 8;
+  const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
   for (uint32_t j4 = first; j4 < quads; j4 += stride) {
     const uint4 r = philox(make_uint4(j4, sweep, lid, wctr), rk);
-    ea_cs_quad<kCount>(s, Jg, j4, colour, (uint32_t)U.L, U.N, U.fL, r, t4, t8, t12, AddTo{C, buf, n});
+    const EaQuadGeom q = ea_quad_geom<3>(j4, colour, (uint32_t)U.L, U.fL);
+    ea_quad_update<3, kCount>(s, q, ea_quad_couplings<3>(Jg, q, colour, U.N), colour, U.N, r, t4, t8, t12,
+                              AddTo{C, buf, n});
   }
-  if (kCount)  // a last, partial quad (N/2 not a multiple of 4)
-    for (int k = 0; k < n; ++k) add3(C, buf[k][0], buf[k][1], buf[k][2]);
 }
 
 // Counts per bit the words a[i] (or a[i] ^ b[i]) for i = lane, lane + 32, ...

@@ -246,78 +246,115 @@ __device__ __forceinline__ void ea_quad_update(uint32_t *__restrict__ w, const E
   *reinterpret_cast<uint4 *>(own + q.j0) = make_uint4(nw[0], nw[1], nw[2], nw[3]);
 }
 
-// Update of the quad j = 4 j4 .. 4 j4 + 3 of colour `colour` in one
-// word-lattice w (colour-split) with group couplings J (colour-split).
-// Any even L: per-site neighbour indices.  add(a0, a1, a2) receives the
-// post-update count of each site when kCount.
-template <bool kCount, typename AddFn>
-__device__ __forceinline__ void ea_cs_quad(uint32_t *__restrict__ w, const uint32_t *__restrict__ J,
-                                           uint32_t j4, int colour, uint32_t L, uint32_t N,
-                                           const FastDiv &fL, uint4 r, uint32_t t4, uint32_t t8,
-                                           uint32_t t12, AddFn add) {
-  const uint32_t half = N >> 1;
-  const uint32_t oc = (uint32_t)colour ^ 1u;
-  uint32_t *own = w + (uint32_t)colour * half;
-  const uint32_t *oth = w + oc * half;
-  const uint32_t *Jx = J, *Jy = J + N, *Jz = J + 2 * N;
-  const uint32_t co = (uint32_t)colour * half, ot = oc * half;
-  if ((L & 7u) == 0) {
-    const EaQuadGeom q = ea_quad_geom<3>(j4, colour, L, fL);
-    ea_quad_update<3, kCount>(w, q, ea_quad_couplings<3>(J, q, colour, N), colour, N, r, t4, t8, t12, add);
-    return;
-  }
-  const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-  for (uint32_t k = 0; k < 4; ++k) {
-    const uint32_t j = 4 * j4 + k;
-    if (j >= half) break;
-    const CsSite st = cs_site(j, colour, L, fL);
-    const uint32_t S = own[j];
-    const Flip f = ea_flip(S ^ oth[st.xp >> 1] ^ Jx[co + j], S ^ oth[st.xm >> 1] ^ Jx[ot + (st.xm >> 1)],
-                           S ^ oth[st.yp >> 1] ^ Jy[co + j], S ^ oth[st.ym >> 1] ^ Jy[ot + (st.ym >> 1)],
-                           S ^ oth[st.zp >> 1] ^ Jz[co + j], S ^ oth[st.zm >> 1] ^ Jz[ot + (st.zm >> 1)],
-                           rr[k], t4, t8, t12);
-    own[j] = S ^ f.F;
-    if (kCount) {
-      uint32_t a0, a1, a2;
-      ea_after(f, a0, a1, a2);
-      add(a0, a1, a2);
-    }
-  }
+// ---------------------------------------------------------------- sites
+// For L % 8 != 0 a quad of colour indices crosses rows, and a thread that
+// took the quad would read every word of its four sites and neighbours by
+// itself, four words apart from the next lane's.  So lanes take consecutive
+// sites: each warp load is then contiguous.  A Philox call serves four
+// consecutive sites; the four lanes of a quad draw four different calls and
+// pass the words on.
+
+// Lane q of a quad of lanes holds the words v[0..3] of its call; afterwards
+// v[s] is word q of the call of lane s (a 4 x 4 transpose).
+__device__ __forceinline__ void quad_transpose(uint32_t (&v)[4]) {
+  const uint32_t q = threadIdx.x & 3u;
+  uint32_t x = (q & 1u) ? v[0] : v[1], y = (q & 1u) ? v[2] : v[3];
+  x = __shfl_xor_sync(0xffffffffu, x, 1);
+  y = __shfl_xor_sync(0xffffffffu, y, 1);
+  if (q & 1u) v[0] = x, v[2] = y;
+  else v[1] = x, v[3] = y;
+  x = (q & 2u) ? v[0] : v[2];
+  y = (q & 2u) ? v[1] : v[3];
+  x = __shfl_xor_sync(0xffffffffu, x, 2);
+  y = __shfl_xor_sync(0xffffffffu, y, 2);
+  if (q & 2u) v[0] = x, v[1] = y;
+  else v[2] = x, v[3] = y;
 }
 
-// Update of the quad j = 4 j4 .. 4 j4 + 3 of colour `colour` in one 2D
-// word-lattice w with group couplings J ([2][colour][N/2]), as ea_cs_quad.
-template <bool kCount, typename AddFn>
-__device__ __forceinline__ void ea_cs_quad2(uint32_t *__restrict__ w, const uint32_t *__restrict__ J,
-                                            uint32_t j4, int colour, uint32_t L, uint32_t N,
-                                            const FastDiv &fL, uint4 r, uint32_t t4, uint32_t t8, AddFn add) {
+// Colour indices of the neighbours of a site and the words of its bonds; the
+// z entries are unused in 2D.
+struct EaSite {
+  uint32_t j, xp, xm, yp, ym, zp, zm;
+};
+
+struct EaSiteJ {
+  uint32_t xp, xm, yp, ym, zp, zm;
+};
+
+template <int kDim>
+__device__ __forceinline__ EaSite ea_site(uint32_t j, int colour, uint32_t L, const FastDiv &fL) {
+  const CsSite st = kDim == 3 ? cs_site(j, colour, L, fL) : cs_site2(j, colour, L, fL);
+  EaSite e;
+  e.j = j;
+  e.xp = st.xp >> 1;
+  e.xm = st.xm >> 1;
+  e.yp = st.yp >> 1;
+  e.ym = st.ym >> 1;
+  e.zp = st.zp >> 1;
+  e.zm = st.zm >> 1;
+  return e;
+}
+
+template <int kDim>
+__device__ __forceinline__ EaSiteJ ea_site_couplings(const uint32_t *__restrict__ J, const EaSite &e, int colour,
+                                                     uint32_t N) {
+  const uint32_t half = N >> 1, co = (uint32_t)colour * half, ot = ((uint32_t)colour ^ 1u) * half;
+  EaSiteJ c;
+  c.xp = J[co + e.j];
+  c.xm = J[ot + e.xm];
+  c.yp = J[N + co + e.j];
+  c.ym = J[N + ot + e.ym];
+  c.zp = kDim == 3 ? J[2 * N + co + e.j] : 0u;
+  c.zm = kDim == 3 ? J[2 * N + ot + e.zm] : 0u;
+  return c;
+}
+
+// Metropolis update of the site in word-lattice w with uniform r; returns the
+// flip mask and the bit-sliced count of unsatisfied bonds before it.
+template <int kDim>
+__device__ __forceinline__ Flip ea_site_update(uint32_t *__restrict__ w, const EaSite &e, const EaSiteJ &c, int colour,
+                                               uint32_t N, uint32_t r, uint32_t t4, uint32_t t8, uint32_t t12) {
   const uint32_t half = N >> 1;
-  const uint32_t oc = (uint32_t)colour ^ 1u;
   uint32_t *own = w + (uint32_t)colour * half;
-  const uint32_t *oth = w + oc * half;
-  const uint32_t *Jx = J, *Jy = J + N;
-  const uint32_t co = (uint32_t)colour * half, ot = oc * half;
-  if ((L & 7u) == 0) {
-    const EaQuadGeom q = ea_quad_geom<2>(j4, colour, L, fL);
-    ea_quad_update<2, kCount>(w, q, ea_quad_couplings<2>(J, q, colour, N), colour, N, r, t4, t8, 0u, add);
-    return;
-  }
-  const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
+  const uint32_t *oth = w + ((uint32_t)colour ^ 1u) * half;
+  const uint32_t S = own[e.j];
+  Flip f;
+  if (kDim == 3)
+    f = ea_flip(S ^ oth[e.xp] ^ c.xp, S ^ oth[e.xm] ^ c.xm, S ^ oth[e.yp] ^ c.yp, S ^ oth[e.ym] ^ c.ym,
+                S ^ oth[e.zp] ^ c.zp, S ^ oth[e.zm] ^ c.zm, r, t4, t8, t12);
+  else
+    f = ea_flip2(S ^ oth[e.xp] ^ c.xp, S ^ oth[e.xm] ^ c.xm, S ^ oth[e.yp] ^ c.yp, S ^ oth[e.ym] ^ c.ym, r, t4, t8);
+  own[e.j] = S ^ f.F;
+  return f;
+}
+
+// One colour phase of one 3D word-lattice by the warps `warp`, warp + warps,
+// ... (all lanes), each 128 consecutive colour indices at a time: lane l draws
+// the call of quad l of them, and sites 32 s + l take their words from lane
+// 8 s + l / 4.  add(f, on) receives each site's Flip and whether the lane has
+// a site.
+template <typename AddFn>
+__device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, int colour,
+                                               uint32_t L, uint32_t N, const FastDiv &fL, const RoundKeys &rk,
+                                               uint32_t sweep, uint32_t lid, uint32_t t4, uint32_t t8, uint32_t t12,
+                                               uint32_t warp, uint32_t warps, AddFn add) {
+  const uint32_t half = N >> 1, lane = threadIdx.x & 31u, wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
+  for (uint32_t base = 128u * warp; base < half; base += 128u * warps) {
+    const uint4 v = philox(make_uint4((base >> 2) + lane, sweep, lid, wctr), rk);
 #pragma unroll
-  for (uint32_t k = 0; k < 4; ++k) {
-    const uint32_t j = 4 * j4 + k;
-    if (j >= half) break;
-    const CsSite st = cs_site2(j, colour, L, fL);
-    const uint32_t S = own[j];
-    const Flip f = ea_flip2(S ^ oth[st.xp >> 1] ^ Jx[co + j], S ^ oth[st.xm >> 1] ^ Jx[ot + (st.xm >> 1)],
-                            S ^ oth[st.yp >> 1] ^ Jy[co + j], S ^ oth[st.ym >> 1] ^ Jy[ot + (st.ym >> 1)], rr[k],
-                            t4, t8);
-    own[j] = S ^ f.F;
-    if (kCount) {
-      uint32_t a0, a1, a2;
-      ea_after2(f, a0, a1, a2);
-      add(a0, a1, a2);
+    for (uint32_t s = 0; s < 4; ++s) {
+      const uint32_t from = 8u * s + (lane >> 2);
+      const uint32_t x = __shfl_sync(0xffffffffu, v.x, from), y = __shfl_sync(0xffffffffu, v.y, from);
+      const uint32_t z = __shfl_sync(0xffffffffu, v.z, from), u = __shfl_sync(0xffffffffu, v.w, from);
+      const uint32_t r = (lane & 2u) ? ((lane & 1u) ? u : z) : ((lane & 1u) ? y : x);
+      const uint32_t j = base + 32u * s + lane;
+      const bool on = j < half;
+      Flip f = {};
+      if (on) {
+        const EaSite e = ea_site<3>(j, colour, L, fL);
+        f = ea_site_update<3>(w, e, ea_site_couplings<3>(J, e, colour, N), colour, N, r, t4, t8, t12);
+      }
+      add(f, on);
     }
   }
 }

@@ -57,68 +57,101 @@ struct NoAdd {
   __device__ void operator()(uint32_t, uint32_t, uint32_t) const {}
 };
 
-// One quad update in kDim dimensions (the group's couplings start at J), any L.
-template <int kDim>
-__device__ __forceinline__ void ea_quad(uint32_t *w, const uint32_t *J, uint32_t j4, int colour, uint32_t L,
-                                        uint32_t N, const FastDiv &fL, uint4 r, uint32_t t4, uint32_t t8,
-                                        uint32_t t12) {
-  if (kDim == 3)
-    ea_cs_quad<false>(w, J, j4, colour, L, N, fL, r, t4, t8, t12, NoAdd());
-  else
-    ea_cs_quad2<false>(w, J, j4, colour, L, N, fL, r, t4, t8, NoAdd());
+constexpr uint32_t kSlots = 4;  // slots of one (set, group) per thread of a colour phase
+
+// Place of thread item k: (a, grp) and the first slot of its block, with the
+// item's number among those of the slot block (fquads: quads per colour).
+struct EaItem {
+  uint32_t st, a, grp, t0, t1, j4;
+};
+
+__device__ __forceinline__ EaItem ea_item(const Geom &g, uint32_t k, const FastDiv &ftb) {
+  const uint32_t quads = ((uint32_t)g.N / 2 + 3) / 4;
+  const uint32_t G = (uint32_t)g.n_real / 32, T = (uint32_t)g.n_temps, TB = (T + kSlots - 1) / kSlots;
+  EaItem x;
+  const uint32_t sb = fdiv(k, g.fquads);
+  x.j4 = k - sb * quads;
+  x.st = fdiv(sb, ftb);  // sb = (a G + grp) TB + tb
+  x.a = fdiv(x.st, g.fgrp);
+  x.grp = x.st - x.a * G;
+  x.t0 = (sb - x.st * TB) * kSlots;
+  x.t1 = min(x.t0 + kSlots, T);
+  return x;
 }
 
-// Slots per thread of msc_phase_kernel: four when the updates can share the
-// quad's geometry and couplings (L % 8 == 0), else one.
-__host__ __device__ constexpr uint32_t ea_slots(bool row_quads) { return row_quads ? 4u : 1u; }
-
-// One colour phase over all word-lattices.  Thread k takes one quad of
-// colour sites (j4) in the word-lattices (a, grp, t) of kS consecutive
-// slots t of one replica set a and group grp, one slot after the other.
-// When L % 8 == 0 those updates share the quad's geometry and coupling
-// words, read once (ea_cs.cuh); each word-lattice draws its own uniforms,
-// so the mapping of updates to threads does not change the result.
-// kPair (w = 64, Sec. 5: 64 spins per variable): groups 2q and 2q + 1 of
-// one (set, slot) share their uniforms, keyed by q.  kRowQuads: L % 8 == 0
-// (else every site takes its own neighbour indices).  ftb divides by the
-// number of slot blocks ceil(n_temps / kS).  Register bounds: two CTAs per
-// SM for the shared form (its coupling words stay live across the slots),
-// three for the generic one.
-template <int kDim, bool kPair, bool kRowQuads>
-__global__ void __launch_bounds__(256, kRowQuads ? 2 : 3)
+// One colour phase over all word-lattices, L % 8 == 0.  Thread k takes one
+// quad of colour sites (j4) in the word-lattices (a, grp, t) of kSlots
+// consecutive slots t of one replica set a and group grp, one slot after the
+// other.  Those updates share the quad's geometry and coupling words, read
+// once (ea_cs.cuh); each word-lattice draws its own uniforms, so the mapping
+// of updates to threads does not change the result.  kPair (w = 64, Sec. 5:
+// 64 spins per variable): groups 2q and 2q + 1 of one (set, slot) share their
+// uniforms, keyed by q.  ftb divides by the number of slot blocks.  Register
+// bound: two CTAs per SM (the coupling words stay live across the slots).
+// The geometry does not depend on the previous phase and comes before
+// griddep_wait().
+template <int kDim, bool kPair>
+__global__ void __launch_bounds__(256, 2)
     msc_phase_kernel(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, Geom g, uint32_t total,
                      FastDiv ftb, const uint32_t *__restrict__ thr, RoundKeys rk, uint32_t sweep, int colour) {
-  griddep_wait();
   griddep_release();
-  const uint32_t L = (uint32_t)g.L, N = (uint32_t)g.N, quads = (N / 2 + 3) / 4;
-  constexpr uint32_t kS = ea_slots(kRowQuads);
-  const uint32_t G = (uint32_t)g.n_real / 32, T = (uint32_t)g.n_temps, TB = (T + kS - 1) / kS;
-  const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
-  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
-    const uint32_t sb = fdiv(k, g.fquads), j4 = k - sb * quads;
-    const uint32_t st = fdiv(sb, ftb), tb = sb - st * TB;  // sb = (a G + grp) TB + tb
-    const uint32_t a = fdiv(st, g.fgrp), grp = st - a * G;
-    const uint32_t rkey = kPair ? grp >> 1 : grp;
-    uint32_t *ws = w + (size_t)st * T * N;  // slot t of (a, grp) is word-lattice st T + t
-    const uint32_t *Jg = J + (size_t)grp * kDim * N;
-    const uint32_t t0 = tb * kS, t1 = t0 + kS < T ? t0 + kS : T;
-    if (kRowQuads) {
-      const EaQuadGeom q = ea_quad_geom<kDim>(j4, colour, L, g.fL);
-      const EaQuadJ c = ea_quad_couplings<kDim>(Jg, q, colour, N);
+  const uint32_t N = (uint32_t)g.N, wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= total) return;
+  const EaItem x = ea_item(g, k, ftb);
+  const uint32_t rkey = kPair ? x.grp >> 1 : x.grp;
+  uint32_t *ws = w + (size_t)x.st * (uint32_t)g.n_temps * N;  // slot t of (a, grp) is word-lattice st T + t
+  const EaQuadGeom q = ea_quad_geom<kDim>(x.j4, colour, (uint32_t)g.L, g.fL);
+  griddep_wait();
+  const EaQuadJ c = ea_quad_couplings<kDim>(J + (size_t)x.grp * kDim * N, q, colour, N);
 #pragma unroll 1
-      for (uint32_t t = t0; t < t1; ++t) {
-        const uint4 r = philox(make_uint4(j4, sweep, lattice_id(a, rkey, t), wctr), rk);
-        const uint32_t t4 = __ldg(thr + 4 * t + 1), t8 = __ldg(thr + 4 * t + 2);
-        const uint32_t t12 = kDim == 3 ? __ldg(thr + 4 * t + 3) : 0u;
-        ea_quad_update<kDim, false>(ws + (size_t)t * N, q, c, colour, N, r, t4, t8, t12, NoAdd());
-      }
-    } else {
-      const uint32_t t = t0;  // kS = 1: the slot block is the slot
-      const uint4 r = philox(make_uint4(j4, sweep, lattice_id(a, rkey, t), wctr), rk);
-      const uint32_t t4 = __ldg(thr + 4 * t + 1), t8 = __ldg(thr + 4 * t + 2);
-      const uint32_t t12 = kDim == 3 ? __ldg(thr + 4 * t + 3) : 0u;
-      ea_quad<kDim>(ws + (size_t)t * N, Jg, j4, colour, L, N, g.fL, r, t4, t8, t12);
-    }
+  for (uint32_t t = x.t0; t < x.t1; ++t) {
+    const uint4 r = philox(make_uint4(x.j4, sweep, lattice_id(x.a, rkey, t), wctr), rk);
+    const uint32_t t4 = __ldg(thr + 4 * t + 1), t8 = __ldg(thr + 4 * t + 2);
+    const uint32_t t12 = kDim == 3 ? __ldg(thr + 4 * t + 3) : 0u;
+    ea_quad_update<kDim, false>(ws + (size_t)t * N, q, c, colour, N, r, t4, t8, t12, NoAdd());
+  }
+}
+
+// The same for any even L.  Thread k takes one site (lanes consecutive colour
+// indices, so that every load of a warp is contiguous) in up to kSlots slots,
+// with its neighbour indices and coupling words found once; the four lanes of
+// a quad draw the calls of four slots and exchange their words (quad_transpose).
+// A thread per quad and slot read its words four apart from the next lane's and
+// looked up each site's geometry and couplings again for every slot: 10 sweeps
+// of 256 x 30 x 2 lattices of L = 12 with 2 measurements and exchanges took 151
+// us, 135 here.
+template <int kDim, bool kPair>
+__global__ void __launch_bounds__(256)
+    msc_site_phase_kernel(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, Geom g, uint32_t total,
+                          FastDiv ftb, const uint32_t *__restrict__ thr, RoundKeys rk, uint32_t sweep, int colour) {
+  griddep_release();
+  const uint32_t N = (uint32_t)g.N;
+  const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x, lane4 = id & 3u;
+  const EaItem x = ea_item(g, min(id >> 2, total - 1), ftb);  // (lanes beyond the end draw the last quad again)
+  const uint32_t rkey = kPair ? x.grp >> 1 : x.grp;
+  uint32_t r[kSlots];
+  {
+    const uint4 v = philox(make_uint4(x.j4, sweep, lattice_id(x.a, rkey, min(x.t0 + lane4, x.t1 - 1)),
+                                      ctr_w(TAG_UPDATE, (uint32_t)colour, 0)), rk);
+    r[0] = v.x;
+    r[1] = v.y;
+    r[2] = v.z;
+    r[3] = v.w;
+  }
+  quad_transpose(r);  // r[s]: the site's word in slot t0 + s
+  const uint32_t j = 4 * x.j4 + lane4;
+  if ((id >> 2) >= total || j >= N / 2) return;
+  const EaSite e = ea_site<kDim>(j, colour, (uint32_t)g.L, g.fL);
+  uint32_t *ws = w + (size_t)x.st * (uint32_t)g.n_temps * N;
+  griddep_wait();
+  const EaSiteJ c = ea_site_couplings<kDim>(J + (size_t)x.grp * kDim * N, e, colour, N);
+#pragma unroll
+  for (uint32_t s = 0; s < kSlots; ++s) {
+    const uint32_t t = x.t0 + s;
+    if (t >= x.t1) break;
+    ea_site_update<kDim>(ws + (size_t)t * N, e, c, colour, N, r[s], __ldg(thr + 4 * t + 1), __ldg(thr + 4 * t + 2),
+                         kDim == 3 ? __ldg(thr + 4 * t + 3) : 0u);
   }
 }
 
@@ -186,20 +219,20 @@ cudaError_t launch_sweeps_msc_ea(spin_lattice *h, const uint32_t *J, int64_t n_s
   const RoundKeys rk = make_round_keys(h->d.seed);
   const bool pair = h->msc_width == 64;
   const bool row_quads = g.L % 8 == 0;
-  const uint32_t TB = ((uint32_t)g.n_temps + ea_slots(row_quads) - 1) / ea_slots(row_quads);
+  const uint32_t TB = ((uint32_t)g.n_temps + kSlots - 1) / kSlots;
   const uint32_t work = (uint32_t)g.n_sets * (uint32_t)(g.n_real / 32) * TB * (uint32_t)((g.N / 2 + 3) / 4);
   const FastDiv ftb = make_fastdiv(TB);
-  using Kern = decltype(&msc_phase_kernel<3, false, true>);
-  const Kern kerns[2][2][2] = {
-      {{msc_phase_kernel<2, false, false>, msc_phase_kernel<2, false, true>},
-       {msc_phase_kernel<2, true, false>, msc_phase_kernel<2, true, true>}},
-      {{msc_phase_kernel<3, false, false>, msc_phase_kernel<3, false, true>},
-       {msc_phase_kernel<3, true, false>, msc_phase_kernel<3, true, true>}}};
+  using Kern = decltype(&msc_phase_kernel<3, false>);
+  const Kern kerns[2][2][2] = {{{msc_site_phase_kernel<2, false>, msc_phase_kernel<2, false>},
+                                {msc_site_phase_kernel<2, true>, msc_phase_kernel<2, true>}},
+                               {{msc_site_phase_kernel<3, false>, msc_phase_kernel<3, false>},
+                                {msc_site_phase_kernel<3, true>, msc_phase_kernel<3, true>}}};
   const Kern kern = kerns[g.dim == 3][pair][row_quads];
+  const int64_t threads = row_quads ? work : 4 * (int64_t)work;  // < 2^30: fewer than 2^27 words
   for (int64_t k = 0; k < n_sweeps; ++k) {
     const uint32_t sweep = (uint32_t)(h->sweeps_done + k);
     for (int colour = 0; colour < 2; ++colour) {
-      const cudaError_t e = launch_dependent(kern, dim3(capped(work)), dim3(256), 0, h->stream,
+      const cudaError_t e = launch_dependent(kern, dim3(grid_for(threads, 256)), dim3(256), 0, h->stream,
                                              (uint32_t *)h->spins, J, g, work, ftb, (const uint32_t *)h->d_thr,
                                              rk, sweep, colour);
       if (e != cudaSuccess) return e;
