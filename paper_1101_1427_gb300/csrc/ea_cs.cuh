@@ -309,23 +309,36 @@ __device__ __forceinline__ EaSiteJ ea_site_couplings(const uint32_t *__restrict_
   return c;
 }
 
-// Metropolis update of the site in word-lattice w with uniform r; returns the
-// flip mask and the bit-sliced count of unsatisfied bonds before it.
+// The words of a site and its neighbours in word-lattice w.
+struct EaSiteW {
+  uint32_t S, xp, xm, yp, ym, zp, zm;
+};
+
 template <int kDim>
-__device__ __forceinline__ Flip ea_site_update(uint32_t *__restrict__ w, const EaSite &e, const EaSiteJ &c, int colour,
-                                               uint32_t N, uint32_t r, uint32_t t4, uint32_t t8, uint32_t t12) {
+__device__ __forceinline__ EaSiteW ea_site_words(const uint32_t *__restrict__ w, const EaSite &e, int colour,
+                                                 uint32_t N) {
   const uint32_t half = N >> 1;
-  uint32_t *own = w + (uint32_t)colour * half;
   const uint32_t *oth = w + ((uint32_t)colour ^ 1u) * half;
-  const uint32_t S = own[e.j];
-  Flip f;
+  EaSiteW x;
+  x.S = w[(uint32_t)colour * half + e.j];
+  x.xp = oth[e.xp];
+  x.xm = oth[e.xm];
+  x.yp = oth[e.yp];
+  x.ym = oth[e.ym];
+  x.zp = kDim == 3 ? oth[e.zp] : 0u;
+  x.zm = kDim == 3 ? oth[e.zm] : 0u;
+  return x;
+}
+
+// Metropolis flip mask of the site with uniform r, and the bit-sliced count
+// of its unsatisfied bonds.
+template <int kDim>
+__device__ __forceinline__ Flip ea_site_flip(const EaSiteW &x, const EaSiteJ &c, uint32_t r, uint32_t t4, uint32_t t8,
+                                             uint32_t t12) {
   if (kDim == 3)
-    f = ea_flip(S ^ oth[e.xp] ^ c.xp, S ^ oth[e.xm] ^ c.xm, S ^ oth[e.yp] ^ c.yp, S ^ oth[e.ym] ^ c.ym,
-                S ^ oth[e.zp] ^ c.zp, S ^ oth[e.zm] ^ c.zm, r, t4, t8, t12);
-  else
-    f = ea_flip2(S ^ oth[e.xp] ^ c.xp, S ^ oth[e.xm] ^ c.xm, S ^ oth[e.yp] ^ c.yp, S ^ oth[e.ym] ^ c.ym, r, t4, t8);
-  own[e.j] = S ^ f.F;
-  return f;
+    return ea_flip(x.S ^ x.xp ^ c.xp, x.S ^ x.xm ^ c.xm, x.S ^ x.yp ^ c.yp, x.S ^ x.ym ^ c.ym, x.S ^ x.zp ^ c.zp,
+                   x.S ^ x.zm ^ c.zm, r, t4, t8, t12);
+  return ea_flip2(x.S ^ x.xp ^ c.xp, x.S ^ x.xm ^ c.xm, x.S ^ x.yp ^ c.yp, x.S ^ x.ym ^ c.ym, r, t4, t8);
 }
 
 // One colour phase of one 3D word-lattice by the warps `warp`, warp + warps,
@@ -344,15 +357,17 @@ __device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const u
 #pragma unroll
     for (uint32_t s = 0; s < 4; ++s) {
       const uint32_t from = 8u * s + (lane >> 2);
-      const uint32_t x = __shfl_sync(0xffffffffu, v.x, from), y = __shfl_sync(0xffffffffu, v.y, from);
-      const uint32_t z = __shfl_sync(0xffffffffu, v.z, from), u = __shfl_sync(0xffffffffu, v.w, from);
-      const uint32_t r = (lane & 2u) ? ((lane & 1u) ? u : z) : ((lane & 1u) ? y : x);
+      const uint32_t r0 = __shfl_sync(0xffffffffu, v.x, from), r1 = __shfl_sync(0xffffffffu, v.y, from);
+      const uint32_t r2 = __shfl_sync(0xffffffffu, v.z, from), r3 = __shfl_sync(0xffffffffu, v.w, from);
+      const uint32_t r = (lane & 2u) ? ((lane & 1u) ? r3 : r2) : ((lane & 1u) ? r1 : r0);
       const uint32_t j = base + 32u * s + lane;
       const bool on = j < half;
       Flip f = {};
       if (on) {
         const EaSite e = ea_site<3>(j, colour, L, fL);
-        f = ea_site_update<3>(w, e, ea_site_couplings<3>(J, e, colour, N), colour, N, r, t4, t8, t12);
+        const EaSiteW x = ea_site_words<3>(w, e, colour, N);
+        f = ea_site_flip<3>(x, ea_site_couplings<3>(J, e, colour, N), r, t4, t8, t12);
+        w[(uint32_t)colour * half + j] = x.S ^ f.F;
       }
       add(f, on);
     }

@@ -137,161 +137,21 @@ __global__ void overlap_i8_kernel(const int8_t *__restrict__ s, Geom g, long lon
 // ---------------------------------------------------------------- EA, coded words
 // Per word-lattice (a, g, t) and realisation bit b: the number of
 // unsatisfied bonds, of down spins and (set 0 only) of spins that differ
-// from set 1.  Each thread adds its words into bit-sliced vertical counters
-// (plane k holds bit k of 32 per-realisation counts); the counters of a warp
-// are added with shuffles, those of the warps through shared memory, and
-// lane b of warp 0 finally reads count b out of the planes.
-constexpr int kThr = 6;   // per-thread planes: at most 16 sites x 3 bonds = 48 < 64
-constexpr int kWarp = 11; // per-warp planes: at most 32 x 48 = 1536 < 2048
-
-// counter += one bit-plane of weight 2^w
-template <int K>
-__device__ __forceinline__ void vc_add(uint32_t (&C)[K], uint32_t v, int w) {
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    if (k < w) continue;
-    const uint32_t c = C[k] & v;
-    C[k] ^= v;
-    v = c;
-  }
-}
-
-// Sums the per-thread counters of the block; lane b of warp 0 gets count b.
-__device__ long long vc_block_total(const uint32_t (&c)[kThr], uint32_t (*sm)[kWarp]) {
-  uint32_t C[kWarp];
-#pragma unroll
-  for (int k = 0; k < kWarp; ++k) C[k] = k < kThr ? c[k] : 0u;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {  // bit-sliced ripple-carry adds across the warp
-    uint32_t carry = 0;
-#pragma unroll
-    for (int k = 0; k < kWarp; ++k) {
-      const uint32_t a = C[k], b = __shfl_xor_sync(0xffffffffu, C[k], o);
-      C[k] = a ^ b ^ carry;
-      carry = (a & b) | (carry & (a ^ b));
-    }
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < kWarp; ++k) sm[wid][k] = C[k];
-  __syncthreads();
-  long long tot = 0;
-  if (wid == 0) {
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-#pragma unroll
-      for (int k = 0; k < kWarp; ++k) tot += (long long)((sm[w][k] >> lane) & 1u) << k;
-  }
-  __syncthreads();
-  return tot;
-}
-
-template <int kDim>
-__global__ void __launch_bounds__(256) measure_msc_kernel(const uint32_t *__restrict__ w,
-                                                          const uint32_t *__restrict__ J, Geom g,
-                                                          long long *__restrict__ E,
-                                                          long long *__restrict__ M,
-                                                          long long *__restrict__ Q) {
-  griddep_wait();
-  griddep_release();
-  __shared__ uint32_t sm[8][kWarp];
-  const uint32_t G = (uint32_t)g.n_real / 32, T = (uint32_t)g.n_temps;
-  const uint32_t wl = blockIdx.y;
-  const uint32_t t = wl % T, grp = (wl / T) % G, a = wl / (T * G);
-  const uint32_t L = (uint32_t)g.L, N = (uint32_t)g.N;
-  const uint32_t *s = w + (size_t)wl * N;
-  const uint32_t *Jg = J + (size_t)grp * kDim * N;
-  const bool do_q = Q && a == 0 && g.n_sets >= 2;
-  const uint32_t *s1 = s + (size_t)G * T * N;  // set 1, same (g, t)
-  uint32_t CE[kThr] = {}, CM[kThr] = {}, CQ[kThr] = {};
-  const uint32_t half = N / 2;
-  // the bonds (i, i + e_d) of every site count each bond once
-  if ((L & 7u) == 0) {
-    // four consecutive colour indices of one row per step, 16-byte loads
-    const uint32_t quads = half / 4, LH = L / 2;
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < 2 * quads; q += gridDim.x * blockDim.x) {
-      const int c = q >= quads ? 1 : 0;
-      const uint32_t j0 = 4 * (q - (uint32_t)c * quads);
-      const uint32_t co = (uint32_t)c * half, oc = (uint32_t)(c ^ 1) * half;
-      const CsSite st = kDim == 3 ? cs_site(j0, c, L, g.fL) : cs_site2(j0, c, L, g.fL);
-      const uint32_t p = st.i & 1u, jr = st.rb >> 1;
-      const uint4 S = ldv4(s + co + j0), O = ldv4(s + oc + j0);
-      // x + 1: the other colour at the same index (p = 0) or the next (p = 1)
-      const uint32_t jx = j0 + 4 == jr + LH ? jr : j0 + 4;
-      const uint32_t Ox = p ? s[oc + jx] : 0u;
-      const uint4 YP = ldv4(s + oc + (st.yp >> 1));
-      const uint4 ZP = kDim == 3 ? ldv4(s + oc + (st.zp >> 1)) : make_uint4(0, 0, 0, 0);
-      const uint4 JX = ldv4(Jg + co + j0), JY = ldv4(Jg + N + co + j0);
-      const uint4 JZ = kDim == 3 ? ldv4(Jg + 2 * N + co + j0) : make_uint4(0, 0, 0, 0);
-      const uint4 S1 = do_q ? ldv4(s1 + co + j0) : make_uint4(0, 0, 0, 0);
-      const uint32_t sv[4] = {S.x, S.y, S.z, S.w}, ov[4] = {O.x, O.y, O.z, O.w};
-      const uint32_t yv[4] = {YP.x, YP.y, YP.z, YP.w}, zv[4] = {ZP.x, ZP.y, ZP.z, ZP.w};
-      const uint32_t jxv[4] = {JX.x, JX.y, JX.z, JX.w}, jyv[4] = {JY.x, JY.y, JY.z, JY.w};
-      const uint32_t jzv[4] = {JZ.x, JZ.y, JZ.z, JZ.w}, s1v[4] = {S1.x, S1.y, S1.z, S1.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t xp = p ? (k < 3 ? ov[k + 1] : Ox) : ov[k];
-        const uint32_t u0 = sv[k] ^ xp ^ jxv[k], u1 = sv[k] ^ yv[k] ^ jyv[k];
-        const uint32_t u2 = kDim == 3 ? sv[k] ^ zv[k] ^ jzv[k] : 0u;
-        vc_add(CE, u0 ^ u1 ^ u2, 0);
-        vc_add(CE, (u0 & u1) | (u2 & (u0 ^ u1)), 1);
-        if (M) vc_add(CM, sv[k], 0);
-        if (do_q) vc_add(CQ, sv[k] ^ s1v[k], 0);
-      }
-    }
-  } else
-  // storage index k: colour c = k / half, colour index j = k % half
-  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
-    const int c = k >= half ? 1 : 0;
-    const uint32_t j = k - (uint32_t)c * half;
-    const CsSite st = kDim == 3 ? cs_site(j, c, L, g.fL) : cs_site2(j, c, L, g.fL);
-    const uint32_t oc = (uint32_t)(c ^ 1) * half;
-    const uint32_t S = s[k];
-    const uint32_t u0 = S ^ s[oc + (st.xp >> 1)] ^ Jg[k];
-    const uint32_t u1 = S ^ s[oc + (st.yp >> 1)] ^ Jg[N + k];
-    const uint32_t u2 = kDim == 3 ? S ^ s[oc + (st.zp >> 1)] ^ Jg[2 * N + k] : 0u;
-    vc_add(CE, u0 ^ u1 ^ u2, 0);
-    vc_add(CE, (u0 & u1) | (u2 & (u0 ^ u1)), 1);
-    if (M) vc_add(CM, S, 0);
-    if (do_q) vc_add(CQ, S ^ s1[k], 0);
-  }
-  const uint32_t lane = threadIdx.x & 31;
-  const int64_t lat = ((int64_t)a * T + t) * g.n_real + 32 * grp + lane;
-  // E = 2 unsat - kDim N, M = N - 2 down, Q = N - 2 diff: block 0 adds the constants
-  const long long n0 = blockIdx.x == 0 ? (long long)N : 0;
-  // one block per word-lattice stores its counts; several add them to
-  // outputs the host has zeroed
-  const bool direct = gridDim.x == 1;
-  auto put = [direct](long long *p, long long v) {
-    if (direct) *p = v;
-    else add_ll(p, v);
-  };
-  const long long unsat = vc_block_total(CE, sm);
-  if (threadIdx.x < 32 && E) put(&E[lat], 2 * unsat - kDim * n0);
-  if (M) {
-    const long long down = vc_block_total(CM, sm);
-    if (threadIdx.x < 32) put(&M[lat], n0 - 2 * down);
-  }
-  if (do_q) {
-    const long long diff = vc_block_total(CQ, sm);
-    if (threadIdx.x < 32) put(&Q[(int64_t)t * g.n_real + 32 * grp + lane], n0 - 2 * diff);
-  }
-}
-
-
-// The same counts when L % 8 == 0, counted with carry-save adders.  Each
-// word-lattice gets one block of kRowThreads threads (small blocks, so that
-// all of them are resident at once) or, for large lattices, several; a
-// thread takes at most kRowItems quads of four consecutive colour indices of
-// one row.  Per quad the four unsatisfied-bond sums (weight 1) and carries
-// (weight 2) of E, and the four words of M and of Q (weight 1), go through
-// carry-save adders into running planes of weight 1, 2, 4 (and 8 for E);
-// only what carries out of those is rippled into the counter.  Then one
-// butterfly per counter over the warp, and the warps of a word-lattice add
-// their counts through shared memory.
-constexpr int kRowThreads = 64;
+// from set 1, counted with carry-save adders.  Each word-lattice gets one
+// block (of 64 threads, so that all of them are resident at once, or of 256
+// where they are few) or, for large lattices, several; a thread takes at most
+// kRowItems groups of four sites: quads of four consecutive colour indices of
+// one row when L % 8 == 0, else four sites a block apart (so that the
+// loads of a warp are contiguous).  Per group the four unsatisfied-bond sums
+// (weight 1) and carries (weight 2) of E, and the four words of M and of Q
+// (weight 1), go through carry-save adders into running planes of weight 1,
+// 2, 4 (and 8 for E); only what carries out of those is rippled into the
+// counter.  Then one butterfly per counter over the warp, and the warps of a
+// word-lattice add their counts through shared memory.
+constexpr int kRowThreads = 64;        // many word-lattices: all their blocks resident at once
+constexpr int kRowThreadsFew = 256;    // few: more warps in flight
 constexpr int kRowItems = 16;
-constexpr int kRP = 8;   // per-thread planes: at most 16 quads x 4 sites x 3 bonds = 192 < 256
+constexpr int kRP = 8;   // per-thread planes: at most 16 groups x 4 sites x 3 bonds = 192 < 256
 constexpr int kRW = 13;  // per-warp planes: at most 32 x 192 = 6144 < 8192
 
 // Running count of weight-1 words: planes o1, o2, o4 and the counter above.
@@ -373,15 +233,15 @@ __device__ __forceinline__ int warp_count(const uint32_t (&C)[kRP]) {
 
 // grid: (blocks per word-lattice, word-lattices), kRowThreads threads; the
 // register bound lets 14 blocks share an SM.
-template <int kDim>
-__global__ void __launch_bounds__(kRowThreads, 14) measure_msc_rows_kernel(const uint32_t *__restrict__ w,
+template <int kDim, bool kQuads, int kThreads>
+__global__ void __launch_bounds__(kThreads, 896 / kThreads) measure_msc_rows_kernel(const uint32_t *__restrict__ w,
                                                                const uint32_t *__restrict__ J, Geom g,
                                                                long long *__restrict__ E,
                                                                long long *__restrict__ M,
                                                                long long *__restrict__ Q) {
   griddep_wait();
   griddep_release();
-  constexpr int kWarps = kRowThreads / 32;
+  constexpr int kWarps = kThreads / 32;
   __shared__ int cnt[3][kWarps][32];
   const uint32_t G = (uint32_t)g.n_real / 32, T = (uint32_t)g.n_temps;
   const uint32_t wl = blockIdx.y, lt = threadIdx.x;
@@ -393,8 +253,9 @@ __global__ void __launch_bounds__(kRowThreads, 14) measure_msc_rows_kernel(const
   const uint32_t *s1 = s + (size_t)G * T * N;  // set 1, same (g, t)
   CsaCount2 ce;
   CsaCount cm, cq;
-  for (uint32_t q = blockIdx.x * kRowThreads + lt; q < 2 * quads; q += gridDim.x * kRowThreads) {
-      const uint32_t c = q >= quads ? 1u : 0u;
+  if (kQuads) {
+  for (uint32_t q = blockIdx.x * kThreads + lt; q < 2 * quads; q += gridDim.x * kThreads) {
+    const uint32_t c = q >= quads ? 1u : 0u;
       const uint32_t j0 = 4 * (q - c * quads);
       const uint32_t co = c * half, oc = (c ^ 1u) * half;
       const CsSite st = kDim == 3 ? cs_site(j0, (int)c, L, g.fL) : cs_site2(j0, (int)c, L, g.fL);
@@ -428,6 +289,30 @@ __global__ void __launch_bounds__(kRowThreads, 14) measure_msc_rows_kernel(const
         cq.add4(S.x ^ S1.x, S.y ^ S1.y, S.z ^ S1.z, S.w ^ S1.w);
       }
     }
+  } else {
+    // storage index k: colour c = k / half, colour index j = k % half; the
+    // last group of a thread may be short
+    for (uint32_t k0 = blockIdx.x * 4 * kThreads + lt; k0 < N; k0 += gridDim.x * 4 * kThreads) {
+      uint32_t sum[4], car[4], S[4], D[4];
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) {
+        const uint32_t k = k0 + i * kThreads;
+        sum[i] = car[i] = S[i] = D[i] = 0u;
+        if (k >= N) continue;
+        const uint32_t c = k >= half ? 1u : 0u, oc = (c ^ 1u) * half;
+        const CsSite st = kDim == 3 ? cs_site(k - c * half, (int)c, L, g.fL) : cs_site2(k - c * half, (int)c, L, g.fL);
+        S[i] = s[k];
+        const uint32_t u0 = S[i] ^ s[oc + (st.xp >> 1)] ^ Jg[k], u1 = S[i] ^ s[oc + (st.yp >> 1)] ^ Jg[N + k];
+        const uint32_t u2 = kDim == 3 ? S[i] ^ s[oc + (st.zp >> 1)] ^ Jg[2 * N + k] : 0u;
+        sum[i] = u0 ^ u1 ^ u2;
+        car[i] = (u0 & u1) | (u2 & (u0 ^ u1));
+        if (do_q) D[i] = S[i] ^ s1[k];
+      }
+      ce.add(sum, car);
+      if (M) cm.add4(S[0], S[1], S[2], S[3]);
+      if (do_q) cq.add4(D[0], D[1], D[2], D[3]);
+    }
+  }
   ce.flush();
   cm.flush();
   cq.flush();
@@ -602,13 +487,13 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
     if (Q) cudaMemsetAsync(Q, 0, sizeof(int64_t) * g.n_temps * g.n_real, st);
     return launch_measure_msc2d(h, E, M);
   }
-  // EA coded words: blocks (or, with L % 8 == 0, parts of kRowThreads
-  // threads) per word-lattice, at most 16 sites (quads) per thread; with one
-  // per word-lattice the counts are stored, not added, and need no zeroing
-  const bool rows = h->d.layout == SPIN_MSC1 && g.L % 8 == 0;
-  const int64_t row_items = 2 * (g.N / 8);  // quads of both colours
-  const unsigned gx = rows ? (unsigned)((row_items + kRowThreads * kRowItems - 1) / (kRowThreads * kRowItems))
-                           : (unsigned)((g.N + 256 * 16 - 1) / (256 * 16));
+  // EA coded words: parts of kRowThreads (or kRowThreadsFew) threads per
+  // word-lattice, at most kRowItems groups of four sites per thread; with one
+  // part per word-lattice the counts are stored, not added, and need no zeroing
+  const int64_t n_wl = (int64_t)g.n_sets * (g.n_real / 32) * g.n_temps;
+  const bool few = n_wl < 152 * 10;
+  const int per_part = (few ? kRowThreadsFew : kRowThreads) * kRowItems;
+  const unsigned gx = (unsigned)((g.N / 4 + per_part - 1) / per_part);
   const bool coded_direct = h->d.layout == SPIN_MSC1 && gx == 1;
   if (!coded_direct) {
     if (E) cudaMemsetAsync(E, 0, sizeof(int64_t) * nl, st);
@@ -641,14 +526,15 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
                            dim3(256), 0, st, (const int8_t *)h->spins, g, (long long *)Q);
     return e;
   }
-  const int64_t n_wl = (int64_t)g.n_sets * (g.n_real / 32) * g.n_temps;
-  if (rows)
-    return launch_dependent(g.dim == 3 ? measure_msc_rows_kernel<3> : measure_msc_rows_kernel<2>,
-                            dim3(gx, (unsigned)n_wl), dim3(kRowThreads), 0, st,
-                            (const uint32_t *)h->spins, (const uint32_t *)J, g, (long long *)E, (long long *)M,
-                            (g.n_sets >= 2) ? (long long *)Q : nullptr);
-  return launch_dependent(g.dim == 3 ? measure_msc_kernel<3> : measure_msc_kernel<2>, dim3(gx, (unsigned)n_wl),
-                          dim3(256), 0, st, (const uint32_t *)h->spins,
+  const bool quads = g.L % 8 == 0;
+  using Kern = decltype(&measure_msc_rows_kernel<3, true, kRowThreads>);
+  const Kern kerns[2][2][2] = {
+      {{measure_msc_rows_kernel<2, false, kRowThreads>, measure_msc_rows_kernel<2, false, kRowThreadsFew>},
+       {measure_msc_rows_kernel<2, true, kRowThreads>, measure_msc_rows_kernel<2, true, kRowThreadsFew>}},
+      {{measure_msc_rows_kernel<3, false, kRowThreads>, measure_msc_rows_kernel<3, false, kRowThreadsFew>},
+       {measure_msc_rows_kernel<3, true, kRowThreads>, measure_msc_rows_kernel<3, true, kRowThreadsFew>}}};
+  const Kern kern = kerns[g.dim == 3][quads][few];
+  return launch_dependent(kern, dim3(gx, (unsigned)n_wl), dim3(few ? kRowThreadsFew : kRowThreads), 0, st, (const uint32_t *)h->spins,
                           (const uint32_t *)J, g, (long long *)E, (long long *)M,
                           (g.n_sets >= 2) ? (long long *)Q : nullptr);
 }

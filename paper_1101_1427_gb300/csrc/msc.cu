@@ -146,49 +146,71 @@ __global__ void __launch_bounds__(256)
   uint32_t *ws = w + (size_t)x.st * (uint32_t)g.n_temps * N;
   griddep_wait();
   const EaSiteJ c = ea_site_couplings<kDim>(J + (size_t)x.grp * kDim * N, e, colour, N);
+  // all slots' words first, so that their latencies overlap
+  EaSiteW v[kSlots];
+#pragma unroll
+  for (uint32_t s = 0; s < kSlots; ++s)
+    v[s] = ea_site_words<kDim>(ws + (size_t)min(x.t0 + s, x.t1 - 1) * N, e, colour, N);
 #pragma unroll
   for (uint32_t s = 0; s < kSlots; ++s) {
     const uint32_t t = x.t0 + s;
     if (t >= x.t1) break;
-    ea_site_update<kDim>(ws + (size_t)t * N, e, c, colour, N, r[s], __ldg(thr + 4 * t + 1), __ldg(thr + 4 * t + 2),
-                         kDim == 3 ? __ldg(thr + 4 * t + 3) : 0u);
+    const Flip f = ea_site_flip<kDim>(v[s], c, r[s], __ldg(thr + 4 * t + 1), __ldg(thr + 4 * t + 2),
+                                      kDim == 3 ? __ldg(thr + 4 * t + 3) : 0u);
+    ws[(size_t)t * N + (uint32_t)colour * (N / 2) + j] = v[s].S ^ f.F;
   }
 }
 
-// words -> one int8 per spin, [n_sets][n_temps][n_real][N]
-__global__ void unpack_msc_kernel(const uint32_t *__restrict__ w, int8_t *__restrict__ out, Geom g) {
+// Words <-> one int8 per spin, [n_sets][n_temps][n_real][N]: a thread takes
+// kSites consecutive sites of a word-lattice in all 32 realisations, the
+// kSites bytes of each in one access (256 x 30 x 2 x L = 12 to bytes: 17.4 us
+// with one site and single bytes).  kSites 4: N is a multiple of 4, the byte
+// buffer 4-byte aligned.
+template <int kSites>
+__device__ __forceinline__ int64_t first_lat(const Geom &g, int64_t wl) {
   const int G = g.n_real / 32;
-  const int64_t total = (int64_t)g.n_sets * G * g.n_temps * g.N;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t wl = k / g.N, i = k - wl * g.N;
-    const int t = (int)(wl % g.n_temps);
-    const int grp = (int)((wl / g.n_temps) % G);
-    const int a = (int)(wl / ((int64_t)g.n_temps * G));
-    const uint32_t v = w[wl * g.N + cs_word((uint32_t)i, colour_of(g, (uint32_t)i), (uint32_t)(g.N / 2))];
-    for (int b = 0; b < 32; ++b) {
-      const int64_t lat = ((int64_t)a * g.n_temps + t) * g.n_real + 32 * grp + b;
-      out[lat * g.N + i] = ((v >> b) & 1u) ? (int8_t)-1 : (int8_t)1;
-    }
+  const int64_t q = wl / g.n_temps;
+  const int t = (int)(wl - q * g.n_temps), a = (int)(q / G), grp = (int)(q - (int64_t)a * G);
+  return ((int64_t)a * g.n_temps + t) * g.n_real + 32 * grp;
+}
+
+template <int kSites, typename Bytes>
+__global__ void unpack_msc_kernel(const uint32_t *__restrict__ w, Bytes *__restrict__ out, Geom g, uint32_t total,
+                                  FastDiv fitems) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= total) return;
+  const uint32_t wl = fdiv(k, fitems), i = (k - wl * fitems.d) * kSites, N = (uint32_t)g.N;
+  uint32_t v[kSites];
+#pragma unroll
+  for (int s = 0; s < kSites; ++s) v[s] = w[(size_t)wl * N + cs_word(i + s, colour_of(g, i + s), N / 2)];
+  Bytes *o = out + (size_t)first_lat<kSites>(g, wl) * (N / kSites) + i / kSites;
+#pragma unroll 8
+  for (int b = 0; b < 32; ++b) {
+    uint32_t x = 0;
+#pragma unroll
+    for (int s = 0; s < kSites; ++s) x |= ((v[s] >> b & 1u) * 0xFEu | 1u) << (8 * s);  // 0x01 | 0xFE = -1
+    o[(size_t)b * (N / kSites)] = (Bytes)x;
   }
 }
 
-__global__ void pack_msc_kernel(const int8_t *__restrict__ in, uint32_t *__restrict__ w, Geom g) {
-  const int G = g.n_real / 32;
-  const int64_t total = (int64_t)g.n_sets * G * g.n_temps * g.N;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t wl = k / g.N, i = k - wl * g.N;
-    const int t = (int)(wl % g.n_temps);
-    const int grp = (int)((wl / g.n_temps) % G);
-    const int a = (int)(wl / ((int64_t)g.n_temps * G));
-    uint32_t v = 0;
-    for (int b = 0; b < 32; ++b) {
-      const int64_t lat = ((int64_t)a * g.n_temps + t) * g.n_real + 32 * grp + b;
-      v |= (in[lat * g.N + i] < 0 ? 1u : 0u) << b;
-    }
-    w[wl * g.N + cs_word((uint32_t)i, colour_of(g, (uint32_t)i), (uint32_t)(g.N / 2))] = v;
+template <int kSites, typename Bytes>
+__global__ void pack_msc_kernel(const Bytes *__restrict__ in, uint32_t *__restrict__ w, Geom g, uint32_t total,
+                                FastDiv fitems) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= total) return;
+  const uint32_t wl = fdiv(k, fitems), i = (k - wl * fitems.d) * kSites, N = (uint32_t)g.N;
+  const Bytes *p = in + (size_t)first_lat<kSites>(g, wl) * (N / kSites) + i / kSites;
+  uint32_t v[kSites];
+#pragma unroll
+  for (int s = 0; s < kSites; ++s) v[s] = 0u;
+#pragma unroll 8
+  for (int b = 0; b < 32; ++b) {
+    const uint32_t x = p[(size_t)b * (N / kSites)];
+#pragma unroll
+    for (int s = 0; s < kSites; ++s) v[s] |= (x >> (8 * s + 7) & 1u) << b;  // the sign
   }
+#pragma unroll
+  for (int s = 0; s < kSites; ++s) w[(size_t)wl * N + cs_word(i + s, colour_of(g, i + s), N / 2)] = v[s];
 }
 
 unsigned capped(int64_t n) {
@@ -254,16 +276,30 @@ cudaError_t launch_pack_msc2d(spin_lattice *h, const int8_t *in);   // msc2d.cu
 cudaError_t launch_unpack_msc(spin_lattice *h, int8_t *out) {
   if (h->d.model != SPIN_EA) return launch_unpack_msc2d(h, out);
   const Geom &g = h->g;
-  const int64_t words = (int64_t)g.n_sets * (g.n_real / 32) * g.n_temps * g.N;
-  unpack_msc_kernel<<<capped(words), 256, 0, h->stream>>>((const uint32_t *)h->spins, out, g);
+  const uint32_t sites = (g.N & 3) == 0 && ((uintptr_t)out & 3u) == 0 ? 4 : 1;
+  const uint32_t items = (uint32_t)(g.N / sites);
+  const uint32_t total = (uint32_t)((int64_t)g.n_sets * (g.n_real / 32) * g.n_temps) * items;  // < 2^27
+  if (sites == 4)
+    unpack_msc_kernel<4><<<grid_for(total, 256), 256, 0, h->stream>>>((const uint32_t *)h->spins, (uint32_t *)out, g,
+                                                                      total, make_fastdiv(items));
+  else
+    unpack_msc_kernel<1><<<grid_for(total, 256), 256, 0, h->stream>>>((const uint32_t *)h->spins, (uint8_t *)out, g,
+                                                                      total, make_fastdiv(items));
   return cudaGetLastError();
 }
 
 cudaError_t launch_pack_msc(spin_lattice *h, const int8_t *in) {
   if (h->d.model != SPIN_EA) return launch_pack_msc2d(h, in);
   const Geom &g = h->g;
-  const int64_t words = (int64_t)g.n_sets * (g.n_real / 32) * g.n_temps * g.N;
-  pack_msc_kernel<<<capped(words), 256, 0, h->stream>>>(in, (uint32_t *)h->spins, g);
+  const uint32_t sites = (g.N & 3) == 0 && ((uintptr_t)in & 3u) == 0 ? 4 : 1;
+  const uint32_t items = (uint32_t)(g.N / sites);
+  const uint32_t total = (uint32_t)((int64_t)g.n_sets * (g.n_real / 32) * g.n_temps) * items;  // < 2^27
+  if (sites == 4)
+    pack_msc_kernel<4><<<grid_for(total, 256), 256, 0, h->stream>>>((const uint32_t *)in, (uint32_t *)h->spins, g,
+                                                                    total, make_fastdiv(items));
+  else
+    pack_msc_kernel<1><<<grid_for(total, 256), 256, 0, h->stream>>>((const uint8_t *)in, (uint32_t *)h->spins, g, total,
+                                                                    make_fastdiv(items));
   return cudaGetLastError();
 }
 

@@ -39,3 +39,34 @@ def test_batched_sites_equal_per_handle_runs(L, n_real, T):
     for lat in lats:
         lat.sync()
         lat.close()
+
+
+@pytest.mark.parametrize("dim,L,n_real,T", [(2, 6, 32, 3), (2, 16, 64, 2), (2, 50, 32, 2), (2, 90, 32, 1), (3, 4, 32, 2),
+                                            (3, 8, 32, 2), (3, 12, 64, 3), (3, 18, 32, 2), (3, 26, 32, 1)])
+def test_counts_and_bytes_equal_bytes(dim, L, n_real, T):
+    """E, M and Q (one and several parts per word-lattice), and the conversion
+    from and to bytes at any address."""
+    coded = sp.Lattice(B.SPIN_EA, dim, L, B.SPIN_MSC1, n_real=n_real, n_temps=T, n_sets=2, seed=4)
+    i8 = sp.Lattice(B.SPIN_EA, dim, L, B.SPIN_I8, n_real=n_real, n_temps=T, n_sets=2, seed=4)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(L)
+    n = i8.spins.numel()
+    raw = 1 - 2 * (torch.rand(n + 4, device="cuda", generator=gen) < 0.3).to(torch.int8)
+    words = []
+    for off in (0, 1):
+        s = raw[off:off + n]
+        B.spin_pack_i8(coded.h, s)
+        B.spin_pack_i8(i8.h, s.clone())
+        for x, y in zip(coded.measure(), i8.measure()):
+            assert torch.equal(x, y)
+        words.append(coded.spins.clone())
+        for o in (0, 2):
+            out = torch.zeros(n + 4, dtype=torch.int8, device="cuda")
+            B.spin_unpack_i8(coded.h, out[o:o + n])
+            coded.sync()
+            assert torch.equal(out[o:o + n], s) and not out[:o].any() and not out[o + n:].any()
+    B.spin_pack_i8(coded.h, raw[1:1 + n].clone())
+    coded.sync()
+    assert torch.equal(coded.spins, words[1])
+    for lat in (coded, i8):
+        lat.close()
