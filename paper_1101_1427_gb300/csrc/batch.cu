@@ -76,6 +76,7 @@ struct BatchParams {
   int n_units;
   int measure_every, pt_every, extra;
   uint32_t staged_words;  // dynamic shared memory for couplings, in words
+  uint32_t smem_words;    // all of it; more than staged_words: EA words stay resident
   int64_t n_sweeps;
   uint64_t timeout_ns;
   RoundKeys keys[kMaxHandles];
@@ -86,8 +87,8 @@ static_assert(sizeof(BatchParams) <= 32764, "batch parameters exceed the kernel 
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
+constexpr int kPairThreads = 256;      // per CTA, two CTAs per SM
+constexpr int kResidentThreads = 512;  // one CTA per SM that keeps words in shared memory
 constexpr int kPl = 12;  // per-lane counter planes (counts < 4096)
 
 __device__ __forceinline__ uint32_t ld_acquire(const unsigned *p) {
@@ -111,16 +112,22 @@ struct Sync {
   int extra;  // arrivals that never come (fault injection for the timeout test)
 };
 
-// Returns false if the team (or the whole launch) has failed.
-__device__ bool team_barrier(Sync &sy) {
-  __shared__ int s_ok;
+// A team barrier in two halves: the arrival makes the CTA's writes before it
+// visible to every CTA whose wait returns true; work that touches none of the
+// team's data may come in between.  The wait returns false if the team (or the
+// whole launch) has failed.
+__device__ __forceinline__ void team_arrive(Sync &sy) {
   __syncthreads();
   sy.target += sy.size;
+  // release: the CTA's writes (ordered before this by the barrier above)
+  // become visible to every CTA that acquires the final count
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(sy.ctr) : "memory");
+}
+
+__device__ bool team_wait(const Sync &sy) {
+  __shared__ int s_ok;
   if (threadIdx.x == 0) {
     int ok = 1;
-    // release: the CTA's writes (ordered before this by the barrier above)
-    // become visible to every CTA that acquires the final count
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(sy.ctr) : "memory");
     const unsigned want = sy.target + (unsigned)sy.extra;
     const uint64_t t0 = globaltimer();
     while ((int)(ld_acquire(sy.ctr) - want) < 0) {
@@ -139,6 +146,11 @@ __device__ bool team_barrier(Sync &sy) {
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+__device__ __forceinline__ bool team_barrier(Sync &sy) {
+  team_arrive(sy);
+  return team_wait(sy);
 }
 
 // Harley-Seal counting of 1-bit planes: eight planes go through seven
@@ -297,12 +309,17 @@ __device__ __forceinline__ void count_words(HsCount &hc, const uint32_t *a, cons
   for (; i < N; i += stride) ripple_at<0>(hc.C, b ? (a[i] ^ b[i]) : a[i]);
 }
 
+// What a CTA of kThreads threads does for its unit.
+template <int kThreads>
+struct Cta {
+static constexpr int kWarps = kThreads / 32;
+
 // Per-bit counts of the set bits of n_items word arrays of N words each
 // (item k: a_k[i], or a_k[i] ^ b_k[i]), every item split over several warps
 // when there are fewer items than warps; cnt[k][b] receives item k's count
 // for bit b.  Called by the whole CTA.
 template <typename ItemFn>
-__device__ void cta_bit_counts(int n_items, uint32_t N, ItemFn item, int (*cnt)[32]) {
+static __device__ void cta_bit_counts(int n_items, uint32_t N, ItemFn item, int (*cnt)[32]) {
   __syncthreads();
   for (int k = threadIdx.x; k < n_items * 32; k += kThreads) (&cnt[0][0])[k] = 0;
   __syncthreads();
@@ -322,7 +339,7 @@ __device__ void cta_bit_counts(int n_items, uint32_t N, ItemFn item, int (*cnt)[
 
 // Bitwise exchange of the bits set in A between two word arrays of N words
 // (N a multiple of 4, 16-byte aligned), by the whole CTA.
-__device__ __forceinline__ void cta_swap_bits(uint32_t *w0, uint32_t *w1, uint32_t N, uint32_t A) {
+static __device__ __forceinline__ void cta_swap_bits(uint32_t *w0, uint32_t *w1, uint32_t N, uint32_t A) {
   uint4 *v0 = reinterpret_cast<uint4 *>(w0), *v1 = reinterpret_cast<uint4 *>(w1);
   const uint32_t n4 = N >> 2;
   uint32_t i = threadIdx.x;
@@ -348,23 +365,73 @@ struct NoCount {
 };
 
 // ---------------------------------------------------------------- EA unit
-__device__ bool ea_sweep(const BatchUnit &U, const uint32_t *Jsrc, int part, const RoundKeys &rk,
+// The word-lattices of a CTA, numbered g = t * n_sets + a: whole slots while
+// the team has at most n_T CTAs, single word-lattices beyond that.
+struct Owned {
+  int g0, g1;
+};
+
+static __device__ __forceinline__ Owned ea_owned(const BatchUnit &U, int part) {
+  const int P = U.team_size, W = U.n_T * U.n_sets;
+  Owned o;
+  o.g0 = P <= U.n_T ? (part * U.n_T / P) * U.n_sets : part * W / P;
+  o.g1 = P <= U.n_T ? ((part + 1) * U.n_T / P) * U.n_sets : (part + 1) * W / P;
+  return o;
+}
+
+// Owned word-lattices kept in shared memory for the whole launch: g = first ..
+// first + n - 1 at base + k N.  Word-lattices that another CTA writes or reads
+// are never among them: the owner of (a, t) exchanges it with (a, t + 1), so
+// those with g < g0 + n_sets may be written by the CTA before (part > 0); and
+// there are none when a team has more CTAs than slots, where the overlap reads
+// another CTA's words.
+struct Resident {
+  uint32_t *base;
+  int first, n;
+};
+
+static __device__ __forceinline__ Resident ea_resident(const BatchUnit &U, int part, uint32_t *base, uint32_t room) {
+  const Owned o = ea_owned(U, part);
+  Resident r;
+  r.base = base;
+  r.first = part > 0 ? min(o.g0 + U.n_sets, o.g1) : o.g0;
+  r.n = U.team_size <= U.n_T ? min(o.g1 - r.first, (int)(room / U.N)) : 0;
+  return r;
+}
+
+// Copies the resident word-lattices in (to_shared) or out, by the whole CTA.
+static __device__ __forceinline__ void ea_resident_copy(const BatchUnit &U, const Resident &R, bool to_shared) {
+  const uint32_t n4 = U.N / 4;
+  for (int k = 0; k < R.n; ++k) {
+    const int g = R.first + k, a = g % U.n_sets, t = g / U.n_sets;
+    uint4 *home = reinterpret_cast<uint4 *>(U.w + a * U.set_stride + (size_t)t * U.N);
+    uint4 *here = reinterpret_cast<uint4 *>(R.base + (size_t)k * U.N);
+    for (uint32_t i = threadIdx.x; i < n4; i += blockDim.x) {
+      if (to_shared) here[i] = home[i];
+      else home[i] = here[i];
+    }
+  }
+  __syncthreads();
+}
+
+static __device__ bool ea_sweep(const BatchUnit &U, const Resident &R, const uint32_t *Jsrc, int part, const RoundKeys &rk,
                          Sync &sy, uint32_t s_abs, bool measure, bool pt, long long meas_row,
                          uint32_t pt_step) {
   __shared__ int e_cnt[64][32];   // per owned word-lattice counts (energies, then M, then Q)
   __shared__ uint32_t masks[64];  // accept masks per owned word-lattice that starts a pair
-  // Owned word-lattices, numbered g = t * n_sets + a: whole slots while the
-  // team has at most n_T CTAs, single word-lattices beyond that.
-  const int P = U.team_size, W = U.n_T * U.n_sets;
-  const int g0 = P <= U.n_T ? (part * U.n_T / P) * U.n_sets : part * W / P;
-  const int g1 = P <= U.n_T ? ((part + 1) * U.n_T / P) * U.n_sets : (part + 1) * W / P;
+  const int P = U.team_size;
+  const Owned own = ea_owned(U, part);
+  const int g0 = own.g0, g1 = own.g1;
   const int n_w = g1 - g0;  // <= 64
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // warps per word-lattice when there are fewer word-lattices than warps
   const int wpw = n_w >= kWarps ? 1 : kWarps / n_w;
   const bool need_e = measure || pt;
   const uint32_t N = U.N;
-  auto words = [&](int a, int t) { return U.w + a * U.set_stride + (size_t)t * N; };
+  auto words = [&](int a, int t) -> uint32_t * {
+    const int k = t * U.n_sets + a - R.first;
+    return k >= 0 && k < R.n ? R.base + (size_t)k * N : U.w + a * U.set_stride + (size_t)t * N;
+  };
   for (int colour = 0; colour < 2; ++colour) {
     if (colour == 1 && need_e)
       for (int k = threadIdx.x; k < n_w * 32; k += kThreads) (&e_cnt[0][0])[k] = 0;
@@ -515,7 +582,7 @@ __device__ bool ea_sweep(const BatchUnit &U, const uint32_t *Jsrc, int part, con
 // One colour phase over the rows [r0, r1) of a 2D int8 lattice: four chunks
 // per thread and iteration, all their loads issued before any store.
 template <int kCount>
-__device__ void ising_rows_phase(const BatchUnit &U, const RoundKeys &rk, uint32_t sweep, int colour, int r0,
+static __device__ void ising_rows_phase(const BatchUnit &U, const RoundKeys &rk, uint32_t sweep, int colour, int r0,
                                  int r1, long long &anti, long long &down) {
   const int L = U.L;
   const uint32_t chunks = (uint32_t)L >> 3;
@@ -564,7 +631,7 @@ __device__ void ising_rows_phase(const BatchUnit &U, const RoundKeys &rk, uint32
 // One sweep of the team's rows.  Measurements come out of the phases: the
 // magnetisation from the sites each phase updated, the energy from the
 // updated sites of colour 1, since every bond has exactly one such end.
-__device__ bool ising_sweep(const BatchUnit &U, int part, const RoundKeys &rk, Sync &sy, uint32_t s_abs,
+static __device__ bool ising_sweep(const BatchUnit &U, int part, const RoundKeys &rk, Sync &sy, uint32_t s_abs,
                             bool measure, long long meas_row) {
   const int P = U.team_size;
   const int r0 = part * U.L / P, r1 = (part + 1) * U.L / P;
@@ -594,85 +661,104 @@ __device__ bool ising_sweep(const BatchUnit &U, int part, const RoundKeys &rk, S
 }
 
 // ---------------------------------------------------------------- coded Ising unit
-// One colour phase over the rows [r0, r1) of a 2D coded lattice, as the
-// per-phase kernel does it: each warp takes 32 consecutive blocks (128
-// same-colour sites each); lane l draws the Philox call 32 b + l of block b
-// and the warp's ballots of (r < thr4), (r < thr8) are the block's
-// acceptance masks; then lane b updates block b.
-template <int kCount>
-__device__ void msc2d_rows_phase(const BatchUnit &U, const RoundKeys &rk, uint32_t sweep, int colour, int r0,
-                                 int r1, uint4 (*mk)[32][2], long long &anti, long long &down) {
-  const int L = U.L, wpr = L / 64, bpr = L / 256;
-  const uint32_t thr4 = __ldg(U.thr + 4 * U.slot + 1), thr8 = __ldg(U.thr + 4 * U.slot + 2);
+// Acceptance masks of one block of 128 sites, drawn by one thread as in
+// msc2d_phase_kernel (msc2d.cu).
+struct Masks {
+  uint4 m4, m8;
+};
+
+static __device__ __forceinline__ Masks msc2d_draw(const BatchUnit &U, const RoundKeys &rk, uint32_t sweep, int colour,
+                                                   uint32_t gb, uint32_t thr4, uint32_t thr8) {
+  const PhiloxX0 pre = philox_x0_setup(sweep, U.lid, rk);
   const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t fb = (uint32_t)r0 * (uint32_t)bpr, nblk = (uint32_t)(r1 - r0) * (uint32_t)bpr;
-  for (uint32_t g0 = (uint32_t)warp * 32u; g0 < nblk; g0 += kWarps * 32u) {
-    const uint32_t cnt = nblk - g0 < 32u ? nblk - g0 : 32u;
-    uint32_t j4 = 32u * (fb + g0) + (uint32_t)lane;
+  const MaskBits b4(thr4), b8(thr8);
+  uint32_t A[4] = {0u, 0u, 0u, 0u}, E[4] = {0u, 0u, 0u, 0u};
 #pragma unroll 4
-    for (uint32_t b = 0; b < cnt; ++b, j4 += 32u) {
-      const uint4 r = philox(make_uint4(j4, sweep, U.lid, wctr), rk);
-      const uint32_t a0 = __ballot_sync(0xffffffffu, r.x < thr4);
-      const uint32_t a1 = __ballot_sync(0xffffffffu, r.y < thr4);
-      const uint32_t a2 = __ballot_sync(0xffffffffu, r.z < thr4);
-      const uint32_t a3 = __ballot_sync(0xffffffffu, r.w < thr4);
-      const uint32_t e0 = __ballot_sync(0xffffffffu, r.x < thr8);
-      const uint32_t e1 = __ballot_sync(0xffffffffu, r.y < thr8);
-      const uint32_t e2 = __ballot_sync(0xffffffffu, r.z < thr8);
-      const uint32_t e3 = __ballot_sync(0xffffffffu, r.w < thr8);
-      if (lane == 0) {
-        mk[warp][b][0] = make_uint4(a0, a1, a2, a3);
-        mk[warp][b][1] = make_uint4(e0, e1, e2, e3);
-      }
-    }
-    __syncwarp();
-    if ((uint32_t)lane < cnt) {
-      const uint32_t gb = fb + g0 + (uint32_t)lane;
-      const uint32_t y = gb / (uint32_t)bpr, B = gb - y * (uint32_t)bpr;
-      msc2d_block<kCount>(U.w, L, wpr, bpr, colour, (int)y, B, mk[warp][lane][0], mk[warp][lane][1], anti,
-                          down);
-    }
-    __syncwarp();
+  for (int i = 31; i >= 0; --i) {
+    const uint4 r = philox_x0(pre, philox_x0_shared(32u * gb + (uint32_t)i, wctr, rk), rk);
+    b4.push(A[0], r.x);
+    b4.push(A[1], r.y);
+    b4.push(A[2], r.z);
+    b4.push(A[3], r.w);
+    b8.push(E[0], r.x);
+    b8.push(E[1], r.y);
+    b8.push(E[2], r.z);
+    b8.push(E[3], r.w);
+  }
+  Masks m;
+  m.m4 = make_uint4(b4.mask(A[0]), b4.mask(A[1]), b4.mask(A[2]), b4.mask(A[3]));
+  m.m8 = make_uint4(b8.mask(E[0]), b8.mask(E[1]), b8.mask(E[2]), b8.mask(E[3]));
+  return m;
+}
+
+// One colour phase over the blocks [fb, fb + nblk) of a 2D coded lattice, one
+// thread per block; the masks of the thread's first block are there already.
+template <int kCount>
+static __device__ void msc2d_rows_phase(const BatchUnit &U, const RoundKeys &rk, uint32_t sweep, int colour,
+                                        uint32_t fb, uint32_t nblk, uint32_t thr4, uint32_t thr8, Masks m,
+                                        long long &anti, long long &down) {
+  const int L = U.L, wpr = L / 64, bpr = L / 256;
+  for (uint32_t k = threadIdx.x; k < nblk; k += kThreads) {
+    const uint32_t gb = fb + k;
+    if (k != threadIdx.x) m = msc2d_draw(U, rk, sweep, colour, gb, thr4, thr8);
+    const uint32_t y = gb / (uint32_t)bpr, B = gb - y * (uint32_t)bpr;
+    msc2d_block<kCount>(U.w, L, wpr, bpr, colour, (int)y, B, m.m4, m.m8, anti, down);
   }
 }
 
-// One sweep of the team's rows of a coded lattice, measurements fused as in
-// ising_sweep.
-__device__ bool msc2d_sweep(const BatchUnit &U, int part, const RoundKeys &rk, Sync &sy, uint32_t s_abs,
-                            bool measure, long long meas_row) {
-  const int P = U.team_size;
+// All sweeps of the team's rows of a coded lattice, measurements fused as in
+// ising_sweep.  Each thread draws the masks of its first block of the next
+// phase between the two halves of the team barrier, so that the barrier's
+// latency is covered by the generator.
+static __device__ void msc2d_run(const BatchUnit &U, int part, const RoundKeys &rk, Sync &sy, int64_t n_sweeps,
+                                 int measure_every) {
+  const int P = U.team_size, bpr = U.L / 256;
   const int r0 = part * U.L / P, r1 = (part + 1) * U.L / P;
-  const bool count = measure && (U.E_series || U.M_series);
-  __shared__ uint4 mk[kWarps][32][2];  // acceptance masks, per warp and block
-  long long anti = 0, down = 0;
-  for (int colour = 0; colour < 2; ++colour) {
-    if (!count) msc2d_rows_phase<0>(U, rk, s_abs, colour, r0, r1, mk, anti, down);
-    else if (colour == 0) msc2d_rows_phase<1>(U, rk, s_abs, 0, r0, r1, mk, anti, down);
-    else msc2d_rows_phase<2>(U, rk, s_abs, 1, r0, r1, mk, anti, down);
-    if (colour == 1 && count) {
-      anti = warp_sum(anti);
-      down = warp_sum(down);
-      if ((threadIdx.x & 31) == 0) {
-        const long long N = (long long)U.N;
-        const long long idx = meas_row * U.n_lat + U.lat_index;
-        const bool first = part == 0 && threadIdx.x == 0;
-        if (U.E_series)
-          atomicAdd((unsigned long long *)&U.E_series[idx], (unsigned long long)(2 * anti - (first ? 2 * N : 0)));
-        if (U.M_series)
-          atomicAdd((unsigned long long *)&U.M_series[idx], (unsigned long long)(-2 * down + (first ? N : 0)));
+  const uint32_t fb = (uint32_t)r0 * (uint32_t)bpr, nblk = (uint32_t)(r1 - r0) * (uint32_t)bpr;
+  const uint32_t thr4 = __ldg(U.thr + 4 * U.slot + 1), thr8 = __ldg(U.thr + 4 * U.slot + 2);
+  long long meas_row = 0;
+  Masks m = {};
+  if (threadIdx.x < nblk) m = msc2d_draw(U, rk, U.sweep0, 0, fb + threadIdx.x, thr4, thr8);
+  for (int64_t k = 0; k < n_sweeps; ++k) {
+    const uint32_t s_abs = U.sweep0 + (uint32_t)k;
+    const bool measure = measure_every > 0 && ((s_abs + 1u) % (uint32_t)measure_every) == 0u;
+    const bool count = measure && (U.E_series || U.M_series);
+    long long anti = 0, down = 0;
+    for (int colour = 0; colour < 2; ++colour) {
+      if (!count) msc2d_rows_phase<0>(U, rk, s_abs, colour, fb, nblk, thr4, thr8, m, anti, down);
+      else if (colour == 0) msc2d_rows_phase<1>(U, rk, s_abs, 0, fb, nblk, thr4, thr8, m, anti, down);
+      else msc2d_rows_phase<2>(U, rk, s_abs, 1, fb, nblk, thr4, thr8, m, anti, down);
+      if (colour == 1 && count) {
+        anti = warp_sum(anti);
+        down = warp_sum(down);
+        if ((threadIdx.x & 31) == 0) {
+          const long long N = (long long)U.N;
+          const long long idx = meas_row * U.n_lat + U.lat_index;
+          const bool first = part == 0 && threadIdx.x == 0;
+          if (U.E_series)
+            atomicAdd((unsigned long long *)&U.E_series[idx], (unsigned long long)(2 * anti - (first ? 2 * N : 0)));
+          if (U.M_series)
+            atomicAdd((unsigned long long *)&U.M_series[idx], (unsigned long long)(-2 * down + (first ? N : 0)));
+        }
       }
+      if (colour == 1 && k + 1 == n_sweeps) break;
+      team_arrive(sy);
+      if (threadIdx.x < nblk)
+        m = msc2d_draw(U, rk, s_abs + (uint32_t)colour, colour ^ 1, fb + threadIdx.x, thr4, thr8);
+      if (!team_wait(sy)) return;
     }
-    if (!team_barrier(sy)) return false;
+    if (measure) ++meas_row;
   }
-  return true;
 }
+};
 
-__global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constant__ BatchParams prm,
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 512 / kThreads) batch_kernel(const __grid_constant__ BatchParams prm,
                                                          int *err) {
+  using C = Cta<kThreads>;
   __shared__ BatchUnit U;
   __shared__ RoundKeys rk;
-  extern __shared__ __align__(16) uint32_t sJ[];  // couplings of an EA unit, when staged
+  extern __shared__ __align__(16) uint32_t sJ[];  // an EA unit's couplings, when staged, then its resident words
   // CTA -> unit: teams are consecutive CTA ranges in unit order
   int lo = 0, hi = prm.n_units - 1;
   while (lo < hi) {
@@ -694,11 +780,22 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
   Sync sy{U.bar, 0u, U.team_size, err, prm.timeout_ns, prm.extra};
   // the couplings never change during a launch: stage them once if they fit
   const uint32_t *Jsrc = U.J;
+  typename C::Resident R = {sJ, 0, 0};
+  uint32_t used = 0;
   if (U.kind == 0 && 3u * U.N <= prm.staged_words) {
     for (uint32_t k = threadIdx.x; k < 3u * U.N / 4u; k += blockDim.x)
       reinterpret_cast<uint4 *>(sJ)[k] = __ldg(reinterpret_cast<const uint4 *>(U.J) + k);
     __syncthreads();
     Jsrc = sJ;
+    used = 3u * U.N;
+  }
+  if (U.kind == 0 && prm.smem_words > prm.staged_words) {
+    R = C::ea_resident(U, part, sJ + used, prm.smem_words - used);
+    C::ea_resident_copy(U, R, true);
+  }
+  if (U.kind == 2) {
+    C::msc2d_run(U, part, rk, sy, prm.n_sweeps, prm.measure_every);
+    return;
   }
   long long meas_row = 0;
   uint32_t pt_step = U.pt0;
@@ -706,16 +803,15 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
     const uint32_t s_abs = U.sweep0 + (uint32_t)k;
     const bool measure = prm.measure_every > 0 && ((s_abs + 1u) % (uint32_t)prm.measure_every) == 0u;
     const bool pt = prm.pt_every > 0 && ((s_abs + 1u) % (uint32_t)prm.pt_every) == 0u;
-    bool ok;
-    if (U.kind == 0)
-      ok = ea_sweep(U, Jsrc, part, rk, sy, s_abs, measure, pt, meas_row, pt_step);
-    else if (U.kind == 1)
-      ok = ising_sweep(U, part, rk, sy, s_abs, measure, meas_row);
-    else
-      ok = msc2d_sweep(U, part, rk, sy, s_abs, measure, meas_row);
-    if (!ok) return;
+    const bool ok = U.kind == 0 ? C::ea_sweep(U, R, Jsrc, part, rk, sy, s_abs, measure, pt, meas_row, pt_step)
+                                : C::ising_sweep(U, part, rk, sy, s_abs, measure, meas_row);
+    if (!ok) break;  // (the resident words go home all the same)
     if (measure) ++meas_row;
     if (pt) ++pt_step;
+  }
+  if (R.n > 0) {
+    __syncthreads();
+    C::ea_resident_copy(U, R, false);
   }
 }
 
@@ -762,24 +858,44 @@ struct Tuned {
 };
 static std::map<std::vector<long long>, Tuned> g_tuned;  // autotuner cache, by batch signature
 
-// Relative cost of one sweep of a unit, per CTA-time, with measurement and
-// exchange every sweep (calibrated on GB300: a coded EA word-site costs ~4x
-// an int8 Ising site and ~8x a coded Ising site); the autotuner rescales
-// the Ising share and adds ea_n0 sites of fixed cost per EA word-lattice
-// (barriers and set-up weigh more, per site, in small lattices).
-static double unit_work(const BatchUnit &U, double ising_scale, double ea_n0) {
-  if (U.kind == 0) return 48.0 * U.n_sets * U.n_T * ((double)U.N + ea_n0);
-  if (U.kind == 1) return 12.0 * ising_scale * (double)U.N;
-  return 6.0 * ising_scale * (double)U.N;
+// Time of one sweep of a unit with a team of P CTAs, with measurement and
+// exchange every sweep, in ns (calibrated on GB300 with two CTAs per SM: EA
+// units of L = 16, 24, 32 with one word-lattice per CTA take 21, 42, 55 us, L =
+// 8 with four 15 us, so about 12 us of barriers and reductions and 2.16 ns per
+// word-site; a CTA sweeps 4.9 coded Ising sites per ns).  What counts is the
+// CTA with the most word-lattices or rows: a team of 9 for 32 slots is no
+// faster than one of 8.  The autotuner rescales the Ising share and adds
+// ea_n0 sites per EA word-lattice.
+static double unit_time(const BatchUnit &U, int P, double ising_scale, double ea_n0) {
+  if (U.kind == 0) {
+    const int W = U.n_T * U.n_sets;
+    const int owned = P <= U.n_T ? (U.n_T + P - 1) / P * U.n_sets : (W + P - 1) / P;
+    return 12000.0 + 2.16 * owned * ((double)U.N + ea_n0);
+  }
+  const double rows = (U.L + P - 1) / P;
+  return 4000.0 + (U.kind == 1 ? 0.45 : 0.205) * ising_scale * rows * U.L;
+}
+
+// The next larger team for which the unit's time falls (cap + 1: none).
+static int next_team(const BatchUnit &U, int P, int cap) {
+  if (U.kind != 0) return P + 1;
+  const int W = U.n_T * U.n_sets;
+  if (P < U.n_T) {
+    const int m = (U.n_T + P - 1) / P;  // slots of the largest share, more than one
+    return (U.n_T + m - 2) / (m - 1);
+  }
+  const int o = (W + P - 1) / P;
+  return o > 1 ? (W + o - 2) / (o - 1) : cap + 1;
 }
 
 // Distributes `grid` CTAs over the units: every unit gets its minimum (EA:
-// at most 64 owned word-lattices per CTA; Ising: 1), then CTAs go one by
-// one to the unit with the largest work per CTA, up to each unit's maximum
-// (EA: one word-lattice per CTA; Ising: 8 rows per CTA).  Returns the CTAs
-// used.
+// at most 64 owned word-lattices per CTA; Ising: 1), then the unit with the
+// longest time gets its next larger team, as long as one fits, up to each
+// unit's maximum (EA: one word-lattice per CTA; Ising: 8 rows, or 256 coded
+// blocks, per CTA).  Returns the CTAs used.
 static int assign_teams(BatchUnit *units, int n, int grid, double ising_scale, double ea_n0) {
   std::vector<int> P(n), cap(n);
+  std::vector<double> time(n);
   int used = 0;
   for (int u = 0; u < n; ++u) {
     if (units[u].kind == 0) {
@@ -796,18 +912,21 @@ static int assign_teams(BatchUnit *units, int n, int grid, double ising_scale, d
       cap[u] = std::max(1, units[u].L * (units[u].L / 256) / 256);
     }
     used += P[u];
+    time[u] = unit_time(units[u], P[u], ising_scale, ea_n0);
   }
-  while (used < grid) {
+  for (;;) {
     int best = -1;
-    double bw = -1;
     for (int u = 0; u < n; ++u)
-      if (P[u] < cap[u] && unit_work(units[u], ising_scale, ea_n0) / P[u] > bw) {
-        bw = unit_work(units[u], ising_scale, ea_n0) / P[u];
-        best = u;
-      }
+      if (time[u] >= 0.0 && (best < 0 || time[u] > time[best])) best = u;
     if (best < 0) break;
-    ++P[best];
-    ++used;
+    const int next = next_team(units[best], P[best], cap[best]);
+    if (next > cap[best] || used + next - P[best] > grid) {
+      time[best] = -1.0;  // stays as it is
+      continue;
+    }
+    used += next - P[best];
+    P[best] = next;
+    time[best] = unit_time(units[best], next, ising_scale, ea_n0);
   }
   int first = 0;
   for (int u = 0; u < n; ++u) {
@@ -963,18 +1082,54 @@ static bool batch_item_ok(const spin_batch_item &it, int32_t pt_every) {
   return false;
 }
 
+// Dynamic shared memory of a CTA that has its SM to itself, beside ~26 KB of
+// counters and masks.
+constexpr int kResidentSmem = 196 * 1024;
+
+// One 512-thread CTA per SM with word-lattices in shared memory, against two
+// of 256 threads that read them from L2: the update is bound by the latency of
+// those loads at 16 warps per SM.  For batches of EA units alone whose
+// word-lattices are small enough that most of a CTA's fit (32 KB at L = 20),
+// and whose units are large enough for three CTAs and more each (a unit takes
+// whole CTAs) but have no more CTAs than slots.  1024 x 32 x 2 of L = 16, 8
+// sweeps with E, M, Q and an exchange after each: 523 -> 485 us.
+static bool resident_preferred(const BatchParams &prm, int sms) {
+  double total = 0.0;
+  for (int u = 0; u < prm.n_units; ++u) {
+    const BatchUnit &U = prm.units[u];
+    if (U.kind != 0 || U.N > 8192u) return false;
+    total += (double)U.n_sets * U.n_T * U.N;
+  }
+  for (int u = 0; u < prm.n_units; ++u) {
+    const BatchUnit &U = prm.units[u];
+    const double share = sms * (double)U.n_sets * U.n_T * U.N / total;
+    if (share < 3.0 || share > (double)U.n_T) return false;
+  }
+  return true;
+}
+
+static bool resident(const BatchParams &prm) { return prm.smem_words > prm.staged_words; }
+
 static cudaError_t batch_launch(BatchParams &prm, int grid, cudaStream_t st, int *err) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = (size_t)prm.staged_words * 4;
+  cfg.blockDim = dim3(resident(prm) ? kResidentThreads : kPairThreads);
+  cfg.dynamicSmemBytes = (size_t)prm.smem_words * 4;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, batch_kernel, prm, err);
+  return resident(prm) ? cudaLaunchKernelEx(&cfg, batch_kernel<kResidentThreads>, prm, err)
+                       : cudaLaunchKernelEx(&cfg, batch_kernel<kPairThreads>, prm, err);
+}
+
+static cudaError_t batch_occupancy(const BatchParams &prm, int *per_sm) {
+  const size_t smem = (size_t)prm.smem_words * 4;
+  return resident(prm)
+             ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, batch_kernel<kResidentThreads>, kResidentThreads, smem)
+             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, batch_kernel<kPairThreads>, kPairThreads, smem);
 }
 
 // The launch parameters are built in function-static buffers and the tuning
@@ -1018,8 +1173,10 @@ extern "C" int spin_batch_run(const spin_batch_item *items, int n_items, int64_t
   }
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 12288 * 4) !=
-        cudaSuccess)
+    if (cudaFuncSetAttribute(batch_kernel<kResidentThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kResidentSmem) != cudaSuccess ||
+        cudaFuncSetAttribute(batch_kernel<kPairThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, 12288 * 4) !=
+            cudaSuccess)
       return SPIN_ECUDA;
     attr = true;
   }
@@ -1051,14 +1208,23 @@ extern "C" int spin_batch_run(const spin_batch_item *items, int n_items, int64_t
   for (int u = 0; u < prm.n_units; ++u)
     if (prm.units[u].kind == 0 && 3u * prm.units[u].N <= 12288u)
       prm.staged_words = std::max(prm.staged_words, 3u * prm.units[u].N);
+  // CTAs per SM: autotuned once per batch signature (see spin_batch_tune)
+  std::vector<long long> sig;
+  for (int u = 0; u < prm.n_units; ++u) {
+    sig.push_back(prm.units[u].kind);
+    sig.push_back(prm.units[u].L);
+    sig.push_back(prm.units[u].n_T);
+    sig.push_back(prm.units[u].n_sets);
+  }
+  const auto it = g_tuned.find(sig);
+  const int asked = h0->batch_ctas_per_sm > 0 ? h0->batch_ctas_per_sm : it != g_tuned.end() ? it->second.ctas_per_sm : 0;
   // co-resident grid
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kThreads,
-                                                    (size_t)prm.staged_words * 4) != cudaSuccess ||
-      per_sm < 1)
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return SPIN_ECUDA;
+  prm.smem_words = asked <= 1 && resident_preferred(prm, sms) ? kResidentSmem / 4 : prm.staged_words;
+  if (batch_occupancy(prm, &per_sm) != cudaSuccess || per_sm < 1) return SPIN_ECUDA;
   // Ising series rows are accumulated with atomics: zero the rows of this call
   for (int k = 0; k < n_items; ++k) {
     spin_lattice *h = items[k].lat;
@@ -1069,18 +1235,9 @@ extern "C" int spin_batch_run(const spin_batch_item *items, int n_items, int64_t
     if (items[k].M_series && cudaMemsetAsync(items[k].M_series, 0, 8 * n_meas * h->n_lat, st) != cudaSuccess)
       return SPIN_ECUDA;
   }
-  // CTAs per SM: autotuned once per batch signature (see spin_batch_tune)
-  std::vector<long long> sig;
-  for (int u = 0; u < prm.n_units; ++u) {
-    sig.push_back(prm.units[u].kind);
-    sig.push_back(prm.units[u].L);
-    sig.push_back(prm.units[u].n_T);
-    sig.push_back(prm.units[u].n_sets);
-  }
-  int bps = std::min(per_sm, h0->batch_ctas_per_sm > 0 ? h0->batch_ctas_per_sm : 2);
+  int bps = std::min(per_sm, h0->batch_ctas_per_sm > 0 ? h0->batch_ctas_per_sm : 2);  // (1 where words are resident)
   double scale = h0->batch_ising_scale > 0.0 ? h0->batch_ising_scale : 1.0;
   double n0 = h0->batch_ea_n0 > 0.0 ? h0->batch_ea_n0 - 1.0 : 0.0;
-  auto it = g_tuned.find(sig);
   if (it != g_tuned.end()) {
     if (h0->batch_ctas_per_sm <= 0) bps = std::min(per_sm, it->second.ctas_per_sm);
     if (h0->batch_ising_scale <= 0.0) scale = it->second.ising_scale;
@@ -1116,7 +1273,8 @@ extern "C" int spin_batch_tune(const spin_batch_item *items, int n_items, int64_
   if (!items || n_items <= 0 || n_items > kMaxHandles) return SPIN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream_v;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kThreads, 0) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<kPairThreads>, kPairThreads, 0) !=
+      cudaSuccess)
     return SPIN_ECUDA;
   // back up the spins and counters; series outputs are not written
   std::vector<spin_batch_item> tmp(items, items + n_items);
