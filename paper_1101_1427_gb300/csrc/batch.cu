@@ -262,8 +262,23 @@ struct AddTo {
   }
 };
 
-// One colour phase of one word-lattice (colour-split) by `stride` threads,
-// quads first, first + stride, ...  With kCount the post-update number of
+// The counting passes of a CTA go over the chunks (128 sites: 32 quads, one per
+// lane) of all its word-lattices in turn, an equal share of them per warp, so
+// that ten word-lattices take eight warps 1.25 times and not twice as long as
+// eight; a warp sums up its part of each word-lattice that it touches.
+struct Share {
+  uint32_t c, end;  // chunks of all word-lattices
+};
+
+__device__ __forceinline__ Share warp_share(uint32_t chunks, uint32_t warp, uint32_t warps) {
+  Share s;
+  s.c = chunks * warp / warps;
+  s.end = chunks * (warp + 1) / warps;
+  return s;
+}
+
+// One colour phase of the chunks [c0, c1) of one word-lattice (colour-split)
+// by a warp.  With kCount the post-update number of
 // unsatisfied bonds of each updated (colour-1) site is added to C: every
 // bond joins a colour-0 and a colour-1 site, so summing over colour-1 sites
 // counts each bond once.
@@ -271,12 +286,11 @@ template <bool kCount>
 __device__ __forceinline__ void ea_phase_warp(uint32_t *__restrict__ s, const uint32_t *__restrict__ Jg,
                                               const BatchUnit &U, const RoundKeys &rk, uint32_t sweep,
                                               uint32_t lid, int colour, uint32_t t4, uint32_t t8,
-                                              uint32_t t12, uint32_t first, uint32_t stride,
-                                              uint32_t (&C)[kPl]) {
+                                              uint32_t t12, uint32_t c0, uint32_t c1, uint32_t (&C)[kPl]) {
   uint32_t buf[4][3];
   int n = 0;
   if ((U.L & 7) != 0) {  // whole warps: lanes take consecutive sites
-    ea_sites_phase(s, Jg, colour, (uint32_t)U.L, U.N, U.fL, rk, sweep, lid, t4, t8, t12, first >> 5, stride >> 5,
+    ea_sites_phase(s, Jg, colour, (uint32_t)U.L, U.N, U.fL, rk, sweep, lid, t4, t8, t12, c0, c1,
                    [&](const Flip &f, bool on) {
                      if (!kCount) return;
                      uint32_t a0 = 0, a1 = 0, a2 = 0;
@@ -287,7 +301,8 @@ __device__ __forceinline__ void ea_phase_warp(uint32_t *__restrict__ s, const ui
   }
   const uint32_t quads = U.N / 8;
   const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
-  for (uint32_t j4 = first; j4 < quads; j4 += stride) {
+  const uint32_t end = min(32u * c1, quads);
+  for (uint32_t j4 = 32u * c0 + (threadIdx.x & 31u); j4 < end; j4 += 32u) {
     const uint4 r = philox(make_uint4(j4, sweep, lid, wctr), rk);
     const EaQuadGeom q = ea_quad_geom<3>(j4, colour, (uint32_t)U.L, U.fL);
     ea_quad_update<3, kCount>(s, q, ea_quad_couplings<3>(Jg, q, colour, U.N), colour, U.N, r, t4, t8, t12,
@@ -295,18 +310,18 @@ __device__ __forceinline__ void ea_phase_warp(uint32_t *__restrict__ s, const ui
   }
 }
 
-// Counts per bit the words a[i] (or a[i] ^ b[i]) for i = lane, lane + 32, ...
-__device__ __forceinline__ void count_words(HsCount &hc, const uint32_t *a, const uint32_t *b, uint32_t N,
-                                            uint32_t first, uint32_t stride) {
-  uint32_t i = first;
-  for (; i + 7 * stride < N; i += 8 * stride) {
+// Counts per bit the words a[i] (or a[i] ^ b[i]) of i in [i0, i1), by a warp.
+__device__ __forceinline__ void count_words(HsCount &hc, const uint32_t *a, const uint32_t *b, uint32_t i0,
+                                            uint32_t i1) {
+  uint32_t i = i0 + (threadIdx.x & 31u);
+  for (; i + 7 * 32 < i1; i += 8 * 32) {
     uint32_t x[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) x[k] = b ? (a[i + stride * k] ^ b[i + stride * k]) : a[i + stride * k];
+    for (int k = 0; k < 8; ++k) x[k] = b ? (a[i + 32 * k] ^ b[i + 32 * k]) : a[i + 32 * k];
     hc.add8(x);
   }
   hc.flush();
-  for (; i < N; i += stride) ripple_at<0>(hc.C, b ? (a[i] ^ b[i]) : a[i]);
+  for (; i < i1; i += 32) ripple_at<0>(hc.C, b ? (a[i] ^ b[i]) : a[i]);
 }
 
 // What a CTA of kThreads threads does for its unit.
@@ -315,24 +330,24 @@ struct Cta {
 static constexpr int kWarps = kThreads / 32;
 
 // Per-bit counts of the set bits of n_items word arrays of N words each
-// (item k: a_k[i], or a_k[i] ^ b_k[i]), every item split over several warps
-// when there are fewer items than warps; cnt[k][b] receives item k's count
-// for bit b.  Called by the whole CTA.
+// (item k: a_k[i], or a_k[i] ^ b_k[i]), shared out among the warps in chunks
+// of 256 words; cnt[k][b] receives item k's count for bit b.  Called by the
+// whole CTA.
 template <typename ItemFn>
 static __device__ void cta_bit_counts(int n_items, uint32_t N, ItemFn item, int (*cnt)[32]) {
   __syncthreads();
   for (int k = threadIdx.x; k < n_items * 32; k += kThreads) (&cnt[0][0])[k] = 0;
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wpi = n_items >= kWarps ? 1 : kWarps / n_items;
-  for (int k = warp / wpi; k < n_items; k += kWarps / wpi) {
+  const uint32_t per = (N + 255) / 256, lane = threadIdx.x & 31u;
+  Share sh = warp_share(per * (uint32_t)n_items, threadIdx.x >> 5, kWarps);
+  while (sh.c < sh.end) {
+    const uint32_t k = sh.c / per, c0 = sh.c - k * per, c1 = min(per, c0 + (sh.end - sh.c));
     const uint32_t *a = nullptr, *b = nullptr;
-    item(k, a, b);
+    item((int)k, a, b);
     HsCount hc;
-    count_words(hc, a, b, N, (uint32_t)((warp % wpi) * 32 + lane), (uint32_t)(wpi * 32));
-    const int c = warp_bit_counts(hc.C);
-    if (wpi == 1) cnt[k][lane] = c;
-    else atomicAdd(&cnt[k][lane], c);
+    count_words(hc, a, b, 256 * c0, min(256 * c1, N));
+    atomicAdd(&cnt[k][lane], warp_bit_counts(hc.C));
+    sh.c += c1 - c0;
   }
   __syncthreads();
 }
@@ -424,8 +439,8 @@ static __device__ bool ea_sweep(const BatchUnit &U, const Resident &R, const uin
   const int g0 = own.g0, g1 = own.g1;
   const int n_w = g1 - g0;  // <= 64
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // warps per word-lattice when there are fewer word-lattices than warps
-  const int wpw = n_w >= kWarps ? 1 : kWarps / n_w;
+  // chunks of one colour of a word-lattice
+  const uint32_t per = ((U.N / 2 + 3) / 4 + 31) / 32;
   const bool need_e = measure || pt;
   const uint32_t N = U.N;
   auto words = [&](int a, int t) -> uint32_t * {
@@ -459,22 +474,23 @@ static __device__ bool ea_sweep(const BatchUnit &U, const Resident &R, const uin
       __syncthreads();
       continue;
     }
-    for (int wi = warp / wpw; wi < n_w; wi += kWarps / wpw) {
+    Share sh = warp_share(per * (uint32_t)n_w, (uint32_t)warp, kWarps);
+    while (sh.c < sh.end) {
+      const int wi = (int)(sh.c / per);
+      const uint32_t c0 = sh.c - (uint32_t)wi * per, c1 = min(per, c0 + (sh.end - sh.c));
+      sh.c += c1 - c0;
       const int g = g0 + wi, a = g % U.n_sets, t = g / U.n_sets;
       uint32_t *s = words(a, t);
       const uint32_t lid = lattice_id((uint32_t)a, (uint32_t)U.rgrp, (uint32_t)t);
       const uint32_t t4 = __ldg(U.thr + 4 * t + 1), t8 = __ldg(U.thr + 4 * t + 2), t12 = __ldg(U.thr + 4 * t + 3);
-      const uint32_t first = (uint32_t)((warp % wpw) * 32 + lane), stride = (uint32_t)(wpw * 32);
       uint32_t C[kPl];
 #pragma unroll
       for (int k = 0; k < kPl; ++k) C[k] = 0;
       if (colour == 1 && need_e) {
-        ea_phase_warp<true>(s, Jsrc, U, rk, s_abs, lid, 1, t4, t8, t12, first, stride, C);
-        const int cnt = warp_bit_counts(C);
-        if (wpw == 1) e_cnt[wi][lane] = cnt;
-        else atomicAdd(&e_cnt[wi][lane], cnt);
+        ea_phase_warp<true>(s, Jsrc, U, rk, s_abs, lid, 1, t4, t8, t12, c0, c1, C);
+        atomicAdd(&e_cnt[wi][lane], warp_bit_counts(C));
       } else {
-        ea_phase_warp<false>(s, Jsrc, U, rk, s_abs, lid, colour, t4, t8, t12, first, stride, C);
+        ea_phase_warp<false>(s, Jsrc, U, rk, s_abs, lid, colour, t4, t8, t12, c0, c1, C);
       }
     }
     __syncthreads();
@@ -858,22 +874,26 @@ struct Tuned {
 };
 static std::map<std::vector<long long>, Tuned> g_tuned;  // autotuner cache, by batch signature
 
+static constexpr double kEaFixedUs = 13.0, kLatticeUs = 0.45, kQuadUs = 1.0e-3, kSiteUs = 2.0e-3, kUnstaged = 1.6;
+
 // Time of one sweep of a unit with a team of P CTAs, with measurement and
-// exchange every sweep, in ns (calibrated on GB300 with two CTAs per SM: EA
-// units of L = 16, 24, 32 with one word-lattice per CTA take 21, 42, 55 us, L =
-// 8 with four 15 us, so about 12 us of barriers and reductions and 2.16 ns per
-// word-site; a CTA sweeps 4.9 coded Ising sites per ns).  What counts is the
-// CTA with the most word-lattices or rows: a team of 9 for 32 slots is no
-// faster than one of 8.  The autotuner rescales the Ising share and adds
-// ea_n0 sites per EA word-lattice.
+// exchange every sweep, in us (fitted to the times at which the units of the
+// uneven batch end, two CTAs per SM): for EA units a fixed part (barriers,
+// reductions) and, for the CTA with the most word-lattices n of N sites, a part
+// per word-site, larger where the quads of a row do not fit (L % 8 != 0) or the
+// couplings are not staged; 6.2 coded Ising sites per ns and CTA.  What counts
+// is the largest share: a team of 9 for 32 slots is no faster than one of 8.
+// The autotuner rescales the Ising share and adds ea_n0 sites per EA
+// word-lattice.
 static double unit_time(const BatchUnit &U, int P, double ising_scale, double ea_n0) {
   if (U.kind == 0) {
     const int W = U.n_T * U.n_sets;
     const int owned = P <= U.n_T ? (U.n_T + P - 1) / P * U.n_sets : (W + P - 1) / P;
-    return 12000.0 + 2.16 * owned * ((double)U.N + ea_n0);
+    const double per_site = (U.L % 8 != 0 ? kSiteUs : kQuadUs) * (3u * U.N > 12288u ? kUnstaged : 1.0);
+    return kEaFixedUs + owned * (kLatticeUs + per_site * ((double)U.N + ea_n0));
   }
   const double rows = (U.L + P - 1) / P;
-  return 4000.0 + (U.kind == 1 ? 0.45 : 0.205) * ising_scale * rows * U.L;
+  return 3.0 + (U.kind == 1 ? 0.45e-3 : 0.16e-3) * ising_scale * rows * U.L;
 }
 
 // The next larger team for which the unit's time falls (cap + 1: none).
@@ -1082,9 +1102,9 @@ static bool batch_item_ok(const spin_batch_item &it, int32_t pt_every) {
   return false;
 }
 
-// Dynamic shared memory of a CTA that has its SM to itself, beside ~26 KB of
+// Dynamic shared memory of a CTA that has its SM to itself, beside 9 KB of
 // counters and masks.
-constexpr int kResidentSmem = 196 * 1024;
+constexpr int kResidentSmem = 212 * 1024;
 
 // One 512-thread CTA per SM with word-lattices in shared memory, against two
 // of 256 threads that read them from L2: the update is bound by the latency of

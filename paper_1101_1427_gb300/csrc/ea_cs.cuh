@@ -341,18 +341,18 @@ __device__ __forceinline__ Flip ea_site_flip(const EaSiteW &x, const EaSiteJ &c,
   return ea_flip2(x.S ^ x.xp ^ c.xp, x.S ^ x.xm ^ c.xm, x.S ^ x.yp ^ c.yp, x.S ^ x.ym ^ c.ym, r, t4, t8);
 }
 
-// One colour phase of one 3D word-lattice by the warps `warp`, warp + warps,
-// ... (all lanes), each 128 consecutive colour indices at a time: lane l draws
-// the call of quad l of them, and sites 32 s + l take their words from lane
-// 8 s + l / 4.  add(f, on) receives each site's Flip and whether the lane has
+// One colour phase of the chunks [c0, c1) (128 consecutive colour indices
+// each) of one 3D word-lattice by a warp: lane l draws the call of quad l of a
+// chunk, and sites 32 s + l take their words from lane 8 s + l / 4.  add(f, on) receives each site's Flip and whether the lane has
 // a site.
 template <typename AddFn>
 __device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, int colour,
                                                uint32_t L, uint32_t N, const FastDiv &fL, const RoundKeys &rk,
                                                uint32_t sweep, uint32_t lid, uint32_t t4, uint32_t t8, uint32_t t12,
-                                               uint32_t warp, uint32_t warps, AddFn add) {
+                                               uint32_t c0, uint32_t c1, AddFn add) {
   const uint32_t half = N >> 1, lane = threadIdx.x & 31u, wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
-  for (uint32_t base = 128u * warp; base < half; base += 128u * warps) {
+  const uint32_t end = min(128u * c1, half);
+  for (uint32_t base = 128u * c0; base < end; base += 128u) {
     const uint4 v = philox(make_uint4((base >> 2) + lane, sweep, lid, wctr), rk);
 #pragma unroll
     for (uint32_t s = 0; s < 4; ++s) {
