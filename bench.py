@@ -72,7 +72,7 @@ EA_PT_ALU_PER_WORD = 28 + 10 + 1
 # (one launch captured with ncu, summarised in profiles/), valid while the
 # kernel's sources (comments removed) hash to KERNEL_TRAFFIC_SRC_SHA; otherwise reported as null.
 KERNEL_TRAFFIC_BYTES = 100_685_056 + 12_079_616
-KERNEL_TRAFFIC_SRC_SHA = "b52d13f1d06b3ad2"
+KERNEL_TRAFFIC_SRC_SHA = "aa56021a4a46da97"
 
 
 def kernel_sha():

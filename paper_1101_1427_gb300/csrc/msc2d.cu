@@ -364,8 +364,10 @@ __global__ void msc2d_measure_kernel(const uint32_t *__restrict__ w, Msc2d m, in
                                      long long *__restrict__ E, long long *__restrict__ M) {
   const int64_t lat = blockIdx.y;
   const uint32_t blocks = (uint32_t)m.L * (uint32_t)m.bpr;  // blocks of 4 colour-0 words per lattice
+  griddep_wait();
+  griddep_release();
   const uint32_t *wl = w + lat * m.lat_words;
-  long long anti = 0, down = 0;
+  int anti = 0, down = 0;  // (at most 64 blocks of 512 bonds per thread, L < 2^16)
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < blocks; k += gridDim.x * blockDim.x) {
     const uint32_t y = k / (uint32_t)m.bpr, B = k - y * (uint32_t)m.bpr;
     const uint32_t yu = y == 0 ? (uint32_t)m.L - 1 : y - 1, yd = y == (uint32_t)m.L - 1 ? 0 : y + 1;
@@ -390,17 +392,23 @@ __global__ void msc2d_measure_kernel(const uint32_t *__restrict__ w, Msc2d m, in
     down += __popc(s.x) + __popc(s.y) + __popc(s.z) + __popc(s.w) + __popc(o.x) + __popc(o.y) + __popc(o.z) +
             __popc(o.w);
   }
-  anti = warp_sum(anti);
-  down = warp_sum(down);
+  // one pair of atomics per CTA: per warp, their queue at the lattice's two
+  // sums took most of the time (3 x L = 16384: 126 us)
+  __shared__ int red[8][2];
+  anti = __reduce_add_sync(0xffffffffu, anti);
+  down = __reduce_add_sync(0xffffffffu, down);
   if ((threadIdx.x & 31) == 0) {
-    const long long N = (long long)m.L * m.L;
-    atomicAdd((unsigned long long *)&E[lat], (unsigned long long)(2 * anti));
-    atomicAdd((unsigned long long *)&M[lat], (unsigned long long)(-2 * down));
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      atomicAdd((unsigned long long *)&E[lat], (unsigned long long)(-2 * N));
-      atomicAdd((unsigned long long *)&M[lat], (unsigned long long)N);
-    }
+    red[threadIdx.x >> 5][0] = anti;
+    red[threadIdx.x >> 5][1] = down;
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  long long a = 0, d = 0;
+  for (int k = 0; k < 8; ++k) a += red[k][0], d += red[k][1];
+  const long long N = (long long)m.L * m.L;
+  const bool first = blockIdx.x == 0;
+  atomicAdd((unsigned long long *)&E[lat], (unsigned long long)(2 * a - (first ? 2 * N : 0)));
+  atomicAdd((unsigned long long *)&M[lat], (unsigned long long)((first ? N : 0) - 2 * d));
 }
 
 cudaError_t launch_measure_msc2d(spin_lattice *h, int64_t *E, int64_t *M) {
@@ -412,11 +420,10 @@ cudaError_t launch_measure_msc2d(spin_lattice *h, int64_t *E, int64_t *M) {
   cudaMemsetAsync(e, 0, sizeof(long long) * h->n_lat, h->stream);
   cudaMemsetAsync(mm, 0, sizeof(long long) * h->n_lat, h->stream);
   const int64_t blocks = (int64_t)m.L * m.bpr;  // one thread per block of 4 colour-0 words
-  unsigned gx = grid_for(blocks, 256);
-  if (gx > 4096u) gx = 4096u;
-  msc2d_measure_kernel<<<dim3(gx, (unsigned)h->n_lat), 256, 0, h->stream>>>(
-      (const uint32_t *)h->spins, m, h->n_lat, e, mm);
-  return cudaGetLastError();
+  unsigned gx = grid_for(blocks, 256 * 4);  // a few blocks per thread, where there are enough
+  if (gx > 1024u) gx = 1024u;
+  return launch_dependent(msc2d_measure_kernel, dim3(gx, (unsigned)h->n_lat), dim3(256), 0, h->stream,
+                          (const uint32_t *)h->spins, m, h->n_lat, e, mm);
 }
 
 }  // namespace spin
