@@ -18,12 +18,14 @@
 // one measurement at L = 128 went from 601 to 388 us.  Sums whose spins are far from unit
 // length, where an FP32 product could overflow or vanish, are formed in FP64.
 //
-// A lattice has kHeisParts partials whatever its size; lattices of at least
-// kHeisClusterSites sites take a cluster of kHeisCluster CTAs per partial,
-// whose sums rank 0 adds in rank order, so that 512 CTAs instead of 64 share
-// the work.  The rule depends on the lattice size alone, so that the sums do
-// not depend on how many lattices a call takes; below 2^17 sites a larger
-// grid has no site for some threads.
+// A lattice has kHeisParts partials whatever its size; large lattices take a
+// cluster of 2, 4 or 8 CTAs per partial, whose sums rank 0 adds in rank order,
+// so that up to 512 CTAs share the work.  The rule depends on the lattice size
+// alone, so that the sums do not depend on how many lattices a call takes.  It
+// keeps 32 sites and more per thread (16 from 2^21 sites on), since the FP64
+// additions of the tree cost a thread as much as several sites: with 8 CTAs per
+// partial, 8 lattices of L = 64 took 123 us and 4 of L = 80 68 us, with one 37
+// and 39; one of L = 80 26 against 33, of L = 100 30 against 55.
 #pragma once
 #include <cooperative_groups.h>
 #include <stdint.h>
@@ -32,11 +34,12 @@
 
 namespace spin {
 
-constexpr int kHeisParts = 64;                      // partials per lattice
-constexpr int kHeisCluster = 8;                     // CTAs per partial of a large lattice
-constexpr int64_t kHeisClusterSites = 1 << 17;
+constexpr int kHeisParts = 64;  // partials per lattice
 
-inline int heis_measure_cluster(int64_t N) { return N >= kHeisClusterSites ? kHeisCluster : 1; }
+// CTAs per partial of a lattice of N sites.
+inline int heis_measure_cluster(int64_t N) {
+  return N >= (1 << 21) ? 8 : N >= (1 << 20) ? 4 : N >= (1 << 19) ? 2 : 1;
+}
 
 // The exact sum a + b = s + e (Knuth; no assumption on magnitudes).
 __device__ __forceinline__ float two_sum(float a, float b, float &e) {

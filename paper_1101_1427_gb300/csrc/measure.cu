@@ -475,10 +475,11 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
     double *partial = (double *)h->d_scratch64;
     const int c = heis_measure_cluster(g.N);
     const dim3 grid((unsigned)(kHeisParts * c), (unsigned)nl);
-    cudaError_t e = c == 1 ? launch_dependent(measure_heis_kernel<1>, grid, dim3(256), 0, st,
-                                              (const float4 *)h->spins, g, partial)
-                           : launch_clusters(measure_heis_kernel<kHeisCluster>, grid, dim3(256), c, 0, st,
-                                             (const float4 *)h->spins, g, partial);
+    const auto kern = c == 8   ? measure_heis_kernel<8>
+                      : c == 4 ? measure_heis_kernel<4>
+                      : c == 2 ? measure_heis_kernel<2>
+                               : measure_heis_kernel<1>;
+    const cudaError_t e = launch_clusters(kern, grid, dim3(256), c, 0, st, (const float4 *)h->spins, g, partial);
     if (e != cudaSuccess) return e;
     return launch_dependent(finish_heis_kernel, dim3(grid_for(4 * nl, 128)), dim3(128), 0, st,
                             (const double *)partial, nl, Ef, Mf);

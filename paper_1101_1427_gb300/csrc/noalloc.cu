@@ -89,7 +89,11 @@ extern "C" int spin_heis_measure_noalloc(const float *spins, int32_t dim, int32_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const cudaError_t e =
-      cudaLaunchKernelEx(&cfg, c == 1 ? heis_partials_kernel<1> : heis_partials_kernel<spin::kHeisCluster>,
+      cudaLaunchKernelEx(&cfg,
+                         c == 8   ? heis_partials_kernel<8>
+                         : c == 4 ? heis_partials_kernel<4>
+                         : c == 2 ? heis_partials_kernel<2>
+                                  : heis_partials_kernel<1>,
                          (const float4 *)spins, (int)dim, (uint32_t)L, fL, N, part);
   if (e != cudaSuccess) return SPIN_ECUDA;
   heis_finish_kernel<<<(4 * n_lat + 127) / 128, 128, 0, st>>>(part, n_lat, Ef, Mf);

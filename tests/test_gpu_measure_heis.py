@@ -1,5 +1,5 @@
-"""Heisenberg energy and magnetisation on either side of the size (2^17
-sites) from which a cluster of CTAs shares each partial sum, against FP64
+"""Heisenberg energy and magnetisation on either side of the sizes (2^19, 2^20,
+2^21 sites) from which clusters of 2, 4, 8 CTAs share each partial sum, against FP64
 sums of the same FP32 spins, and bit for bit against the allocation-free
 entry point."""
 import numpy as np
@@ -12,7 +12,8 @@ import paper_1101_1427_gb300 as sp  # noqa: E402
 from paper_1101_1427_gb300 import _binding as B  # noqa: E402
 
 
-@pytest.mark.parametrize("dim,L,n_lat", [(2, 4, 5), (2, 362, 2), (2, 364, 2), (3, 50, 1), (3, 52, 3), (3, 64, 1)])
+@pytest.mark.parametrize("dim,L,n_lat", [(2, 4, 5), (2, 362, 2), (2, 724, 1), (2, 726, 2), (3, 52, 3), (3, 80, 1),
+                                            (3, 82, 1), (3, 102, 2), (3, 126, 1), (3, 128, 1)])
 def test_heisenberg_sums(dim, L, n_lat):
     N = L ** dim
     rng = np.random.default_rng(N)
