@@ -57,13 +57,17 @@ __global__ void __launch_bounds__(256) ising2d_phase_kernel(int8_t *__restrict__
                                                             const uint32_t *__restrict__ thr,
                                                             Geom g, RoundKeys rk, uint32_t sweep,
                                                             int colour) {
-  griddep_wait();
   griddep_release();
   const int chunks = L >> 3;
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int64_t lat = blockIdx.z;
   if (m >= chunks || y >= L) return;
+  const uint32_t t = slot_of32(g, (uint32_t)lat);
+  const uint32_t thr4 = __ldg(thr + 4 * t + 1), thr8 = __ldg(thr + 4 * t + 2);
+  const uint32_t j4 = (uint32_t)y * (uint32_t)chunks + (uint32_t)m;
+  const uint4 r = philox(make_uint4(j4, sweep, lattice_id32(g, (uint32_t)lat), ctr_w(TAG_UPDATE, colour, 0)), rk);
+  griddep_wait();  // the words need no spin
   int8_t *base = spins + lat * (int64_t)L * L;
   const int yu = y == 0 ? L - 1 : y - 1, yd = y == L - 1 ? 0 : y + 1;
   const uint64_t *row = reinterpret_cast<const uint64_t *>(base + (int64_t)y * L);
@@ -74,10 +78,6 @@ __global__ void __launch_bounds__(256) ising2d_phase_kernel(int8_t *__restrict__
   const int p = (colour + y) & 1;
   const int xe = p ? (m == chunks - 1 ? 0 : 8 * m + 8) : (m == 0 ? L - 1 : 8 * m - 1);
   const uint64_t lb = (uint8_t)base[(int64_t)y * L + xe], rb = lb;
-  const uint32_t t = slot_of32(g, (uint32_t)lat);
-  const uint32_t thr4 = __ldg(thr + 4 * t + 1), thr8 = __ldg(thr + 4 * t + 2);
-  const uint32_t j4 = (uint32_t)y * (uint32_t)chunks + (uint32_t)m;
-  const uint4 r = philox(make_uint4(j4, sweep, lattice_id32(g, (uint32_t)lat), ctr_w(TAG_UPDATE, colour, 0)), rk);
   long long unused_a = 0, unused_d = 0;
   reinterpret_cast<uint64_t *>(base + (int64_t)y * L)[m] =
       ising_chunk<0>(C, U, D, lb, rb, r, p, thr4, thr8, unused_a, unused_d);
@@ -355,12 +355,16 @@ __global__ void __launch_bounds__(256) phase_generic_kernel(int8_t *__restrict__
                                                             uint32_t sweep, int colour) {
   const uint32_t L = (uint32_t)g.L, LL = L * L, N = (uint32_t)g.N, half = N / 2;
   const uint32_t quads = (half + 3) / 4;
+  bool waited = false;
+  griddep_release();
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
     const uint32_t lat = fdiv(k, g.fquads), j4 = k - lat * quads;
     int8_t *s = spins + (size_t)lat * N;
     const int8_t *Jr = J ? J + (size_t)(lat - fdiv(lat, g.freal) * (uint32_t)g.n_real) * g.dim * N : nullptr;
     const uint32_t t = slot_of32(g, lat);
     const uint4 r = philox(make_uint4(j4, sweep, lattice_id32(g, lat), ctr_w(TAG_UPDATE, colour, 0)), rk);
+    if (!waited) griddep_wait();  // the words need no spin
+    waited = true;
 #pragma unroll
     for (uint32_t q = 0; q < 4; ++q) {
       const uint32_t j = 4 * j4 + q;
@@ -515,11 +519,11 @@ cudaError_t launch_sweeps_i8(spin_lattice *h, const int8_t *J, int64_t n_sweeps)
         const uint32_t total = (uint32_t)(h->n_lat * ((g.N / 2 + 3) / 4));
         unsigned grid = grid_for(total, 256);
         if (grid > 1u << 20) grid = 1u << 20;
-        phase_generic_kernel<<<grid, 256, 0, h->stream>>>((int8_t *)h->spins, J, h->d_thr, g,
-                                                           total, rk, sweep, colour);
+        const cudaError_t e = launch_dependent(phase_generic_kernel, dim3(grid), dim3(256), 0, h->stream,
+                                               (int8_t *)h->spins, J, (const uint32_t *)h->d_thr, g, total, rk, sweep,
+                                               colour);
+        if (e != cudaSuccess) return e;
       }
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
     }
   }
   return cudaSuccess;
