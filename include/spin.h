@@ -30,10 +30,12 @@
  * by the caller; the library only borrows device pointers while the work it
  * enqueued on the handle's stream runs.  A handle owns small workspaces
  * (threshold tables, reduction partials, an error word), allocated by
- * spin_init, and one lattice-sized working buffer allocated by the first
- * sweep call that needs it (the fused 2D int8 pass, the coded path of int8
- * lattices, long Heisenberg calls), with, for the resident 3D Heisenberg
- * sweeps, one counter per CTA; all are freed by spin_destroy.
+ * spin_init, and one working buffer allocated by the first sweep call that
+ * needs it (the fused 2D int8 pass; the bit planes of longer calls on int8
+ * ferromagnets, for small lattices with the acceptance masks of the sweeps
+ * ahead, at most about 32 MB or two sweeps' masks; long Heisenberg calls),
+ * with, for the resident 3D Heisenberg sweeps, one counter per CTA; all are
+ * freed by spin_destroy.
  *
  * Errors: every entry point returns 0 (SPIN_OK) or a negative SPIN_E* code
  * and never throws.  Work is asynchronous on the handle's stream; kernel
@@ -330,14 +332,19 @@ int spin_set_counters(spin_lattice *lat, int64_t sweeps_done, int64_t pt_steps_d
  * with L % 256 != 0), 3 = resident: one CTA per lattice holds the whole
  * lattice in shared memory for all sweeps of a call and measures E and M
  * itself (default for L % 8 == 0, L <= 128; the paper's tempering code
- * likewise maps replicas to thread blocks, Sec. 6), 4 = coded: a call of at
- * least 4 sweeps packs the lattices into a handle-owned 1-bit buffer
- * (L^2 / 8 bytes per lattice, allocated on first use, kept until
- * spin_destroy), runs the synchronous multi-spin-coded sweep (Sec. 5) and
- * unpacks them, shorter calls take the fused pass (default for
- * L % 256 == 0, L > 128); all four give identical results.  3D int8
- * ferromagnet: 0 = colour phases, 3 = resident (default for L % 8 == 0,
- * L <= 24), identical results.  Heisenberg: 0 = the full-accuracy FP32
+ * likewise maps replicas to thread blocks, Sec. 6); calls long enough to
+ * win back a second launch draw the acceptance masks of many sweeps ahead
+ * with the whole GPU and hold the lattice as bit planes), 4 = coded: a call
+ * of at least 4 sweeps packs the lattices into bit planes in the handle's
+ * working buffer (synchronous multi-spin coding, Sec. 5), sweeps, measures
+ * and exchanges there and unpacks them at its end, shorter calls take the
+ * fused pass (default for L % 256 == 0, L > 128); all four give identical
+ * results.  3D int8 ferromagnet: 0 = colour phases, 3 = resident (default
+ * for L % 8 == 0, L <= 24), identical results.  A handle whose variant was
+ * never set takes the bit planes for every other L % 8 == 0 too, in two and
+ * three dimensions, in calls of at least 2 sweeps (4 where the fused pass is
+ * its default); where no working buffer can be had (no memory, or inside a
+ * stream capture before an uncaptured call made it) it takes its variant.  Heisenberg: 0 = the full-accuracy FP32
  * library functions (default), 2 = the paper's "fast_math" mode (Sec. 4):
  * rho = sqrt(1 - z^2) from the hardware reciprocal square root, sin and cos
  * of the azimuth from the hardware sine and cosine on [-pi, pi), and the
@@ -432,7 +439,8 @@ int spin_set_update_order(spin_lattice *lat, int32_t order, int32_t tile, int32_
  * (1 .. 100000; a multiple of the hits in the double-checkerboard order)
  * with the given couplings and HOST betas for every choice that leaves the
  * handle's chain unchanged -- the kernel variants of the int8 ferromagnet
- * (spin_set_variant: 0, 1, 3, 4 where supported) -- and, for a
+ * (spin_set_variant: 0, 1, 3, 4 where supported, and the default form of a
+ * handle whose variant was never set) -- and, for a
  * double-checkerboard handle whose tile edge was left open (tile 0), every
  * supported tile edge (each gives its own chain, Sec. 3.2).  The fastest
  * choice is set on the handle and cached per (model, layout, dim, L,

@@ -304,6 +304,7 @@ constexpr int kTapeExtra = 4;           // sweeps by which a half is longer than
 // for one CTA of the next masks only, which may run at the same time.
 constexpr int kResSpread = 200 * 1024;
 constexpr int kTapeSpread = 20 * 1024;
+constexpr int64_t kResMinTape = 512;
 constexpr int64_t kResMaxSweeps = 4096;  // per launch, so that none runs for long
 
 }  // namespace
@@ -333,7 +334,9 @@ uint4 *tape_of(const spin_lattice *h) {
 bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
   const Planes m = make_planes(h->g.dim, h->g.L);
   const size_t per = tape_sweep_bytes(h, m);
-  int64_t sweeps = n_sweeps < kResMaxSweeps ? n_sweeps : kResMaxSweeps;
+  // (calls of growing length make few buffers: a power of two, at least 512)
+  int64_t sweeps = kResMinTape;
+  while (sweeps < n_sweeps && sweeps < kResMaxSweeps) sweeps *= 2;
   if (sweeps > 1 && (size_t)sweeps * per > kTapeMax) sweeps = (int64_t)(kTapeMax / per) + 1;
   const size_t need = planes_pair_bytes(h) + 2 * (size_t)(sweeps + kTapeExtra) * per;
   if (h->d_pingpong && h->pingpong_bytes >= need) return true;

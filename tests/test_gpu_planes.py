@@ -20,7 +20,8 @@ def twin(dim, L, n_temps, n_real, seed):
 @pytest.mark.parametrize("dim,L,n_temps,n_real", [
     (2, 136, 3, 2), (2, 200, 1, 1), (2, 264, 2, 1), (2, 520, 5, 1), (2, 1000, 3, 1), (2, 512, 4, 1), (2, 2056, 40, 1),
     (3, 32, 4, 1), (3, 40, 3, 1), (3, 48, 1, 2), (3, 56, 1, 1), (3, 72, 2, 1), (3, 80, 3, 1), (3, 96, 1, 1),
-    (3, 104, 1, 1), (3, 128, 1, 1), (3, 136, 2, 1), (3, 264, 1, 1), (3, 192, 5, 1)])
+    (3, 104, 1, 1), (3, 128, 1, 1), (3, 136, 2, 1), (3, 264, 1, 1), (3, 192, 5, 1),
+    (2, 4096, 1, 1), (2, 4112, 1, 1), (2, 2832, 3, 1)])
 def test_planes_equal_the_colour_phases(dim, L, n_temps, n_real):
     beta = 0.4407 if dim == 2 else 0.2216544
     betas = [beta * (1 + 0.02 * t) for t in range(n_temps)]
