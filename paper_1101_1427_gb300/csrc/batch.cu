@@ -310,10 +310,22 @@ __device__ __forceinline__ void ea_phase_warp(uint32_t *__restrict__ s, const ui
   }
 }
 
-// Counts per bit the words a[i] (or a[i] ^ b[i]) of i in [i0, i1), by a warp.
+// Counts per bit the words a[i] (or a[i] ^ b[i]) of i in [i0, i1), by a warp;
+// the loads of sixteen words per lane are under way together.
 __device__ __forceinline__ void count_words(HsCount &hc, const uint32_t *a, const uint32_t *b, uint32_t i0,
                                             uint32_t i1) {
   uint32_t i = i0 + (threadIdx.x & 31u);
+  for (; i + 15 * 32 < i1; i += 16 * 32) {
+    uint32_t x[8], y[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = a[i + 32 * k], y[k] = a[i + 32 * (k + 8)];
+    if (b) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] ^= b[i + 32 * k], y[k] ^= b[i + 32 * (k + 8)];
+    }
+    hc.add8(x);
+    hc.add8(y);
+  }
   for (; i + 7 * 32 < i1; i += 8 * 32) {
     uint32_t x[8];
 #pragma unroll
@@ -358,14 +370,18 @@ static __device__ __forceinline__ void cta_swap_bits(uint32_t *w0, uint32_t *w1,
   uint4 *v0 = reinterpret_cast<uint4 *>(w0), *v1 = reinterpret_cast<uint4 *>(w1);
   const uint32_t n4 = N >> 2;
   uint32_t i = threadIdx.x;
-  for (; i + kThreads < n4; i += 2 * kThreads) {
-    uint4 x0 = v0[i], x1 = v1[i], y0 = v0[i + kThreads], y1 = v1[i + kThreads];
-    uint4 d = make_uint4((x0.x ^ x1.x) & A, (x0.y ^ x1.y) & A, (x0.z ^ x1.z) & A, (x0.w ^ x1.w) & A);
-    uint4 e = make_uint4((y0.x ^ y1.x) & A, (y0.y ^ y1.y) & A, (y0.z ^ y1.z) & A, (y0.w ^ y1.w) & A);
-    v0[i] = make_uint4(x0.x ^ d.x, x0.y ^ d.y, x0.z ^ d.z, x0.w ^ d.w);
-    v1[i] = make_uint4(x1.x ^ d.x, x1.y ^ d.y, x1.z ^ d.z, x1.w ^ d.w);
-    v0[i + kThreads] = make_uint4(y0.x ^ e.x, y0.y ^ e.y, y0.z ^ e.z, y0.w ^ e.w);
-    v1[i + kThreads] = make_uint4(y1.x ^ e.x, y1.y ^ e.y, y1.z ^ e.z, y1.w ^ e.w);
+  constexpr int kU = 4;  // pairs of 16-byte words under way per thread
+  for (; i + (kU - 1) * kThreads < n4; i += kU * kThreads) {
+    uint4 x[kU], y[kU];
+#pragma unroll
+    for (int k = 0; k < kU; ++k) x[k] = v0[i + k * kThreads], y[k] = v1[i + k * kThreads];
+#pragma unroll
+    for (int k = 0; k < kU; ++k) {
+      const uint4 d = make_uint4((x[k].x ^ y[k].x) & A, (x[k].y ^ y[k].y) & A, (x[k].z ^ y[k].z) & A,
+                                 (x[k].w ^ y[k].w) & A);
+      v0[i + k * kThreads] = make_uint4(x[k].x ^ d.x, x[k].y ^ d.y, x[k].z ^ d.z, x[k].w ^ d.w);
+      v1[i + k * kThreads] = make_uint4(y[k].x ^ d.x, y[k].y ^ d.y, y[k].z ^ d.z, y[k].w ^ d.w);
+    }
   }
   for (; i < n4; i += kThreads) {
     const uint4 x0 = v0[i], x1 = v1[i];

@@ -353,6 +353,14 @@ __device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const u
   const uint32_t half = N >> 1, lane = threadIdx.x & 31u, wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
   const uint32_t end = min(128u * c1, half);
   for (uint32_t base = 128u * c0; base < end; base += 128u) {
+    // the words of the four sites first, so that their latencies overlap
+    EaSite e[4];
+    EaSiteW x[4];
+#pragma unroll
+    for (uint32_t s = 0; s < 4; ++s) {
+      e[s] = ea_site<3>(min(base + 32u * s + lane, half - 1), colour, L, fL);
+      x[s] = ea_site_words<3>(w, e[s], colour, N);
+    }
     const uint4 v = philox(make_uint4((base >> 2) + lane, sweep, lid, wctr), rk);
 #pragma unroll
     for (uint32_t s = 0; s < 4; ++s) {
@@ -364,10 +372,8 @@ __device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const u
       const bool on = j < half;
       Flip f = {};
       if (on) {
-        const EaSite e = ea_site<3>(j, colour, L, fL);
-        const EaSiteW x = ea_site_words<3>(w, e, colour, N);
-        f = ea_site_flip<3>(x, ea_site_couplings<3>(J, e, colour, N), r, t4, t8, t12);
-        w[(uint32_t)colour * half + j] = x.S ^ f.F;
+        f = ea_site_flip<3>(x[s], ea_site_couplings<3>(J, e[s], colour, N), r, t4, t8, t12);
+        w[(uint32_t)colour * half + j] = x[s].S ^ f.F;
       }
       add(f, on);
     }
