@@ -239,7 +239,7 @@ def config_rooflines(side, i8_value, sms, mhz):
                 "per_flip": per_flip, "peak_basis": basis, "kernel": kernel}
 
     out = {"2d_ising_L16384_i8": line(i8_value, philox2d, f"{WIDE_MULS_PER_FLIP} wide multiplies (Philox)",
-                                      mul_basis, "msc2d_pack/phase/unpack (coded path of the int8 layout)")}
+                                      mul_basis, "planes_phase_kernel (bit planes of the int8 layout)")}
     for key, name in (("heisenberg_L128_fp32_flips_per_ns", "3d_heisenberg_L128_fp32"),
                       ("heisenberg_L128_fp32_fast_flips_per_ns", "3d_heisenberg_L128_fp32_fast")):
         out[name] = line(side.get(key), heis, f"{HEIS_WIDE_MULS_PER_FLIP} wide multiplies (one Philox call)",
@@ -459,8 +459,8 @@ def dcb(torch, sp, B, stream):
 def ising_pt_sizes(torch, sp, B, stream):
     """The tempering benchmark over lattice sizes (the paper plots its flip
     time against L, Sec. 6): 20 int8 replicas, beta in [0.1, 0.15], one
-    exchange per 100 sweeps, with the resident kernel (L <= 128) and the
-    fused pass (L >= 32)."""
+    exchange per 100 sweeps, with one CTA per lattice (variant 3, L <= 128)
+    and the fused pass (L >= 32)."""
     import numpy as np
     out = {}
     betas = list(np.linspace(0.1, 0.15, 20))
@@ -486,8 +486,8 @@ def ising_pt_sizes(torch, sp, B, stream):
 
 def ising2d_small(torch, sp, B, stream):
     """2D Ising L = 64, int8, beta = 0.4407, 1000 sweeps with E and M after
-    every sweep (one spin_run call), with the resident kernel (which
-    measures itself: one launch) and with the fused pass plus a separate
+    every sweep (one spin_run call), with one CTA per lattice (variant 3,
+    which measures itself) and with the fused pass plus a separate
     measurement per sweep."""
     out = {}
     for variant, name in ((3, "resident"), (1, "fused")):
@@ -509,8 +509,8 @@ def ising_pt(torch, sp, B, stream):
     """The paper's tempering benchmark for the 2D ferromagnet (Sec. 6): 20
     int8 replicas at equally spaced beta in [0.1, 0.15], one exchange step
     per 100 (and per 10) sweeps; flips/ns counts spin flips of all replicas.
-    Each size runs its default kernel: resident (whole lattice in one CTA)
-    at L = 64, the fused pass at L = 2048."""
+    Each size runs its default form: a CTA per lattice on masks drawn ahead
+    at L = 64, bit planes with a launch per colour phase at L = 2048."""
     import numpy as np
     out = {}
     betas = list(np.linspace(0.1, 0.15, 20))
@@ -823,7 +823,7 @@ def run_case(name):
     a, b = _events(torch)
     if name in ("msc2d", "fused2d", "i8coded"):
         # fused2d: two-sweep calls of the int8 lattices (the fused pass);
-        # i8coded: four-sweep calls (pack, coded sweeps, unpack)
+        # i8coded: four-sweep calls (packed to bit planes, swept, unpacked)
         layout = B.SPIN_MSC1 if name == "msc2d" else B.SPIN_I8
         n = 4 if name == "i8coded" else 2
         lat = sp.Lattice(B.SPIN_ISING, 2, L, layout, n_temps=3, seed=1)

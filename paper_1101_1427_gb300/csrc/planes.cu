@@ -7,7 +7,7 @@
 // bytes; on planes the generator and its two or three comparisons per word
 // are nearly all that is left.  Measured against them (us per call of the
 // byte kernels -> here): one 3D L = 512, 4 sweeps and a measurement, 859 ->
-// 535; three L = 1000, 20 sweeps and 2 measurements, 164 -> 111; 20 x L = 512,
+// 530; three L = 1000, 20 sweeps and 2 measurements, 164 -> 111; 20 x L = 512,
 // 20 sweeps and 2 exchanges, 135 -> 113 (packed once instead of per exchange).
 #include <algorithm>
 

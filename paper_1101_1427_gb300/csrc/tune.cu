@@ -1,7 +1,7 @@
 // Per-handle autotuner: kernel form and double-checkerboard tile edge.
 //
 // The int8 ferromagnet has several kernel forms that give the same chain
-// (colour phases, fused pass, resident lattice, coded path); which one is
+// (colour phases, fused pass, resident lattice, bit planes); which one is
 // fastest depends on the lattice size, the number of lattices and the call
 // length.  The double-checkerboard order (Sec. 3.2) takes a tile edge T whose
 // best value the paper finds by measurement (Sec. 3.5, Fig. blocks: tiles against
