@@ -6,6 +6,9 @@
 // set <=> J = -1.  The 32 realisations of a word share one
 // uniform per site and sweep (the paper's footnote to Sec. 5), so one Philox
 // call serves four word-sites.
+#include <algorithm>
+#include <cmath>
+
 #include "ea_cs.cuh"
 #include "internal.h"
 
@@ -57,6 +60,9 @@ struct NoAdd {
   __device__ void operator()(uint32_t, uint32_t, uint32_t) const {}
 };
 
+constexpr int kResThreads = 512;    // at most, msc_res_kernel
+constexpr int64_t kResSweeps = 1024;  // sweeps per launch
+constexpr size_t kResSmem = 227 * 1024 - 64;  // beside its thresholds
 constexpr uint32_t kSlots = 4;  // slots of one (set, group) per thread of a colour phase
 
 // Place of thread item k: (a, grp) and the first slot of its block, with the
@@ -161,6 +167,80 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// Several sweeps of lattices that fit in shared memory: a CTA holds the words
+// of one slot block (kSlots slots of one set and group) and the group's
+// couplings, and runs every sweep of the call with a barrier per colour phase
+// instead of a launch.  Items, draws and updates are those of the phase kernels.
+// Bound by the latency of a phase in one CTA (L = 12: 1.9 us for two sites per
+// thread in four slots, 3.6 with a launch per phase): 10 sweeps of 256 x 30 x 2
+// lattices of L = 12 with 2 measurements and exchanges 116 -> 100 us.
+template <int kDim, bool kPair, bool kRow>
+__global__ void __launch_bounds__(kResThreads)
+    msc_res_kernel(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, Geom g, FastDiv ftb,
+                   const uint32_t *__restrict__ thr, RoundKeys rk, uint32_t sweep0, uint32_t n_sweeps) {
+  extern __shared__ uint4 msc_res_smem[];
+  __shared__ uint32_t s_thr[kSlots][4];
+  griddep_release();
+  const uint32_t N = (uint32_t)g.N, half = N / 2, quads = (half + 3) / 4, lane4 = threadIdx.x & 3u;
+  const uint32_t G = (uint32_t)g.n_real / 32, T = (uint32_t)g.n_temps, TB = (T + kSlots - 1) / kSlots;
+  const uint32_t st = fdiv(blockIdx.x, ftb), a = fdiv(st, g.fgrp), grp = st - a * G;
+  const uint32_t t0 = (blockIdx.x - st * TB) * kSlots, n_slots = min(kSlots, T - t0);
+  const uint32_t rkey = kPair ? grp >> 1 : grp;
+  uint32_t *sw = reinterpret_cast<uint32_t *>(msc_res_smem), *sJ = sw + kSlots * N;
+  uint32_t *ws = w + ((size_t)st * T + t0) * N;
+  const uint32_t *gJ = J + (size_t)grp * kDim * N;
+  griddep_wait();
+#pragma unroll 8
+  for (uint32_t i = threadIdx.x; i < n_slots * N; i += blockDim.x) sw[i] = ws[i];
+#pragma unroll 8
+  for (uint32_t i = threadIdx.x; i < kDim * N; i += blockDim.x) sJ[i] = gJ[i];
+  if (threadIdx.x < 4 * n_slots) s_thr[threadIdx.x >> 2][threadIdx.x & 3u] = thr[4 * t0 + threadIdx.x];
+  __syncthreads();
+  for (uint32_t k = 0; k < n_sweeps; ++k) {
+    const uint32_t sweep = sweep0 + k;
+#pragma unroll 1
+    for (int colour = 0; colour < 2; ++colour) {
+      const uint32_t wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
+      if (kRow) {
+        for (uint32_t j4 = threadIdx.x; j4 < quads; j4 += blockDim.x) {
+          const EaQuadGeom q = ea_quad_geom<kDim>(j4, colour, (uint32_t)g.L, g.fL);
+          const EaQuadJ c = ea_quad_couplings<kDim>(sJ, q, colour, N);
+#pragma unroll 1
+          for (uint32_t s = 0; s < n_slots; ++s) {
+            const uint4 r = philox(make_uint4(j4, sweep, lattice_id(a, rkey, t0 + s), wctr), rk);
+            ea_quad_update<kDim, false>(sw + s * N, q, c, colour, N, r, s_thr[s][1], s_thr[s][2], s_thr[s][3],
+                                        NoAdd());
+          }
+        }
+      } else {
+        // whole warps, for the exchange of words between lanes
+        for (uint32_t id = threadIdx.x; (id & ~31u) < 4 * quads; id += blockDim.x) {
+          const uint32_t j4 = min(id >> 2, quads - 1), j = id;
+          const uint4 v = philox(make_uint4(j4, sweep, lattice_id(a, rkey, t0 + min(lane4, n_slots - 1)), wctr), rk);
+          uint32_t r[kSlots] = {v.x, v.y, v.z, v.w};
+          quad_transpose(r);  // r[s]: the site's word in slot t0 + s
+          if (j >= half) continue;
+          const EaSite e = ea_site<kDim>(j, colour, (uint32_t)g.L, g.fL);
+          const EaSiteJ c = ea_site_couplings<kDim>(sJ, e, colour, N);
+          EaSiteW x[kSlots];
+#pragma unroll
+          for (uint32_t s = 0; s < kSlots; ++s)
+            x[s] = ea_site_words<kDim>(sw + min(s, n_slots - 1) * N, e, colour, N);
+#pragma unroll
+          for (uint32_t s = 0; s < kSlots; ++s) {
+            if (s >= n_slots) break;
+            const Flip f = ea_site_flip<kDim>(x[s], c, r[s], s_thr[s][1], s_thr[s][2], s_thr[s][3]);
+            sw[s * N + (uint32_t)colour * half + j] = x[s].S ^ f.F;
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+#pragma unroll 8
+  for (uint32_t i = threadIdx.x; i < n_slots * N; i += blockDim.x) ws[i] = sw[i];
+}
+
 // Words <-> one int8 per spin, [n_sets][n_temps][n_real][N]: a thread takes
 // kSites consecutive sites of a word-lattice in all 32 realisations, the
 // kSites bytes of each in one access (256 x 30 x 2 x L = 12 to bytes: 17.4 us
@@ -236,6 +316,52 @@ cudaError_t launch_couplings_msc(spin_lattice *h) {
   return cudaGetLastError();
 }
 
+namespace {
+using ResKern = decltype(&msc_res_kernel<3, false, false>);
+
+// Sweeps of a call with the lattices in shared memory (msc_res_kernel): CTAs,
+// threads and shared memory; grid 0 where the phase launches are better.
+struct MscRes {
+  unsigned grid = 0;
+  int threads = 0;
+  size_t smem = 0;
+};
+
+// The rule compares two estimates in us, fitted to calls of 2 to 16 sweeps of
+// 1 to 2048 word-lattices, 3D L = 4 ... 20 and 2D L = 8 ... 94.  Here: start and
+// loading (per word and thread, once per round of CTAs), then a sweep per
+// round of CTAs; the phases: the larger of latency and words, and half the
+// smaller.  Measured, phases against here, 4 and 16 sweeps: 3D L = 6, 512
+// word-lattices x 4 slots, 28 / 116 against 17 / 44; L = 12, 480 word-lattices,
+// 35 / 121 against 27 / 74; L = 16, the same, 46 / 170 against 42 / 115; L = 20, 64
+// word-lattices, 22 / 92 against 85 / 261 (phases).
+MscRes msc_res_plan(const spin_lattice *h, int64_t n_sweeps) {
+  const Geom &g = h->g;
+  MscRes p;
+  const size_t smem = (size_t)(kSlots + (uint32_t)g.dim) * (size_t)g.N * 4;
+  if (n_sweeps < 3 || smem > kResSmem) return p;
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool row = g.L % 8 == 0;
+  const uint32_t quads = (uint32_t)((g.N / 2 + 3) / 4), items = row ? quads : 4 * quads;
+  const uint32_t rounds = (items + kResThreads - 1) / kResThreads;
+  const uint32_t T = (uint32_t)g.n_temps, TB = (T + kSlots - 1) / kSlots, st = (uint32_t)g.n_sets * (uint32_t)(g.n_real / 32);
+  const int threads = std::max(128, (int)(((items + rounds - 1) / rounds + 31) / 32 * 32));  // 128: to load with
+  const double n = (double)n_sweeps, per_sm = std::ceil((double)st * TB / sms), d = g.dim == 3 ? 1.0 : 0.75;
+  const double frac = (double)items / kResThreads;
+  const double sweep = row ? 1.6 + 1.2 * d * frac * std::min(kSlots, T) : 0.6 + 1.75 * d * frac;
+  const double here = 7.0 + 0.17 * (double)smem / 4.0 / threads * per_sm +
+                      n * sweep * std::max(1.0, per_sm * threads / 448.0);
+  const double lat = row ? 2.0 + 1.1 * std::min(kSlots, T) : 3.3;
+  const double words = (row ? 3.35e-6 : 5.3e-6) * d * (double)st * T * (double)g.N;
+  if (here > 0.95 * (3.5 + n * (std::max(lat, words) + 0.5 * std::min(lat, words)))) return p;
+  p.grid = st * TB;
+  p.threads = threads;
+  p.smem = smem;
+  return p;
+}
+}  // namespace
+
 cudaError_t launch_sweeps_msc_ea(spin_lattice *h, const uint32_t *J, int64_t n_sweeps) {
   const Geom &g = h->g;
   const RoundKeys rk = make_round_keys(h->d.seed);
@@ -250,6 +376,20 @@ cudaError_t launch_sweeps_msc_ea(spin_lattice *h, const uint32_t *J, int64_t n_s
                                {{msc_site_phase_kernel<3, false>, msc_phase_kernel<3, false>},
                                 {msc_site_phase_kernel<3, true>, msc_phase_kernel<3, true>}}};
   const Kern kern = kerns[g.dim == 3][pair][row_quads];
+  const MscRes res = msc_res_plan(h, n_sweeps);
+  if (res.grid) {
+    const ResKern res_kerns[2][2][2] = {{{msc_res_kernel<2, false, false>, msc_res_kernel<2, false, true>},
+                                         {msc_res_kernel<2, true, false>, msc_res_kernel<2, true, true>}},
+                                        {{msc_res_kernel<3, false, false>, msc_res_kernel<3, false, true>},
+                                         {msc_res_kernel<3, true, false>, msc_res_kernel<3, true, true>}}};
+    const ResKern kern = res_kerns[g.dim == 3][pair][row_quads];
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
+    for (int64_t k = 0; e == cudaSuccess && k < n_sweeps; k += kResSweeps)
+      e = launch_dependent(kern, dim3(res.grid), dim3(res.threads), res.smem, h->stream, (uint32_t *)h->spins, J, g,
+                           ftb, (const uint32_t *)h->d_thr, rk, (uint32_t)(h->sweeps_done + k),
+                           (uint32_t)std::min<int64_t>(n_sweeps - k, kResSweeps));
+    return e;
+  }
   const int64_t threads = row_quads ? work : 4 * (int64_t)work;  // < 2^30: fewer than 2^27 words
   for (int64_t k = 0; k < n_sweeps; ++k) {
     const uint32_t sweep = (uint32_t)(h->sweeps_done + k);
