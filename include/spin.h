@@ -35,7 +35,9 @@
  * ferromagnets, for small lattices with the acceptance masks of the sweeps
  * ahead, at most about 32 MB or two sweeps' masks; long Heisenberg calls),
  * with, for the resident 3D Heisenberg sweeps, one counter per CTA; all are
- * freed by spin_destroy.
+ * freed by spin_destroy.  A call that needs a longer working buffer makes one;
+ * the old one is freed at once, or by spin_destroy if a call inside a stream
+ * capture has used it, so that the captured graph can still be replayed.
  *
  * Errors: every entry point returns 0 (SPIN_OK) or a negative SPIN_E* code
  * and never throws.  Work is asynchronous on the handle's stream; kernel

@@ -142,6 +142,7 @@ void free_workspaces(spin_lattice *h) {
                   h->d_scratch64, h->d_err, h->d_pingpong, h->d_ctr, h->d_bar,  h->d_escr, h->d_res_flags};
   for (void *b : bufs)
     if (b) cudaFree(b);
+  for (int k = 0; k < h->n_retired; ++k) cudaFree(h->d_retired[k]);
 }
 
 cudaError_t do_sweeps(spin_lattice *h, const void *J, int64_t n) {
@@ -161,6 +162,36 @@ bool ea(const spin_lattice *h) { return h->d.model == SPIN_EA; }
 }  // namespace
 
 namespace spin {
+cudaError_t working_buffer(spin_lattice *h, size_t bytes, bool in_capture) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (!h->d_pingpong || h->pingpong_bytes < bytes) {
+    if (capturing && !in_capture) return cudaErrorStreamCaptureUnsupported;
+    const bool keep = h->d_pingpong && (h->pingpong_captured || capturing);
+    if (keep && h->n_retired == (int)(sizeof h->d_retired / sizeof h->d_retired[0])) return cudaErrorMemoryAllocation;
+    void *p = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess && h->d_pingpong && !keep) {  // once more in the place of the old one
+      cudaGetLastError();
+      cudaFree(h->d_pingpong);
+      h->d_pingpong = nullptr;
+      h->pingpong_bytes = 0;
+      e = cudaMalloc(&p, bytes);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
+    if (keep) h->d_retired[h->n_retired++] = h->d_pingpong;
+    else if (h->d_pingpong) cudaFree(h->d_pingpong);
+    h->d_pingpong = p;
+    h->pingpong_bytes = bytes;
+    h->pingpong_captured = false;
+  }
+  if (capturing) h->pingpong_captured = true;
+  return cudaSuccess;
+}
+
 int upload_thresholds_for_batch(spin_lattice *h, const double *betas) { return upload_thresholds(h, betas); }
 int upload_pt_tables_for_batch(spin_lattice *h, const double *betas) {
   if (!betas) return SPIN_EINVAL;

@@ -160,13 +160,8 @@ int fused2d_strip_height(int L, int n_lat) {
 cudaError_t launch_fused2d_i8(spin_lattice *h, int64_t n_sweeps) {
   const int L = h->g.L;
   const size_t bytes = (size_t)h->n_lat * (size_t)h->g.N;
-  if (!h->d_pingpong || h->pingpong_bytes < bytes) {
-    if (h->d_pingpong) cudaFree(h->d_pingpong);
-    h->d_pingpong = nullptr;
-    cudaError_t e = cudaMalloc(&h->d_pingpong, bytes);
-    if (e != cudaSuccess) return e;
-    h->pingpong_bytes = bytes;
-  }
+  const cudaError_t made = working_buffer(h, bytes, true);
+  if (made != cudaSuccess) return made;
   const int H = fused2d_strip_height(L, (int)h->n_lat);
   const int threads = L / 16;
   const size_t smem = 3 * (size_t)L;

@@ -324,16 +324,11 @@ constexpr int64_t kSplitMinSweeps = 4;
 cudaError_t sweeps_heis_split(spin_lattice *h, int64_t n_sweeps) {
   const int64_t total = h->n_lat * h->g.N;
   const size_t bytes = (size_t)total * 16;
-  if (!h->d_pingpong || h->pingpong_bytes < bytes) {
-    if (h->d_pingpong) cudaFree(h->d_pingpong);
-    h->d_pingpong = nullptr;
-    cudaError_t e = cudaMalloc(&h->d_pingpong, bytes);
-    if (e != cudaSuccess) return e;
-    h->pingpong_bytes = bytes;
-  }
+  cudaError_t e = working_buffer(h, bytes, true);
+  if (e != cudaSuccess) return e;
   float4 *S = (float4 *)h->d_pingpong;
   heis_to_split_kernel<<<capped_grid(total), 256, 0, h->stream>>>((const float4 *)h->spins, S, h->g, total);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const RoundKeys rk = make_round_keys(h->d.seed);
   const uint32_t half = (uint32_t)(total / 2);

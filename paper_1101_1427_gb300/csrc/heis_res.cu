@@ -308,13 +308,8 @@ bool heis_resident_plan(const spin_lattice *h, HeisResPlan *plan) {
 cudaError_t launch_sweeps_heis_resident(spin_lattice *h, const HeisResPlan &plan, int64_t sweep0, int64_t n_sweeps) {
   const int64_t total = h->n_lat * h->g.N;
   const size_t bytes = (size_t)total * 16;
-  if (!h->d_pingpong || h->pingpong_bytes < bytes) {
-    if (h->d_pingpong) cudaFree(h->d_pingpong);
-    h->d_pingpong = nullptr;
-    cudaError_t e = cudaMalloc(&h->d_pingpong, bytes);
-    if (e != cudaSuccess) return e;
-    h->pingpong_bytes = bytes;
-  }
+  const cudaError_t made = working_buffer(h, bytes, true);
+  if (made != cudaSuccess) return made;
   if (!h->d_res_flags || h->res_flags_n < plan.grid || h->res_base > 0x7fffffffu) {
     if (h->d_res_flags) cudaFree(h->d_res_flags);
     h->d_res_flags = nullptr;

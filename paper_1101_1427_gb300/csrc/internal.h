@@ -59,6 +59,10 @@ struct spin_lattice {
   int *d_err;            // device error word
   void *d_pingpong;      // working buffer of the sweeps that need one (lazy)
   size_t pingpong_bytes;
+  bool pingpong_captured;   // a captured call has used it: it outlives its replacement
+  void *d_retired[8];       // replaced working buffers that captured calls used
+  int n_retired;
+  bool res_smem_set;        // the resident planes kernel may ask for its shared memory on this device
   int tape_half;         // half of the tape in it that was drawn last (planes_res.cu)
   // batched launches (options set with spin_set_batch_options)
   uint64_t batch_timeout_ns;  // bound on every team-barrier wait (0: 2 s)
@@ -80,6 +84,14 @@ struct spin_lattice {
 };
 
 namespace spin {
+
+// api.cu: the handle's working buffer, made or made longer where it holds fewer
+// than `bytes`; with in_capture false never inside a stream capture.  A buffer
+// that a captured call has used is kept until spin_destroy when a longer one
+// takes its place, since the graph may be replayed at any time; a handle
+// lengthens its buffer a few times at most (the masks of planes_res.cu four
+// times, the planes and the fused pass once each).
+cudaError_t working_buffer(spin_lattice *h, size_t bytes, bool in_capture);
 
 // ising_i8.cu
 cudaError_t launch_init_i8(spin_lattice *h);

@@ -383,18 +383,7 @@ bool planes_ready(spin_lattice *h, int64_t n_sweeps) {
   if (resident(h) && planes_res_reserve(h, n_sweeps)) return true;
   if (h->variant == 3) return false;
   const size_t bytes = (size_t)h->n_lat * planes_lattice_bytes(h);
-  if (h->d_pingpong && h->pingpong_bytes >= bytes) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-  void *p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (h->d_pingpong) cudaFree(h->d_pingpong);
-  h->d_pingpong = p;
-  h->pingpong_bytes = bytes;
-  return true;
+  return working_buffer(h, bytes, false) == cudaSuccess;
 }
 
 int planes_run(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,

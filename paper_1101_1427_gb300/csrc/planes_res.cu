@@ -339,20 +339,11 @@ bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
   while (sweeps < n_sweeps && sweeps < kResMaxSweeps) sweeps *= 2;
   if (sweeps > 1 && (size_t)sweeps * per > kTapeMax) sweeps = (int64_t)(kTapeMax / per) + 1;
   const size_t need = planes_pair_bytes(h) + 2 * (size_t)(sweeps + kTapeExtra) * per;
-  if (h->d_pingpong && h->pingpong_bytes >= need) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-  void *p = nullptr;
-  if (cudaMalloc(&p, need) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (h->d_pingpong) cudaFree(h->d_pingpong);
-  h->d_pingpong = p;
-  h->pingpong_bytes = need;
-  cudaFuncSetAttribute(planes_res_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSpread);
-  cudaFuncSetAttribute(planes_res_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSpread);
-  return true;
+  if (working_buffer(h, need, false) != cudaSuccess) return false;
+  if (!h->res_smem_set)
+    h->res_smem_set = cudaFuncSetAttribute(m.dim == 3 ? planes_res_kernel<3> : planes_res_kernel<2>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, kResSpread) == cudaSuccess;
+  return h->res_smem_set;
 }
 
 // The tape for the next sweeps; returns how many it covers (at most n).
