@@ -95,6 +95,11 @@ template <int kC>
 __device__ __forceinline__ void heis_block_partials(const float4 *__restrict__ sl, uint32_t L, const FastDiv &fL,
                                                     int dim, uint32_t N, uint32_t b, uint32_t nb,
                                                     double *__restrict__ out4) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  // rank 0's shared memory may be written once that CTA is known to run: every
+  // CTA says so here and waits for it before the store, behind its sites
+  if (kC > 1) cl.barrier_arrive();
   Sum3 ex, ey, ez, sx, sy, sz;
   float norm2 = 0.0f, count = 0.0f;
   const uint64_t first = b * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)nb * blockDim.x;
@@ -165,8 +170,7 @@ __device__ __forceinline__ void heis_block_partials(const float4 *__restrict__ s
   }
   // the CTAs of the cluster leave their sums in rank 0's shared memory
   __shared__ double all[kC][4];
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_wait();
   if (threadIdx.x < 4) {
     double acc = 0.0;
     for (int k = 0; k < (int)(blockDim.x >> 5); ++k) acc += red[threadIdx.x][k];
