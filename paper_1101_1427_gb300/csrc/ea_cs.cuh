@@ -79,11 +79,10 @@ __device__ __forceinline__ void ea_after(const Flip &f, uint32_t &a0, uint32_t &
   a2 = (f.F & v2) | (~f.F & f.b2);
 }
 
-__device__ __forceinline__ uint4 ldv4(const uint32_t *p) {
-  uint4 v;
-  asm("ld.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
+// Four consecutive words, 16-byte aligned, in global or shared memory: a plain
+// load, which the compiler keeps in order with stores, barriers and
+// griddep_wait().
+__device__ __forceinline__ uint4 ldv4(const uint32_t *p) { return *reinterpret_cast<const uint4 *>(p); }
 
 // ---------------------------------------------------------------- 2D
 // The square lattice (the paper's own Sec. 5 benchmark is 2D): four bonds,
