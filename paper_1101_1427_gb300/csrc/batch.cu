@@ -929,6 +929,13 @@ static int next_team(const BatchUnit &U, int P, int cap) {
   return o > 1 ? (W + o - 2) / (o - 1) : cap + 1;
 }
 
+// The fewest CTAs of a unit (EA: each CTA owns at most 64 word-lattices).
+static int least_team(const BatchUnit &U) {
+  int p = 1;
+  while (U.kind == 0 && U.n_sets * ((U.n_T + p - 1) / p) > 64) ++p;
+  return p;
+}
+
 // Distributes `grid` CTAs over the units: every unit gets its minimum (EA:
 // at most 64 owned word-lattices per CTA; Ising: 1), then the unit with the
 // longest time gets its next larger team, as long as one fits, up to each
@@ -939,17 +946,12 @@ static int assign_teams(BatchUnit *units, int n, int grid, double ising_scale, d
   std::vector<double> time(n);
   int used = 0;
   for (int u = 0; u < n; ++u) {
+    P[u] = least_team(units[u]);
     if (units[u].kind == 0) {
-      // each CTA owns at most 64 word-lattices (set, slot)
-      int p = 1;
-      while (units[u].n_sets * ((units[u].n_T + p - 1) / p) > 64) ++p;
-      P[u] = p;
       cap[u] = units[u].n_T * units[u].n_sets;  // one word-lattice per CTA at most
     } else if (units[u].kind == 1) {
-      P[u] = 1;
       cap[u] = std::max(1, units[u].L / 8);
     } else {  // at least 256 blocks (one per thread) per CTA
-      P[u] = 1;
       cap[u] = std::max(1, units[u].L * (units[u].L / 256) / 256);
     }
     used += P[u];
@@ -1133,14 +1135,18 @@ constexpr int kResidentSmem = 212 * 1024;
 // word-lattices are small enough that most of a CTA's fit (32 KB at L = 20),
 // and whose units are large enough for three CTAs and more each (a unit takes
 // whole CTAs) but have no more CTAs than slots.  1024 x 32 x 2 of L = 16, 8
-// sweeps with E, M, Q and an exchange after each: 523 -> 485 us.
+// sweeps with E, M, Q and an exchange after each: 523 -> 485 us.  A batch whose
+// least teams need more CTAs than there are SMs only fits two to an SM.
 static bool resident_preferred(const BatchParams &prm, int sms) {
   double total = 0.0;
+  int least = 0;
   for (int u = 0; u < prm.n_units; ++u) {
     const BatchUnit &U = prm.units[u];
     if (U.kind != 0 || U.N > 8192u) return false;
     total += (double)U.n_sets * U.n_T * U.N;
+    least += least_team(U);
   }
+  if (least > sms) return false;
   for (int u = 0; u < prm.n_units; ++u) {
     const BatchUnit &U = prm.units[u];
     const double share = sms * (double)U.n_sets * U.n_T * U.N / total;
