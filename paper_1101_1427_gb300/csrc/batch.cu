@@ -1218,14 +1218,16 @@ extern "C" int spin_batch_run(const spin_batch_item *items, int n_items, int64_t
     rc = ensure_batch_ws(h);
     if (rc) return rc;
   }
-  static bool attr = false;
-  if (!attr) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return SPIN_ECUDA;
+  static OncePerDevice limits;
+  if (!limits.done(dev)) {
     if (cudaFuncSetAttribute(batch_kernel<kResidentThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kResidentSmem) != cudaSuccess ||
         cudaFuncSetAttribute(batch_kernel<kPairThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, 12288 * 4) !=
             cudaSuccess)
       return SPIN_ECUDA;
-    attr = true;
+    limits.mark(dev);
   }
   spin_lattice *h0 = items[0].lat;
   static BatchCtl ctl;
@@ -1266,10 +1268,8 @@ extern "C" int spin_batch_run(const spin_batch_item *items, int n_items, int64_t
   const auto it = g_tuned.find(sig);
   const int asked = h0->batch_ctas_per_sm > 0 ? h0->batch_ctas_per_sm : it != g_tuned.end() ? it->second.ctas_per_sm : 0;
   // co-resident grid
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return SPIN_ECUDA;
+  int sms = 0, per_sm = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SPIN_ECUDA;
   prm.smem_words = asked <= 1 && resident_preferred(prm, sms) ? kResidentSmem / 4 : prm.staged_words;
   if (batch_occupancy(prm, &per_sm) != cudaSuccess || per_sm < 1) return SPIN_ECUDA;
   // Ising series rows are accumulated with atomics: the prologue zeroes the

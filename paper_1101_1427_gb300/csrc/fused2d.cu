@@ -165,10 +165,12 @@ cudaError_t launch_fused2d_i8(spin_lattice *h, int64_t n_sweeps) {
   const int H = fused2d_strip_height(L, (int)h->n_lat);
   const int threads = L / 16;
   const size_t smem = 3 * (size_t)L;
-  static bool attr_set = false;
-  if (!attr_set) {
+  static OncePerDevice limit;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!limit.done(dev)) {
     cudaFuncSetAttribute(fused2d_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * 16384);
-    attr_set = true;
+    limit.mark(dev);
   }
   dim3 grid((unsigned)((L + H - 1) / H), (unsigned)h->n_lat);
   const RoundKeys rk = make_round_keys(h->d.seed);

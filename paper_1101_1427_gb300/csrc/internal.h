@@ -9,6 +9,7 @@
 
 #include "../../include/spin.h"
 #include "common.cuh"
+#include "per_device.h"
 #include "pt.cuh"
 
 // NVTX range over one ABI call, so that a profiler's timeline shows which
