@@ -446,7 +446,8 @@ int spin_set_update_order(spin_lattice *lat, int32_t order, int32_t tile, int32_
  * double-checkerboard handle whose tile edge was left open (tile 0), every
  * supported tile edge (each gives its own chain, Sec. 3.2).  The fastest
  * choice is set on the handle and cached per (model, layout, dim, L,
- * lattices, order, hits, n_sweeps) for later handles of that shape.  Trials
+ * lattices, order, hits, n_sweeps) for later handles of that shape (and, where
+ * the tuner does not choose the variant, of the same variant).  Trials
  * run on the handle's buffer after a backup copy (allocated and freed by
  * this call); spins and counters are restored, so results do not depend on
  * whether or when the tuner ran.  best_variant, best_tile (host, optional)

@@ -248,6 +248,7 @@ int spin_init(spin_lattice **out, const spin_desc *desc, void *spins, void *coup
   h->variant = i8 && resident_supported(desc->dim, desc->L)
                    ? 3
                    : (i8_2d && coded_i8_supported(h) ? 4 : (i8_2d && fused2d_supported(desc->L) ? 1 : 0));
+  h->default_variant = h->variant;
   const int nt = desc->n_temps;
   bool ok = cudaMalloc(&h->d_thr, 16 * (size_t)nt) == cudaSuccess &&
             cudaMalloc(&h->d_pt_off, 4 * (size_t)nt) == cudaSuccess &&

@@ -40,6 +40,7 @@ struct spin_lattice {
   int64_t sweeps_done;
   int64_t pt_steps_done;
   int variant;           // int8 sweep: 0 phases, 1 fused, 3 resident, 4 coded
+  int default_variant;   // as spin_init chose it
   int auto_form;         // no variant was asked for: longer int8 calls may take the bit planes
   int msc_width;         // EA coded: realisations sharing one uniform (32 or 64)
   int order;             // spin_update_order

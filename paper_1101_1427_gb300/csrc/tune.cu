@@ -21,15 +21,16 @@ bool dcb_supported(const spin_lattice *h, int tile);
 
 namespace {
 
-// (model, layout, dim, L, lattices, order, hits, requested tile (0: open), call length)
-using Key = std::tuple<int, int, int, int, int64_t, int, int, int, int64_t>;
+// (model, layout, dim, L, lattices, order, hits, requested tile (0: open), call
+// length, form kept (-1: the tuner chooses it))
+using Key = std::tuple<int, int, int, int, int64_t, int, int, int, int64_t, int>;
 std::mutex g_tune_mutex;
 std::map<Key, std::pair<int, int>> g_tuned;  // shape -> (variant, tile)
 
-Key key_of(const spin_lattice *h, int64_t n_sweeps) {
+Key key_of(const spin_lattice *h, int64_t n_sweeps, int form) {
   const bool dcb = h->order != SPIN_ORDER_CHECKERBOARD;
   return Key(h->d.model, h->d.layout, h->d.dim, h->g.L, h->n_lat, h->order, dcb ? h->order_hits : 0,
-             dcb ? h->order_tile : 0, n_sweeps);
+             dcb ? h->order_tile : 0, n_sweeps, form);
 }
 
 int64_t spin_bytes(const spin_lattice *h) {
@@ -70,12 +71,17 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
       if (spin_set_variant(h, v) == SPIN_OK) cand.emplace_back(v, h->order_tile);
       apply(start);
     }
-    if (h->auto_form && spin::planes_wanted(h, n_sweeps, 0)) cand.push_back(start);
+    const std::pair<int, int> unset(h->default_variant + kAuto, h->order_tile);
+    apply(unset);
+    if (spin::planes_wanted(h, n_sweeps, 0)) cand.push_back(unset);
+    apply(start);
   } else {
     cand.push_back(start);
   }
   if (cand.empty()) return SPIN_EINVAL;
-  const Key key = key_of(h, n_sweeps);
+  // (a double-checkerboard or Heisenberg handle keeps its variant, which may be
+  // the fast-math one: choices are not shared between variants there)
+  const Key key = key_of(h, n_sweeps, i8_ferro && !dcb ? -1 : start.first);
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tuned.find(key);
