@@ -32,8 +32,8 @@
  * (threshold tables, reduction partials, an error word), allocated by
  * spin_init, and one working buffer allocated by the first sweep call that
  * needs it (the fused 2D int8 pass; the bit planes of longer calls on int8
- * ferromagnets, for small lattices with the acceptance masks of the sweeps
- * ahead, at most about 32 MB or two sweeps' masks; long Heisenberg calls),
+ * ferromagnets, for small lattices twice and with the acceptance masks of the
+ * sweeps ahead, at most 32 MB of these; long Heisenberg calls),
  * with, for the resident 3D Heisenberg sweeps, one counter per CTA; all are
  * freed by spin_destroy.  A call that needs a longer working buffer makes one;
  * the old one is freed at once, or by spin_destroy if a call inside a stream

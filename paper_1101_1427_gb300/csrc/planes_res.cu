@@ -15,6 +15,8 @@
 // planes instead of its own where the exchange is accepted.  One L = 64, 1000
 // sweeps with E and M after each 1335 -> 265 us; 20 x L = 64, 100 sweeps and 10
 // exchanges 181 -> 55 us; 20 x 3D L = 16, 256 sweeps 234 -> 63 us.
+#include <algorithm>
+
 #include "internal.h"
 #include "planes.cuh"
 
@@ -111,7 +113,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
                                                                  int n_sweeps, ResSeries ser, PtTables pt,
                                                                  RoundKeys rk) {
   constexpr int kT = kDim;
-  constexpr int kAhead = 8;                         // phases fetched ahead (even, at most 2 kTapeExtra)
+  constexpr int kAhead = 8;                         // phases fetched ahead (even)
   __shared__ __align__(16) uint32_t sw[2 * kResThreads];  // [2 colours][words]
   __shared__ int cnt[kResRows + 1][2];
   __shared__ bool exchanged;
@@ -158,12 +160,13 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
   const size_t chunk0 = (size_t)lat * (size_t)(N / 8);  // the lattice's first 8-byte chunk
   griddep_wait();
   griddep_release();
-  // the tape: phase p at ((p n_lat + lat) kT + e) words + word; it is longer
-  // than its sweeps by the phases fetched ahead
+  // the tape: phase p at ((p n_lat + lat) kT + e) words + word
+  const int phases = 2 * n_sweeps;
   const size_t phase_step = (size_t)n_lat * kT * words;
   const uint32_t *tp = tape + (size_t)lat * kT * words + wd;
   uint32_t mk[kAhead][kT];
-  auto fetch = [&](uint32_t (&v)[kT]) {  // the next phase's masks
+  auto fetch = [&](uint32_t (&v)[kT], int p) {  // phase p's masks, one phase after the other
+    if (p >= phases) return;
 #pragma unroll
     for (int e = 0; e < kT; ++e) v[e] = tp[e * words];
     tp += phase_step;
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
       }
     }
 #pragma unroll
-    for (int d = 0; d < kAhead; ++d) fetch(mk[d]);
+    for (int d = 0; d < kAhead; ++d) fetch(mk[d], d);
     __syncthreads();
     if (mine) s[0] = sw[wd], s[1] = sw[words + wd];
   } else {
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
     const uint32_t *own = src + (size_t)lat * 2 * words + wd, *other = src + (size_t)partner * 2 * words + wd;
     const uint32_t w0 = own[0], w1 = own[words], x0 = other[0], x1 = other[words];
 #pragma unroll
-    for (int d = 0; d < kAhead; ++d) fetch(mk[d]);
+    for (int d = 0; d < kAhead; ++d) fetch(mk[d], d);
     if (threadIdx.x == 0) {
       bool acc = false;
       if (partner != lat) {
@@ -216,7 +219,6 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
     }
     __syncthreads();
   }
-  const int phases = 2 * n_sweeps;
   int next = ser.first - 1, rows = 0, written = 0;  // next: sweep (0-based) of the next measurement
   auto write_rows = [&]() {  // rows counted since the last write (the caller has a barrier before)
     if ((int)threadIdx.x < rows) {
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
       const uint32_t v = s[c] ^ (plane_flips<kDim>(s[c], n, 0, mk[d][0], mk[d][1], mk[d][kT - 1]) & valid);
       s[c] = v;
       if (mine) sw[c * words + wd] = v;
-      fetch(mk[d]);
+      fetch(mk[d], p + kAhead);
       if (c == 1) {
         const int sweep = p >> 1;
         const bool row_now = (ser.E || ser.M) && sweep == next, last_now = ser.E_last && sweep == n_sweeps - 1;
@@ -295,8 +297,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
   }
 }
 
-constexpr size_t kTapeMax = 16u << 20;  // bytes of one half of the tape, about
-constexpr int kTapeExtra = 4;           // sweeps by which a half is longer than what it holds
+constexpr size_t kTapeMax = 16u << 20;  // bytes of one half of the tape, at most
 // Dynamic shared memory asked for (not used) to place CTAs.  The few CTAs of
 // the sweeps spread over the SMs: a launch that starts while the masks' CTAs
 // drain would otherwise find its places on a few SMs (20 x L = 64, 256 sweeps:
@@ -337,8 +338,10 @@ bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
   // (calls of growing length make few buffers: a power of two, at least 512)
   int64_t sweeps = kResMinTape;
   while (sweeps < n_sweeps && sweeps < kResMaxSweeps) sweeps *= 2;
-  if (sweeps > 1 && (size_t)sweeps * per > kTapeMax) sweeps = (int64_t)(kTapeMax / per) + 1;
-  const size_t need = planes_pair_bytes(h) + 2 * (size_t)(sweeps + kTapeExtra) * per;
+  // (whole groups of sweeps that are drawn together)
+  sweeps = std::min(sweeps, (int64_t)(kTapeMax / per) / kTapeSweeps * kTapeSweeps);
+  if (sweeps == 0) return false;
+  const size_t need = planes_pair_bytes(h) + 2 * (size_t)sweeps * per;
   if (working_buffer(h, need, false) != cudaSuccess) return false;
   if (!h->res_smem_set)
     h->res_smem_set = cudaFuncSetAttribute(m.dim == 3 ? planes_res_kernel<3> : planes_res_kernel<2>,
@@ -349,9 +352,8 @@ bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
 // The tape for the next sweeps; returns how many it covers (at most n).
 int64_t planes_res_draw(spin_lattice *h, int64_t sweep0, int64_t n, cudaError_t *err) {
   const Planes m = make_planes(h->g.dim, h->g.L);
-  int64_t cover = (int64_t)(tape_half_bytes(h) / tape_sweep_bytes(h, m)) - kTapeExtra;
-  if (cover > n) cover = n;
-  if (cover > kResMaxSweeps) cover = kResMaxSweeps;
+  int64_t cover = (int64_t)(tape_half_bytes(h) / tape_sweep_bytes(h, m)) / kTapeSweeps * kTapeSweeps;
+  cover = std::min(std::min(cover, kResMaxSweeps), n);
   h->tape_half ^= 1;
   const int64_t groups = (cover + kTapeSweeps - 1) / kTapeSweeps;
   const int64_t threads = groups * 2 * h->n_lat * m.blocks;  // < 2^31: 16 bytes of tape each
