@@ -298,13 +298,34 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
 }
 
 constexpr size_t kTapeMax = 16u << 20;  // bytes of one half of the tape, at most
-// Dynamic shared memory asked for (not used) to place CTAs.  The few CTAs of
-// the sweeps spread over the SMs: a launch that starts while the masks' CTAs
-// drain would otherwise find its places on a few SMs (20 x L = 64, 256 sweeps:
-// 145 us against 55 for one lattice).  And beside one of them there is room
-// for one CTA of the next masks only, which may run at the same time.
 constexpr int kResSpread = 200 * 1024;
 constexpr int kTapeSpread = 20 * 1024;
+
+// Dynamic shared memory asked for (not used) to place CTAs: the sweeps' and the
+// masks'.  The few CTAs of the sweeps spread over the SMs: a launch that starts
+// while the masks' CTAs drain would otherwise find its places on a few SMs (20
+// x L = 64, 256 sweeps: 145 us against 55 for one lattice), and beside one of
+// them there is room for one CTA of the next masks only, which may run at the
+// same time.  From more than half as many lattices as SMs on, a CTA that asks
+// for most of an SM waits until it is empty of masks (us per call of 8 / 16 / 32
+// / 100 sweeps, asking for 200 KB / lattices per SM, against here: 152 x 2D L =
+// 64 9.3 / 33 / 35 / 61 and 9.2 / 12 / 18 / 56, 304 x 2D L = 16 18 / 21 / 30 /
+// 44 and 7 / 7 / 9 / 22, 152 x 2D L = 128 33 / 36 / 80 / 181 and 18 / 33 / 59 /
+// 174): there half of it and no such masks do better, and nothing at all for the
+// CTAs of 256 threads and more, of which few fit anyway.
+struct Places {
+  size_t sweeps, masks;
+};
+Places places(const spin_lattice *h, const Planes &m) {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t per_sm = (h->n_lat + sms - 1) / sms;
+  Places p = {0, kTapeSpread};
+  if (2 * h->n_lat <= sms) p.sweeps = kResSpread;
+  else if (per_sm <= 8 && m.blocks < 64) p = {(size_t)(kResSpread / 2 / per_sm), 0};
+  return p;
+}
+
 constexpr int64_t kResMinTape = 512;
 constexpr int64_t kResMaxSweeps = 4096;  // per launch, so that none runs for long
 
@@ -358,7 +379,7 @@ int64_t planes_res_draw(spin_lattice *h, int64_t sweep0, int64_t n, cudaError_t 
   const int64_t groups = (cover + kTapeSweeps - 1) / kTapeSweeps;
   const int64_t threads = groups * 2 * h->n_lat * m.blocks;  // < 2^31: 16 bytes of tape each
   *err = launch_dependent(m.dim == 3 ? planes_tape_kernel<3> : planes_tape_kernel<2>, dim3(grid_for(threads, 128)),
-                          dim3(128), kTapeSpread, h->stream, tape_of(h), m, h->g, (uint32_t)h->n_lat,
+                          dim3(128), places(h, m).masks, h->stream, tape_of(h), m, h->g, (uint32_t)h->n_lat,
                           make_fastdiv((uint32_t)h->n_lat), make_fastdiv(m.blocks), (const uint32_t *)h->d_thr,
                           make_round_keys(h->d.seed), (uint32_t)sweep0, (uint32_t)cover);
   return cover;
@@ -380,12 +401,8 @@ cudaError_t planes_res_sweeps(spin_lattice *h, int64_t at, int64_t n, int from, 
   s.step = call.step;
   s.accepted = (long long *)call.accepted;
   s.labels = call.labels;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t per_sm = (h->n_lat + sms - 1) / sms;
-  const size_t spread = per_sm <= 8 ? (size_t)(kResSpread / per_sm) : 0;
   return launch_dependent(m.dim == 3 ? planes_res_kernel<3> : planes_res_kernel<2>, dim3((unsigned)h->n_lat),
-                          dim3((4 * m.blocks + 31) / 32 * 32), spread, h->stream,
+                          dim3((4 * m.blocks + 31) / 32 * 32), places(h, m).sweeps, h->stream,
                           (const uint64_t *)(call.bytes_in ? h->spins : nullptr),
                           (uint64_t *)(call.bytes_out ? h->spins : nullptr), (const uint32_t *)(p + (size_t)from * buf),
                           p + (size_t)(from ^ 1) * buf, (const uint32_t *)tape, m, h->g, (int)n, s, pt_tables(h),
