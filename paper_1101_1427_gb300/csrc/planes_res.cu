@@ -16,6 +16,7 @@
 // sweeps with E and M after each 1335 -> 265 us; 20 x L = 64, 100 sweeps and 10
 // exchanges 181 -> 55 us; 20 x 3D L = 16, 256 sweeps 234 -> 63 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "planes.cuh"
@@ -165,8 +166,8 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
   const size_t phase_step = (size_t)n_lat * kT * words;
   const uint32_t *tp = tape + (size_t)lat * kT * words + wd;
   uint32_t mk[kAhead][kT];
-  auto fetch = [&](uint32_t (&v)[kT], int p) {  // phase p's masks, one phase after the other
-    if (p >= phases) return;
+  auto fetch = [&](uint32_t (&v)[kT], bool there = true) {  // the next phase's masks, if there is one
+    if (!there) return;
 #pragma unroll
     for (int e = 0; e < kT; ++e) v[e] = tp[e * words];
     tp += phase_step;
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
       }
     }
 #pragma unroll
-    for (int d = 0; d < kAhead; ++d) fetch(mk[d], d);
+    for (int d = 0; d < kAhead; ++d) fetch(mk[d], d < phases);
     __syncthreads();
     if (mine) s[0] = sw[wd], s[1] = sw[words + wd];
   } else {
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
     const uint32_t *own = src + (size_t)lat * 2 * words + wd, *other = src + (size_t)partner * 2 * words + wd;
     const uint32_t w0 = own[0], w1 = own[words], x0 = other[0], x1 = other[words];
 #pragma unroll
-    for (int d = 0; d < kAhead; ++d) fetch(mk[d], d);
+    for (int d = 0; d < kAhead; ++d) fetch(mk[d], d < phases);
     if (threadIdx.x == 0) {
       bool acc = false;
       if (partner != lat) {
@@ -231,11 +232,13 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
     rows = 0;
     __syncthreads();
   };
-  for (int base = 0; base < phases; base += kAhead) {
+  // kAhead phases from `base` on; kLast: the last ones, which fetch no more
+  auto run = [&](int base, auto last_phases) {
+    constexpr bool kLast = decltype(last_phases)::value;
 #pragma unroll
     for (int d = 0; d < kAhead; ++d) {
       const int p = base + d;
-      if (p >= phases) break;  // (after a whole sweep: phases is even)
+      if (kLast && p >= phases) break;  // (after a whole sweep: phases is even)
       const int c = d & 1;
       const uint32_t *O = sw + (c ^ 1) * words;
       const uint32_t o = s[c ^ 1], km = O[il], kp = O[ir];
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
       const uint32_t v = s[c] ^ (plane_flips<kDim>(s[c], n, 0, mk[d][0], mk[d][1], mk[d][kT - 1]) & valid);
       s[c] = v;
       if (mine) sw[c * words + wd] = v;
-      fetch(mk[d], p + kAhead);
+      fetch(mk[d], !kLast || p + kAhead < phases);
       if (c == 1) {
         const int sweep = p >> 1;
         const bool row_now = (ser.E || ser.M) && sweep == next, last_now = ser.E_last && sweep == n_sweeps - 1;
@@ -281,7 +284,11 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
         __syncthreads();
       }
     }
-  }
+  };
+  int base = 0;
+  if (phases > 8 * kAhead)  // (short launches stay with one copy of the code: 20 x L = 64 tempering 53 against 56 us)
+    for (; base + 2 * kAhead <= phases; base += kAhead) run(base, std::false_type());
+  for (; base < phases; base += kAhead) run(base, std::true_type());
   if (rows) write_rows();
   if (ser.E_last && threadIdx.x == 0) ser.E_last[lat] = 2ll * cnt[kResRows][0] - kDim * N;
   if (bytes_out) {
