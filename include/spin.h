@@ -344,8 +344,11 @@ int spin_set_counters(spin_lattice *lat, int64_t sweeps_done, int64_t pt_steps_d
  * results.  3D int8 ferromagnet: 0 = colour phases, 3 = resident (default
  * for L % 8 == 0, L <= 24), identical results.  A handle whose variant was
  * never set takes the bit planes for every other L % 8 == 0 too, in two and
- * three dimensions, in calls of at least 2 sweeps (4 where the fused pass is
- * its default); where no working buffer can be had (no memory, or inside a
+ * three dimensions, in calls long enough to win back the conversions (2 to 16
+ * sweeps by the number of sites; not at all for 2D lattices with fewer than
+ * 550000 sites in all that have no fused pass), and instead of resident where
+ * there are too many lattices from L = 80 (2D) or 24 (3D) on; where no working
+ * buffer can be had (no memory, or inside a
  * stream capture before an uncaptured call made it) it takes its variant.  Heisenberg: 0 = the full-accuracy FP32
  * library functions (default), 2 = the paper's "fast_math" mode (Sec. 4):
  * rho = sqrt(1 - z^2) from the hardware reciprocal square root, sin and cos

@@ -298,8 +298,9 @@ int spin_sweep(spin_lattice *h, const void *couplings, const double *betas, int6
     return SPIN_EINVAL;  // whole compound moves only, and a tile edge chosen
   int rc = upload_thresholds(h, betas);
   if (rc) return rc;
-  if (planes_wanted(h, n_sweeps, 0) && planes_ready(h, n_sweeps))
-    return planes_run(h, betas, n_sweeps, 0, 0, nullptr, nullptr, nullptr, nullptr);
+  const PlanesForm planes = planes_ready(h, planes_form(h, n_sweeps, 0), n_sweeps);
+  if (planes != PlanesForm::none)
+    return planes_run(h, planes, betas, n_sweeps, 0, 0, nullptr, nullptr, nullptr, nullptr);
   cudaError_t e = h->order != SPIN_ORDER_CHECKERBOARD ? launch_sweeps_dcb(h, n_sweeps)
                                                       : do_sweeps(h, ea(h) ? couplings : nullptr, n_sweeps);
   if (e != cudaSuccess) return SPIN_ECUDA;
@@ -347,11 +348,14 @@ int spin_run(spin_lattice *h, const void *couplings, const double *betas, int64_
   if (!h || n_sweeps < 0) return SPIN_EINVAL;
   if (pt_every > 0 && h->d.model == SPIN_HEISENBERG) return SPIN_EINVAL;
   const bool measuring = measure_every > 0 && (E_series || M_series || Q_series || Ef_series || Mf_series);
-  if (!Q_series && !Ef_series && !Mf_series && planes_wanted(h, n_sweeps, pt_every)) {
+  const PlanesForm wanted =
+      Q_series || Ef_series || Mf_series ? PlanesForm::none : planes_form(h, n_sweeps, pt_every);
+  if (wanted != PlanesForm::none) {
     const int rc = upload_thresholds(h, betas);
     if (rc) return rc;
-    if (planes_ready(h, n_sweeps))
-      return planes_run(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
+    const PlanesForm planes = planes_ready(h, wanted, n_sweeps);
+    if (planes != PlanesForm::none)
+      return planes_run(h, planes, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
   }
   int64_t done = 0, k_meas = 0;
   // small int8 ferromagnets: the resident kernel measures E and M itself,

@@ -172,12 +172,15 @@ inline PtTables pt_tables(const spin_lattice *h) {
 bool planes_supported(const spin_lattice *h);
 size_t planes_lattice_bytes(const spin_lattice *h);
 cudaError_t planes_measure(spin_lattice *h, int64_t *E, int64_t *M);
-// whether a call of n sweeps takes them (ising_i8.cu)
-bool planes_wanted(const spin_lattice *h, int64_t n_sweeps, int32_t pt_every);
-// makes the buffers ready; false: no memory, or a capture that must not allocate
-bool planes_ready(spin_lattice *h, int64_t n_sweeps);
+// the form that serves a call of n sweeps best: none (bytes), a launch per colour
+// phase, or one CTA per lattice with the masks drawn ahead
+enum class PlanesForm { none, phases, resident };
+PlanesForm planes_form(const spin_lattice *h, int64_t n_sweeps, int32_t pt_every);
+// makes the buffers ready; what can run in the place of that form (none: no
+// memory, or a capture that must not allocate)
+PlanesForm planes_ready(spin_lattice *h, PlanesForm form, int64_t n_sweeps);
 // the call (SPIN_* status), spin_run without Q; counters advanced
-int planes_run(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
+int planes_run(spin_lattice *h, PlanesForm form, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
                int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels);
 
 // planes_res.cu: the same for lattices small enough for one CTA each
@@ -192,6 +195,7 @@ struct PlanesResCall {
   bool bytes_in, bytes_out;  // from or to the caller's bytes instead of the planes
 };
 bool planes_res_supported(const spin_lattice *h);
+int64_t planes_res_tape_sweeps(const spin_lattice *h);  // sweeps of masks that are drawn together at most
 bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps);
 int64_t planes_res_draw(spin_lattice *h, int64_t sweep0, int64_t n, cudaError_t *err);
 cudaError_t planes_res_sweeps(spin_lattice *h, int64_t at, int64_t n, int from, const PlanesResCall &call);

@@ -421,28 +421,6 @@ cudaError_t launch_couplings_i8(spin_lattice *h) {
 
 cudaError_t launch_fused2d_i8(spin_lattice *h, int64_t n_sweeps);  // fused2d.cu
 bool fused2d_supported(int L);                                     // fused2d.cu
-// Bit planes (planes.cu) for calls of at least this many sweeps: the two
-// conversions cost about as much as the planes save in one or two sweeps of
-// the byte kernels, least against the fused pass.
-constexpr int64_t kCodedMinSweeps = 4;   // variant 4, shorter calls take the fused pass
-constexpr int64_t kPlanesMinSweeps = 2;  // against the colour phases
-bool planes_wanted(const spin_lattice *h, int64_t n_sweeps, int32_t pt_every) {
-  if (!planes_supported(h) || h->order != SPIN_ORDER_CHECKERBOARD || n_sweeps < 1) return false;
-  if (h->variant == 4) return n_sweeps >= kCodedMinSweeps;
-  // Small lattices: the launch that draws the masks ahead costs what the
-  // sweeps must win back from the kernel with the lattice as bytes, about
-  // 0.14 us + 0.13 ns per site and sweep, and 12 us per exchange (us per call
-  // of 4 / 8 / 16 / 64 sweeps, bytes against planes: L = 16 5.1 / 5.5 / 8.1 /
-  // 24 against 7.3 / 7.6 / 7.7 / 16, L = 64 5.5 / 8.7 / 14 / 51 against 8.1 /
-  // 8.9 / 10 / 20, L = 128 14 / 25 / 45 / 171 against 8.7 / 9.7 / 12 / 25).
-  if (h->variant == 3)
-    return (double)n_sweeps * (0.14 + 0.00013 * (double)h->g.N) +
-               (pt_every > 0 ? 12.0 * (double)(n_sweeps / pt_every) : 0.0) >=
-           5.5;
-  if (!h->auto_form) return false;
-  return n_sweeps >= (h->variant == 1 ? kCodedMinSweeps : kPlanesMinSweeps);
-}
-
 // Whole lattice in one CTA's shared memory: 16 KB at L = 128 in 2D, 13.5 KB
 // at L = 24 in 3D (at most four chunks per thread, so that each thread's
 // chunk geometry stays in registers).

@@ -259,13 +259,6 @@ cudaError_t planes_sweeps(spin_lattice *h, int64_t n_sweeps) {
   return cudaSuccess;
 }
 
-// One CTA per lattice with the masks drawn ahead (planes_res.cu) for lattices
-// that fit, unless there are so many that one sweep of masks is large (the
-// phases of so many sites fill the GPU anyway).
-bool resident(const spin_lattice *h) {
-  return planes_res_supported(h) && h->n_lat * h->g.N <= ((int64_t)1 << 26);
-}
-
 // Sweeps, measurements and exchanges of a call.  Its first launch takes the
 // caller's bytes and its last one leaves them there; in between the lattices
 // alternate between two buffers of planes.  An exchange is decided and carried
@@ -378,19 +371,108 @@ size_t planes_lattice_bytes(const spin_lattice *h) {
   return (size_t)make_planes(h->g.dim, h->g.L).blocks * 2 * sizeof(uint4);
 }
 
-bool planes_ready(spin_lattice *h, int64_t n_sweeps) {
-  if (h->sweeps_done + n_sweeps > (int64_t)0xFFFFFFFFll) return false;  // (refused by the other paths)
-  if (resident(h) && planes_res_reserve(h, n_sweeps)) return true;
-  if (h->variant == 3) return false;
-  const size_t bytes = (size_t)h->n_lat * planes_lattice_bytes(h);
-  return working_buffer(h, bytes, false) == cudaSuccess;
+namespace {
+int sm_count() {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
 }
 
-int planes_run(spin_lattice *h, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
-               int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels) {
-  // (the same test as planes_ready: what it reserved is what runs)
-  const bool res = resident(h) && planes_res_reserve(h, n_sweeps);
-  if (res) return run_resident(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
+// Whether one CTA per lattice with the masks drawn ahead (planes_res.cu) is the
+// fastest form of long calls, by the number of lattices.  What ends it is the
+// size of the masks: with few sweeps of them in a half of the buffer a call is
+// many short launches.  Us per call of 32 sweeps, here / phases / the kernel
+// with the lattice as bytes, at sweeps per half in brackets: 2D L = 8 x 38912
+// 308 / 2574 / 334 (6), x 65520 635 / 4263 / 558 (4); L = 32 x 9728 273 / 1740 /
+// 330 (6), x 19456 741 / 3303 / 658 (3); L = 64 x 4864 554 / 842 / 673 (3); L = 96
+// x 2432 621 / 727 / 873 (2); L = 128 x 608 242 / 247 / 347 (6), x 1216 558 / 482
+// / 698 (3); 3D L = 16 x 4864 592 / 995 / 815 (2); L = 24 x 304 135 / 170 / 179
+// (7), x 608 386 / 301 / 358 (3); L = 32 x 152 134 / 153 / 417 (8), x 304 286 /
+// 256 / 629 (4).  Two sizes have a byte kernel whose warps are just full and a
+// word per thread of few warps here: 2D L = 16 x 1216 18 / 247 / 15, x 9728 98 /
+// 1765 / 87; 3D L = 8 x 304 15 / 118 / 14 and 40 / 355 / 40 for 100 sweeps, x
+// 2432 66 / 223 / 55.  An exchange costs one launch here and four to five small
+// ones there, which outweighs that up to the large lattices (33 sweeps, one
+// every 8: 2D L = 16 x 9728 138 / 1950 / 216, L = 8 x 65520 846 / 5007 / 1199, L =
+// 32 x 19456 823 / 3623 / 976, 3D L = 8 x 2432 82 / 292 / 198, but L = 24 x 608
+// 422 / 361 / 475).
+bool resident_pays(const spin_lattice *h, int32_t pt_every) {
+  if (!planes_res_supported(h)) return false;
+  const int64_t N = h->g.N, sweeps = planes_res_tape_sweeps(h);
+  const int64_t words = (int64_t)(planes_lattice_bytes(h) / 8);  // of a colour: its threads
+  if (pt_every > 0 && pt_every <= 10 && h->g.n_temps > 1 && words <= 192) return sweeps >= 2;
+  if (h->g.dim == 2 && N == 256 && h->n_lat > 1024) return false;
+  if (h->g.dim == 3 && N == 512 && h->n_lat > 304) return false;
+  return sweeps >= (words <= 4 ? 6 : words <= 16 ? 4 : words <= 192 ? 2 : words <= 288 ? 4 : 8);
+}
+
+// The conversions of a call cost about what planes save in a few sweeps of the
+// byte kernels.  Us per call, planes / bytes.  Against the fused pass, 4
+// sweeps: one 2D L = 144 21 / 33, 20 x L = 512 30 / 49, three L = 8000 619 / 893
+// (it saves from 2 sweeps on, but for odd numbers of sweeps at least).
+constexpr int64_t kFusedMinSweeps = 4;
+// Against the colour phases in three dimensions, 2 sweeps: one L = 40 14 / 26,
+// three L = 264 198 / 202, one L = 512 293 / 409.
+constexpr int64_t kPhases3MinSweeps = 2;
+// In two dimensions small lattices wait for launches in either form, 3.5 us per
+// sweep (one L = 136 ... 760, 60 sweeps: 220 / 205), and the conversions are
+// lost: the least sweeps by the sites of all lattices (one L = 840: 6 sweeps 27 /
+// 27; one L = 1000: 3 17 / 16, 4 21 / 22; three: 2 16 / 15, 3 19 / 22; 20 x L = 184:
+// 8 38 / 36, 20 80 / 106; 20 x L = 440: 2 19 / 18, 3 22 / 27; one L = 2008: 2 18 / 18).
+int64_t phases2_min_sweeps(int64_t sites) {
+  return sites >= 3500000 ? 2 : sites >= 2400000 ? 3 : sites >= 900000 ? 4
+         : sites >= 700000  ? 6 : sites >= 550000  ? 16 : INT64_MAX;
+}
+}  // namespace
+
+PlanesForm planes_form(const spin_lattice *h, int64_t n, int32_t pt_every) {
+  if (!planes_supported(h) || h->order != SPIN_ORDER_CHECKERBOARD || n < 1) return PlanesForm::none;
+  auto phases_from = [n](int64_t least) { return n >= least ? PlanesForm::phases : PlanesForm::none; };
+  const int64_t N = h->g.N;
+  if (h->variant == 4) return phases_from(kFusedMinSweeps);
+  auto crowded = [h] { return 2 * h->n_lat > sm_count(); };
+  if (h->variant == 3) {
+    // The launch that draws the masks ahead costs what the sweeps must win back
+    // from the kernel with the lattice as bytes, about 0.14 us + 0.13 ns per site
+    // and sweep, and 12 us per exchange (us per call of 4 / 8 / 16 / 64 sweeps,
+    // bytes against planes: L = 16 5.1 / 5.5 / 8.1 / 24 against 7.3 / 7.6 / 7.7 /
+    // 16, L = 64 5.5 / 8.7 / 14 / 51 against 8.1 / 8.9 / 10 / 20, L = 128 14 / 25
+    // / 45 / 171 against 8.7 / 9.7 / 12 / 25); a little more where other lattices'
+    // CTAs are in the way (120 x L = 128: 3 sweeps 11 against 14; 152 x L = 80: 8
+    // sweeps 12 against 14; 450 x L = 32: 24 sweeps 15 against 19).
+    const double wins = (double)n * (0.14 + 0.00013 * (double)N) +
+                        (pt_every > 0 ? 12.0 * (double)(n / pt_every) : 0.0);
+    if (resident_pays(h, pt_every)) return wins >= (N >= 1024 && crowded() ? 8.0 : 5.5) ? PlanesForm::resident : PlanesForm::none;
+    // too many for the masks: the byte kernel up to L = 72 (2D) and 16 (3D), the
+    // phases above (us per call of 4 / 32 sweeps, bytes against phases: 9728 x
+    // L = 64 200 / 1338 against 262 / 1751, 4864 x L = 80 205 / 1326 against 146 /
+    // 852, x L = 128 410 / 2777 against 294 / 1760, x 3D L = 24 421 / 2847
+    // against 410 / 2601)
+    return h->auto_form && N >= 6400 ? phases_from(3) : PlanesForm::none;
+  }
+  if (!h->auto_form) return PlanesForm::none;
+  if (h->variant == 1) return phases_from(kFusedMinSweeps);
+  if (h->g.dim == 2) return phases_from(phases2_min_sweeps(h->n_lat * N));
+  // (3D L = 32: 120 lattices, 4 sweeps 27 by phases against 31, 6 sweeps 36 against 33)
+  if (resident_pays(h, pt_every) && n >= (crowded() ? 6 : kPhases3MinSweeps)) return PlanesForm::resident;
+  return phases_from(kPhases3MinSweeps);
+}
+
+PlanesForm planes_ready(spin_lattice *h, PlanesForm form, int64_t n_sweeps) {
+  if (form == PlanesForm::none || h->sweeps_done + n_sweeps > (int64_t)0xFFFFFFFFll)  // (refused by the other paths)
+    return PlanesForm::none;
+  if (form == PlanesForm::resident) {
+    if (planes_res_reserve(h, n_sweeps)) return form;
+    if (h->variant == 3) return PlanesForm::none;
+  }
+  const size_t bytes = (size_t)h->n_lat * planes_lattice_bytes(h);
+  return working_buffer(h, bytes, false) == cudaSuccess ? PlanesForm::phases : PlanesForm::none;
+}
+
+int planes_run(spin_lattice *h, PlanesForm form, const double *betas, int64_t n_sweeps, int32_t measure_every,
+               int32_t pt_every, int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels) {
+  if (form == PlanesForm::resident)
+    return run_resident(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
   if (transcode(h, true) != cudaSuccess) return SPIN_ECUDA;
   const int rc = run_phases(h, betas, n_sweeps, measure_every, pt_every, E_series, M_series, accepted, labels);
   if (rc == SPIN_ECUDA) return rc;

@@ -358,6 +358,11 @@ uint4 *tape_of(const spin_lattice *h) {
 }
 }  // namespace
 
+int64_t planes_res_tape_sweeps(const spin_lattice *h) {
+  const int64_t most = (int64_t)(kTapeMax / tape_sweep_bytes(h, make_planes(h->g.dim, h->g.L)));
+  return most / kTapeSweeps * kTapeSweeps;  // (whole groups of sweeps that are drawn together)
+}
+
 // The working buffer for calls of n sweeps; false: no memory, or a capture
 // that must not allocate.
 bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
@@ -366,8 +371,7 @@ bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
   // (calls of growing length make few buffers: a power of two, at least 512)
   int64_t sweeps = kResMinTape;
   while (sweeps < n_sweeps && sweeps < kResMaxSweeps) sweeps *= 2;
-  // (whole groups of sweeps that are drawn together)
-  sweeps = std::min(sweeps, (int64_t)(kTapeMax / per) / kTapeSweeps * kTapeSweeps);
+  sweeps = std::min(sweeps, planes_res_tape_sweeps(h));
   if (sweeps == 0) return false;
   const size_t need = planes_pair_bytes(h) + 2 * (size_t)sweeps * per;
   if (working_buffer(h, need, false) != cudaSuccess) return false;

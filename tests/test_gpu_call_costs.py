@@ -35,3 +35,26 @@ def test_masks_ahead_pay_at_one_or_two_lattices_per_sm(L, n_lat, n, part):
     assert whole < 1.2 * parts, (whole, parts)
     lat.sync()
     lat.close()
+
+
+def test_masks_ahead_stay_out_of_many_tiny_lattices():
+    lat = sp.Lattice(B.SPIN_ISING, 3, 8, B.SPIN_I8, n_temps=4, n_real=2432, seed=1)
+    betas = [0.2, 0.21, 0.22, 0.23]
+    whole = us(lambda: lat.sweep(betas, 96))
+    parts = us(lambda: [lat.sweep(betas, 8) for _ in range(12)])
+    assert whole < 1.2 * parts, (whole, parts)
+    lat.sync()
+    lat.close()
+
+
+# lattices that wait for launches in either form, one whose phases are longer
+@pytest.mark.parametrize("L,n_lat,n", [(136, 1, 3), (520, 1, 3), (440, 3, 2), (1000, 1, 2), (1000, 3, 2), (1000, 3, 4),
+                                       (264, 20, 2), (184, 20, 20)])
+def test_conversions_pay(L, n_lat, n):
+    lats = [sp.Lattice(B.SPIN_ISING, 2, L, B.SPIN_I8, n_real=n_lat, seed=1) for _ in range(2)]
+    lats[1].set_variant(0)
+    auto, phases = (us(lambda lat=lat: lat.sweep([0.4], n)) for lat in lats)
+    assert auto < 1.12 * phases, (auto, phases)
+    for lat in lats:
+        lat.sync()
+        lat.close()
