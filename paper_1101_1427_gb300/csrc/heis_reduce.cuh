@@ -22,8 +22,8 @@
 // cluster of 2, 4 or 8 CTAs per partial, whose sums rank 0 adds in rank order,
 // so that up to 512 CTAs share the work.  The rule depends on the lattice size
 // alone, so that the sums do not depend on how many lattices a call takes.  It
-// keeps 32 sites and more per thread (16 from 2^21 sites on), since the FP64
-// additions of the tree cost a thread as much as several sites: with 8 CTAs per
+// keeps 16 sites and more per thread, since the FP64 additions of the tree cost a
+// thread as much as several sites: with 8 CTAs per
 // partial, 8 lattices of L = 64 took 123 us and 4 of L = 80 68 us, with one 37
 // and 39; one of L = 80 26 against 33, of L = 100 30 against 55.
 #pragma once
@@ -67,6 +67,11 @@ struct Sum3 {
     add(p);
     low(__fmaf_rn(a, b, -p));
   }
+  __device__ __forceinline__ void add(const Sum3 &o) {
+    add(o.s);
+    low(o.c);
+    d = __fadd_rn(d, o.d);
+  }
   __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
 };
 
@@ -95,6 +100,10 @@ template <int kC>
 __device__ __forceinline__ void heis_block_partials(const float4 *__restrict__ sl, uint32_t L, const FastDiv &fL,
                                                     int dim, uint32_t N, uint32_t b, uint32_t nb,
                                                     double *__restrict__ out4) {
+  if (kC == 1 && b * (uint64_t)blockDim.x >= N) {  // no site
+    if (threadIdx.x < 4) out4[4 * b + threadIdx.x] = 0.0;
+    return;
+  }
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   // rank 0's shared memory may be written once that CTA is known to run: every
@@ -123,8 +132,27 @@ __device__ __forceinline__ void heis_block_partials(const float4 *__restrict__ s
     norm2 += h.a.x * h.a.x + h.a.y * h.a.y + h.a.z * h.a.z;
     count += 1.0f;
   }
-  double e = -(ex.value() + ey.value() + ez.value());
-  double mx = sx.value(), my = sy.value(), mz = sz.value();
+  // (the three sums of E become one before they become a double, threads convert
+  // what they have summed only, and CTAs without a site left above: a conversion
+  // is 5 FP64 operations, which lattices of a site per thread or less do not win
+  // back.  Us per measurement with all six sums converted by every thread, with
+  // FP64 sums per site, and here: 250 x 2D L = 128 429 / 332 / 336, 150 x L = 92
+  // 198 / 170 / 115, 2000 x 3D L = 8 1529 / 1415 / 145)
+  double e = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
+  if (count > 0.0f) {
+    ex.add(ey);
+    ex.add(ez);
+    e = -ex.value();
+    if (count > 1.0f) {
+      mx = sx.value();
+      my = sy.value();
+      mz = sz.value();
+    } else {  // one site: its components
+      mx = (double)sx.s;
+      my = (double)sy.s;
+      mz = (double)sz.s;
+    }
+  }
   // unit spins: norm2 = count; the whole block decides, as one site's spin
   // enters the products of its neighbours' threads too (a spin that another
   // block reads is caught there: an overflow makes e non-finite)
