@@ -271,11 +271,15 @@ __global__ void heis_renorm_kernel(float4 *__restrict__ s, int64_t total) {
   }
 }
 
-// Whether the threads of a phase draw before they wait for the previous phase
-// (up to 15 % at L = 16 to 32, 2 to 10 % on large lattices).  CTAs that start
-// early find their places while the others still run; a grid of one to three
-// CTAs per SM then lies unevenly (one L = 52, 275 CTAs: 58 instead of 48 us for
-// 10 sweeps), so it waits before it lets the next phase start.
+// Whether the threads of a phase draw before they wait for the previous phase.
+// CTAs that start early find their places while the others still run; a grid of
+// one to three CTAs per SM then lies unevenly, so it waits before it lets the next
+// phase start.  Us per 10 sweeps, late / early, by CTAs per SM: full accuracy in 3D
+// 0.8 (L = 40) 44 / 40, 1.1 47 / 55, 1.8 (L = 52) 48 / 58, 2.8 54 / 59, 3.1 (L = 62)
+// 75 / 60, 4.8 77 / 59, 11 120 / 115, 22 195 / 193; in 2D 0.8 38 / 37, 1.2 42 / 37,
+// 1.5 44 / 44, 2.5 49 / 50, 3.0 50 / 47, 3.5 68 / 52, 5.3 72 / 55, 29 217 / 214.  The
+// fast-math form on the colour-split copy gains in between too (1.8 52 / 50, 2.8
+// 57 / 53), but keeps the line of the other.
 bool draw_early(int64_t half) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
