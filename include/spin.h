@@ -33,7 +33,7 @@
  * spin_init, and one working buffer allocated by the first sweep call that
  * needs it (the fused 2D int8 pass; the bit planes of longer calls on int8
  * ferromagnets, for small lattices twice and with the acceptance masks of the
- * sweeps ahead, at most 32 MB of these; long Heisenberg calls),
+ * sweeps ahead, at most 45 MB of these; long Heisenberg calls),
  * with, for the resident 3D Heisenberg sweeps, one counter per CTA; all are
  * freed by spin_destroy.  A call that needs a longer working buffer makes one;
  * the old one is freed at once, or by spin_destroy if a call inside a stream

@@ -249,6 +249,10 @@ int spin_init(spin_lattice **out, const spin_desc *desc, void *spins, void *coup
                    ? 3
                    : (i8_2d && coded_i8_supported(h) ? 4 : (i8_2d && fused2d_supported(desc->L) ? 1 : 0));
   h->default_variant = h->variant;
+  int dev = 0;
+  h->sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
+  planes_init(h);
   const int nt = desc->n_temps;
   bool ok = cudaMalloc(&h->d_thr, 16 * (size_t)nt) == cudaSuccess &&
             cudaMalloc(&h->d_pt_off, 4 * (size_t)nt) == cudaSuccess &&
@@ -298,7 +302,7 @@ int spin_sweep(spin_lattice *h, const void *couplings, const double *betas, int6
     return SPIN_EINVAL;  // whole compound moves only, and a tile edge chosen
   int rc = upload_thresholds(h, betas);
   if (rc) return rc;
-  const PlanesForm planes = planes_ready(h, planes_form(h, n_sweeps, 0), n_sweeps);
+  const PlanesForm planes = planes_ready(h, planes_form(h, n_sweeps, 0, 0), n_sweeps);
   if (planes != PlanesForm::none)
     return planes_run(h, planes, betas, n_sweeps, 0, 0, nullptr, nullptr, nullptr, nullptr);
   cudaError_t e = h->order != SPIN_ORDER_CHECKERBOARD ? launch_sweeps_dcb(h, n_sweeps)
@@ -349,7 +353,7 @@ int spin_run(spin_lattice *h, const void *couplings, const double *betas, int64_
   if (pt_every > 0 && h->d.model == SPIN_HEISENBERG) return SPIN_EINVAL;
   const bool measuring = measure_every > 0 && (E_series || M_series || Q_series || Ef_series || Mf_series);
   const PlanesForm wanted =
-      Q_series || Ef_series || Mf_series ? PlanesForm::none : planes_form(h, n_sweeps, pt_every);
+      Q_series || Ef_series || Mf_series ? PlanesForm::none : planes_form(h, n_sweeps, measuring ? measure_every : 0, pt_every);
   if (wanted != PlanesForm::none) {
     const int rc = upload_thresholds(h, betas);
     if (rc) return rc;

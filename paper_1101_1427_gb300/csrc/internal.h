@@ -37,6 +37,7 @@ struct spin_lattice {
   void *spins;           // caller-owned
   void *couplings;       // caller-owned (may be NULL)
   int64_t n_lat;         // n_sets * n_temps * n_real lattices
+  int sms;               // of the device
   int64_t sweeps_done;
   int64_t pt_steps_done;
   int variant;           // int8 sweep: 0 phases, 1 fused, 3 resident, 4 coded
@@ -64,6 +65,9 @@ struct spin_lattice {
   bool pingpong_captured;   // a captured call has used it: it outlives its replacement
   void *d_retired[8];       // replaced working buffers that captured calls used
   int n_retired;
+  int res_words;            // words of a colour in that form, its threads (0: not for these lattices)
+  int64_t res_tape_sweeps;  // sweeps of masks that are drawn together at most
+  int res_tape_pad;         // sweeps by which their buffer is longer
   bool res_smem_set;        // the resident planes kernel may ask for its shared memory on this device
   int tape_half;         // half of the tape in it that was drawn last (planes_res.cu)
   // batched launches (options set with spin_set_batch_options)
@@ -175,7 +179,7 @@ cudaError_t planes_measure(spin_lattice *h, int64_t *E, int64_t *M);
 // the form that serves a call of n sweeps best: none (bytes), a launch per colour
 // phase, or one CTA per lattice with the masks drawn ahead
 enum class PlanesForm { none, phases, resident };
-PlanesForm planes_form(const spin_lattice *h, int64_t n_sweeps, int32_t pt_every);
+PlanesForm planes_form(const spin_lattice *h, int64_t n_sweeps, int32_t measure_every, int32_t pt_every);
 // makes the buffers ready; what can run in the place of that form (none: no
 // memory, or a capture that must not allocate)
 PlanesForm planes_ready(spin_lattice *h, PlanesForm form, int64_t n_sweeps);
@@ -194,8 +198,7 @@ struct PlanesResCall {
   int32_t *labels;
   bool bytes_in, bytes_out;  // from or to the caller's bytes instead of the planes
 };
-bool planes_res_supported(const spin_lattice *h);
-int64_t planes_res_tape_sweeps(const spin_lattice *h);  // sweeps of masks that are drawn together at most
+void planes_init(spin_lattice *h);  // res_words, res_tape_sweeps
 bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps);
 int64_t planes_res_draw(spin_lattice *h, int64_t sweep0, int64_t n, cudaError_t *err);
 cudaError_t planes_res_sweeps(spin_lattice *h, int64_t at, int64_t n, int from, const PlanesResCall &call);

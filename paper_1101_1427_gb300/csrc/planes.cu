@@ -372,38 +372,46 @@ size_t planes_lattice_bytes(const spin_lattice *h) {
 }
 
 namespace {
-int sm_count() {
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 // Whether one CTA per lattice with the masks drawn ahead (planes_res.cu) is the
 // fastest form of long calls, by the number of lattices.  What ends it is the
 // size of the masks: with few sweeps of them in a half of the buffer a call is
 // many short launches.  Us per call of 32 sweeps, here / phases / the kernel
 // with the lattice as bytes, at sweeps per half in brackets: 2D L = 8 x 38912
-// 308 / 2574 / 334 (6), x 65520 635 / 4263 / 558 (4); L = 32 x 9728 273 / 1740 /
-// 330 (6), x 19456 741 / 3303 / 658 (3); L = 64 x 4864 554 / 842 / 673 (3); L = 96
-// x 2432 621 / 727 / 873 (2); L = 128 x 608 242 / 247 / 347 (6), x 1216 558 / 482
-// / 698 (3); 3D L = 16 x 4864 592 / 995 / 815 (2); L = 24 x 304 135 / 170 / 179
-// (7), x 608 386 / 301 / 358 (3); L = 32 x 152 134 / 153 / 417 (8), x 304 286 /
-// 256 / 629 (4).  Two sizes have a byte kernel whose warps are just full and a
-// word per thread of few warps here: 2D L = 16 x 1216 18 / 247 / 15, x 9728 98 /
-// 1765 / 87; 3D L = 8 x 304 15 / 118 / 14 and 40 / 355 / 40 for 100 sweeps, x
-// 2432 66 / 223 / 55.  An exchange costs one launch here and four to five small
-// ones there, which outweighs that up to the large lattices (33 sweeps, one
-// every 8: 2D L = 16 x 9728 138 / 1950 / 216, L = 8 x 65520 846 / 5007 / 1199, L =
-// 32 x 19456 823 / 3623 / 976, 3D L = 8 x 2432 82 / 292 / 198, but L = 24 x 608
-// 422 / 361 / 475).
-bool resident_pays(const spin_lattice *h, int32_t pt_every) {
-  if (!planes_res_supported(h)) return false;
-  const int64_t N = h->g.N, sweeps = planes_res_tape_sweeps(h);
-  const int64_t words = (int64_t)(planes_lattice_bytes(h) / 8);  // of a colour: its threads
-  if (pt_every > 0 && pt_every <= 10 && h->g.n_temps > 1 && words <= 192) return sweeps >= 2;
-  if (h->g.dim == 2 && N == 256 && h->n_lat > 1024) return false;
-  if (h->g.dim == 3 && N == 512 && h->n_lat > 304) return false;
-  return sweeps >= (words <= 4 ? 6 : words <= 16 ? 4 : words <= 192 ? 2 : words <= 288 ? 4 : 8);
+// 314 / 2579 / 334 (7), x 65520 637 / 4282 / 558 (4); L = 32 x 9728 282 / 1744 /
+// 330 (7), x 19456 737 / 3299 / 655 (3); L = 64 x 4864 564 / 842 / 673 (3); L = 96
+// x 2432 627 / 727 / 873 (2); L = 112 x 1216 383 / 421 / 593 (4); L = 128 x 608 243 /
+// 249 / 347 (7), x 1024 413 / 382 / 606 (4), x 1216 560 / 479 / 693 (3); 3D L = 16 x
+// 4864 594 / 998 / 816 (2); L = 24 x 304 124 / 169 / 179 (8), x 608 260 / 300 / 356
+// (4); L = 32 x 152 150 / 150 / 418 (10), x 200 206 / 177 / 572 (7), x 304 285 / 256
+// / 629 (5).  Two sizes have a byte kernel whose warps are just full and a word
+// per thread of few warps here: 2D L = 16 x 1216 18 / 247 / 15, x 9728 99 / 1763 /
+// 86; 3D L = 8 x 304 15 / 121 / 14 and 41 / 359 / 40 for 100 sweeps, x 2432 63 / 224 /
+// 55.
+//
+// A measurement costs next to nothing here and about 8 us there (0.6 with the
+// lattice as bytes in one CTA), an exchange one launch here and four to five small
+// ones there: calls with many of them end later.  33 sweeps, an exchange every 8:
+// 2D L = 16 x 9728 137 / 1948 / 215, L = 8 x 65520 891 / 5028 / 1204, L = 32 x 19456
+// 806 / 3630 / 976, 3D L = 8 x 2432 77 / 292 / 197.  30 sweeps, here / phases,
+// nothing, E and M every 10, 5, 1 sweeps: 2D L = 128 x 2048 821 / 699, 825 / 761, 828
+// / 837, 847 / 1392; 3D L = 32 x 200 190 / 167, 192 / 201, 193 / 232, 202 / 444, x 304
+// 279 / 241, 281 / 272, 283 / 305, 291 / 514, x 452 489 / 353, 492 / 382, 495 / 417,
+// 508 / 696.
+bool resident_pays(const spin_lattice *h, int32_t measure_every, int32_t pt_every) {
+  if (!h->res_words) return false;
+  const int64_t N = h->g.N, sweeps = h->res_tape_sweeps;
+  const int words = h->res_words;
+  auto within = [](int32_t every, int most) { return every > 0 && every <= most; };
+  const int32_t swaps = h->g.n_temps > 1 ? pt_every : 0;
+  if (words <= 192) {
+    if (within(swaps, 10) || within(measure_every, 2)) return sweeps >= 2;
+    if (h->g.dim == 2 && N == 256 && h->n_lat > 1024) return false;
+    if (h->g.dim == 3 && N == 512 && h->n_lat > 304) return false;
+    return sweeps >= (words <= 4 ? 6 : words <= 16 ? 4 : 2);
+  }
+  if (sweeps >= (words <= 288 ? 4 : 8)) return true;
+  const int often = h->g.dim == 2 ? 5 : words <= 288 ? 4 : sweeps >= 4 ? 10 : 2;
+  return sweeps >= 2 && (within(swaps, often) || within(measure_every, often));
 }
 
 // The conversions of a call cost about what planes save in a few sweeps of the
@@ -425,12 +433,12 @@ int64_t phases2_min_sweeps(int64_t sites) {
 }
 }  // namespace
 
-PlanesForm planes_form(const spin_lattice *h, int64_t n, int32_t pt_every) {
+PlanesForm planes_form(const spin_lattice *h, int64_t n, int32_t measure_every, int32_t pt_every) {
   if (!planes_supported(h) || h->order != SPIN_ORDER_CHECKERBOARD || n < 1) return PlanesForm::none;
   auto phases_from = [n](int64_t least) { return n >= least ? PlanesForm::phases : PlanesForm::none; };
   const int64_t N = h->g.N;
   if (h->variant == 4) return phases_from(kFusedMinSweeps);
-  auto crowded = [h] { return 2 * h->n_lat > sm_count(); };
+  const bool crowded = 2 * h->n_lat > h->sms;
   if (h->variant == 3) {
     // The launch that draws the masks ahead costs what the sweeps must win back
     // from the kernel with the lattice as bytes, about 0.14 us + 0.13 ns per site
@@ -439,22 +447,29 @@ PlanesForm planes_form(const spin_lattice *h, int64_t n, int32_t pt_every) {
     // 16, L = 64 5.5 / 8.7 / 14 / 51 against 8.1 / 8.9 / 10 / 20, L = 128 14 / 25
     // / 45 / 171 against 8.7 / 9.7 / 12 / 25); a little more where other lattices'
     // CTAs are in the way (120 x L = 128: 3 sweeps 11 against 14; 152 x L = 80: 8
-    // sweeps 12 against 14; 450 x L = 32: 24 sweeps 15 against 19).
+    // sweeps 12 against 14; 450 x L = 32: 24 sweeps 15 against 19), unless the
+    // byte kernel's do not all fit at once (200 x 3D L = 24: 4 sweeps 27 against 19).
     const double wins = (double)n * (0.14 + 0.00013 * (double)N) +
                         (pt_every > 0 ? 12.0 * (double)(n / pt_every) : 0.0);
-    if (resident_pays(h, pt_every)) return wins >= (N >= 1024 && crowded() ? 8.0 : 5.5) ? PlanesForm::resident : PlanesForm::none;
+    const bool in_the_way = crowded && N >= 1024 && (N < 6400 || h->n_lat <= h->sms);
+    if (resident_pays(h, measure_every, pt_every))
+      return wins >= (in_the_way ? 8.0 : 5.5) ? PlanesForm::resident : PlanesForm::none;
     // too many for the masks: the byte kernel up to L = 72 (2D) and 16 (3D), the
     // phases above (us per call of 4 / 32 sweeps, bytes against phases: 9728 x
     // L = 64 200 / 1338 against 262 / 1751, 4864 x L = 80 205 / 1326 against 146 /
     // 852, x L = 128 410 / 2777 against 294 / 1760, x 3D L = 24 421 / 2847
-    // against 410 / 2601)
-    return h->auto_form && N >= 6400 ? phases_from(3) : PlanesForm::none;
+    // against 410 / 2601; with E and M after every sweep the bytes again, 30 sweeps
+    // of 2048 x 3D L = 24 1502 against 1699)
+    return h->auto_form && N >= 6400 && (measure_every < 1 || measure_every > 2) ? phases_from(3) : PlanesForm::none;
   }
   if (!h->auto_form) return PlanesForm::none;
   if (h->variant == 1) return phases_from(kFusedMinSweeps);
   if (h->g.dim == 2) return phases_from(phases2_min_sweeps(h->n_lat * N));
-  // (3D L = 32: 120 lattices, 4 sweeps 27 by phases against 31, 6 sweeps 36 against 33)
-  if (resident_pays(h, pt_every) && n >= (crowded() ? 6 : kPhases3MinSweeps)) return PlanesForm::resident;
+  // (3D L = 32: 84 lattices, 4 sweeps 25 by phases against 19, 120 27 against 31, 6
+  // sweeps 36 against 33, 4 with E and M after each 57 against 32)
+  if (resident_pays(h, measure_every, pt_every) &&
+      n >= (3 * h->n_lat > 2 * h->sms && measure_every < 1 && pt_every < 1 ? 6 : kPhases3MinSweeps))
+    return PlanesForm::resident;
   return phases_from(kPhases3MinSweeps);
 }
 

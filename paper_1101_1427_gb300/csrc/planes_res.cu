@@ -106,7 +106,10 @@ constexpr int kResRows = 32;  // measurement rows kept in shared memory before t
 // least `words` threads.  Bound by latency: about 76 instructions per phase in
 // a chain of shared-memory loads, logic and a barrier (0.10 us per phase of
 // L = 64, 0.13 us of L = 128 and of L = 64 measured after every sweep).
-template <int kDim>
+// kLong: long launches run a copy of the loop that does not look for the end (1000
+// sweeps of one L = 64 measured after each 265 -> 254 us; not in 3D, where the two
+// copies need over 96 registers).
+template <int kDim, bool kPadded, bool kLong>
 __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64_t *bytes_in, uint64_t *bytes_out,
                                                                  const uint32_t *__restrict__ src,
                                                                  uint32_t *__restrict__ dst,
@@ -161,13 +164,14 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
   const size_t chunk0 = (size_t)lat * (size_t)(N / 8);  // the lattice's first 8-byte chunk
   griddep_wait();
   griddep_release();
-  // the tape: phase p at ((p n_lat + lat) kT + e) words + word
+  // the tape: phase p at ((p n_lat + lat) kT + e) words + word; kPadded: it is
+  // longer than its sweeps by the phases fetched ahead
   const int phases = 2 * n_sweeps;
   const size_t phase_step = (size_t)n_lat * kT * words;
   const uint32_t *tp = tape + (size_t)lat * kT * words + wd;
   uint32_t mk[kAhead][kT];
-  auto fetch = [&](uint32_t (&v)[kT], bool there = true) {  // the next phase's masks, if there is one
-    if (!there) return;
+  auto fetch = [&](uint32_t (&v)[kT], bool there) {  // the next phase's masks, if there is one
+    if (!kPadded && !there) return;
 #pragma unroll
     for (int e = 0; e < kT; ++e) v[e] = tp[e * words];
     tp += phase_step;
@@ -232,7 +236,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
     rows = 0;
     __syncthreads();
   };
-  // kAhead phases from `base` on; kLast: the last ones, which fetch no more
+  // kAhead phases from `base` on; kLast: the last ones, with no more to fetch
   auto run = [&](int base, auto last_phases) {
     constexpr bool kLast = decltype(last_phases)::value;
 #pragma unroll
@@ -286,7 +290,7 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
     }
   };
   int base = 0;
-  if (phases > 8 * kAhead)  // (short launches stay with one copy of the code: 20 x L = 64 tempering 53 against 56 us)
+  if (kLong)
     for (; base + 2 * kAhead <= phases; base += kAhead) run(base, std::false_type());
   for (; base < phases; base += kAhead) run(base, std::true_type());
   if (rows) write_rows();
@@ -304,7 +308,12 @@ __global__ void __launch_bounds__(kResThreads, 1) planes_res_kernel(const uint64
   }
 }
 
-constexpr size_t kTapeMax = 16u << 20;  // bytes of one half of the tape, at most
+constexpr size_t kTapeMax = 18u << 20;  // bytes of the sweeps of one half of the tape, at most
+// Sweeps by which a half is longer than what it holds, so that no phase looks
+// whether there is another to fetch (3 to 8 % of the time per phase in 3D), where a
+// half holds kTapePadFrom sweeps or more: 9 MB for both halves at most.
+constexpr int kTapePad = 4;
+constexpr int kTapePadFrom = 16;
 constexpr int kResSpread = 200 * 1024;
 constexpr int kTapeSpread = 20 * 1024;
 
@@ -318,18 +327,26 @@ constexpr int kTapeSpread = 20 * 1024;
 // / 100 sweeps, asking for 200 KB / lattices per SM, against here: 152 x 2D L =
 // 64 9.3 / 33 / 35 / 61 and 9.2 / 12 / 18 / 56, 304 x 2D L = 16 18 / 21 / 30 /
 // 44 and 7 / 7 / 9 / 22, 152 x 2D L = 128 33 / 36 / 80 / 181 and 18 / 33 / 59 /
-// 174): there half of it and no such masks do better, and nothing at all for the
-// CTAs of 256 threads and more, of which few fit anyway.
+// 174): there no such masks and half of the share do better, or the whole where a
+// CTA has 96 threads and more, four of which on an SM are in one another's way (159 x
+// L = 80, 60 sweeps 52 against 56), and nothing at all for the CTAs of 256 threads
+// and more, of which few fit anyway (but longer launches of 3D L = 24 up to a
+// lattice per SM keep the share: 120, 100 sweeps 165 against 182, 8 sweeps 27
+// against 20).
+// Launches that do not follow their masks at once (`at` > 0: between exchanges)
+// ask for the large share again.
 struct Places {
   size_t sweeps, masks;
 };
-Places places(const spin_lattice *h, const Planes &m) {
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t per_sm = (h->n_lat + sms - 1) / sms;
-  Places p = {0, kTapeSpread};
-  if (2 * h->n_lat <= sms) p.sweeps = kResSpread;
-  else if (per_sm <= 8 && m.blocks < 64) p = {(size_t)(kResSpread / 2 / per_sm), 0};
+Places places(const spin_lattice *h, const Planes &m, int64_t at, int64_t n_sweeps) {
+  const int64_t per_sm = (h->n_lat + h->sms - 1) / h->sms;
+  const size_t share = per_sm <= 8 ? (size_t)(kResSpread / per_sm) : 0;
+  const bool crowded = 2 * h->n_lat > h->sms, small = m.blocks < 24, large = m.blocks >= 64;
+  Places p = {share, kTapeSpread};
+  if (!crowded || share == 0) return p;
+  if (!large) p.masks = 0;
+  if (at == 0 && small) p.sweeps = share / 2;
+  if (at == 0 && large) p.sweeps = per_sm == 1 && m.dim == 3 && n_sweeps >= 24 ? share : 0;
   return p;
 }
 
@@ -338,15 +355,15 @@ constexpr int64_t kResMaxSweeps = 4096;  // per launch, so that none runs for lo
 
 }  // namespace
 
-bool planes_res_supported(const spin_lattice *h) {
-  if (!planes_supported(h)) return false;
-  const Planes m = make_planes(h->g.dim, h->g.L);
-  return m.nb <= 16 && 4 * m.blocks <= kResThreads;
-}
-
 namespace {
 size_t tape_sweep_bytes(const spin_lattice *h, const Planes &m) {
   return (size_t)2 * h->n_lat * m.dim * m.blocks * sizeof(uint4);
+}
+auto res_kernel(const spin_lattice *h, int64_t n_sweeps) {
+  const bool pad = h->res_tape_pad != 0;
+  if (h->g.dim == 3) return pad ? planes_res_kernel<3, true, false> : planes_res_kernel<3, false, false>;
+  if (n_sweeps >= 32) return pad ? planes_res_kernel<2, true, true> : planes_res_kernel<2, false, true>;
+  return pad ? planes_res_kernel<2, true, false> : planes_res_kernel<2, false, false>;
 }
 // The working buffer: two buffers of planes, then the two halves of the tape.
 size_t planes_pair_bytes(const spin_lattice *h) { return 2 * (size_t)h->n_lat * planes_lattice_bytes(h); }
@@ -358,9 +375,13 @@ uint4 *tape_of(const spin_lattice *h) {
 }
 }  // namespace
 
-int64_t planes_res_tape_sweeps(const spin_lattice *h) {
-  const int64_t most = (int64_t)(kTapeMax / tape_sweep_bytes(h, make_planes(h->g.dim, h->g.L)));
-  return most / kTapeSweeps * kTapeSweeps;  // (whole groups of sweeps that are drawn together)
+void planes_init(spin_lattice *h) {
+  if (!planes_supported(h)) return;
+  const Planes m = make_planes(h->g.dim, h->g.L);
+  if (m.nb > 16 || 4 * m.blocks > kResThreads) return;
+  h->res_words = (int)(4 * m.blocks);
+  h->res_tape_sweeps = (int64_t)(kTapeMax / tape_sweep_bytes(h, m));
+  h->res_tape_pad = h->res_tape_sweeps >= kTapePadFrom ? kTapePad : 0;
 }
 
 // The working buffer for calls of n sweeps; false: no memory, or a capture
@@ -371,26 +392,31 @@ bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
   // (calls of growing length make few buffers: a power of two, at least 512)
   int64_t sweeps = kResMinTape;
   while (sweeps < n_sweeps && sweeps < kResMaxSweeps) sweeps *= 2;
-  sweeps = std::min(sweeps, planes_res_tape_sweeps(h));
-  if (sweeps == 0) return false;
-  const size_t need = planes_pair_bytes(h) + 2 * (size_t)sweeps * per;
+  sweeps = std::min(sweeps, h->res_tape_sweeps);
+  if (sweeps < kTapeSweeps) return false;
+  const size_t need = planes_pair_bytes(h) + 2 * (size_t)(sweeps + h->res_tape_pad) * per;
   if (working_buffer(h, need, false) != cudaSuccess) return false;
-  if (!h->res_smem_set)
-    h->res_smem_set = cudaFuncSetAttribute(m.dim == 3 ? planes_res_kernel<3> : planes_res_kernel<2>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, kResSpread) == cudaSuccess;
+  if (!h->res_smem_set) {
+    h->res_smem_set = true;
+    for (int64_t n : {1, 32})  // short and long launches
+      h->res_smem_set = h->res_smem_set && cudaFuncSetAttribute(res_kernel(h, n), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                                kResSpread) == cudaSuccess;
+  }
   return h->res_smem_set;
 }
 
 // The tape for the next sweeps; returns how many it covers (at most n).
 int64_t planes_res_draw(spin_lattice *h, int64_t sweep0, int64_t n, cudaError_t *err) {
   const Planes m = make_planes(h->g.dim, h->g.L);
-  int64_t cover = (int64_t)(tape_half_bytes(h) / tape_sweep_bytes(h, m)) / kTapeSweeps * kTapeSweeps;
-  cover = std::min(std::min(cover, kResMaxSweeps), n);
+  int64_t cover = (int64_t)(tape_half_bytes(h) / tape_sweep_bytes(h, m)) - h->res_tape_pad;
+  cover = std::min(cover, kResMaxSweeps);
+  // (whole groups of sweeps that are drawn together, but for the call's last ones)
+  cover = n <= cover ? n : cover / kTapeSweeps * kTapeSweeps;
   h->tape_half ^= 1;
   const int64_t groups = (cover + kTapeSweeps - 1) / kTapeSweeps;
   const int64_t threads = groups * 2 * h->n_lat * m.blocks;  // < 2^31: 16 bytes of tape each
   *err = launch_dependent(m.dim == 3 ? planes_tape_kernel<3> : planes_tape_kernel<2>, dim3(grid_for(threads, 128)),
-                          dim3(128), places(h, m).masks, h->stream, tape_of(h), m, h->g, (uint32_t)h->n_lat,
+                          dim3(128), places(h, m, 0, cover).masks, h->stream, tape_of(h), m, h->g, (uint32_t)h->n_lat,
                           make_fastdiv((uint32_t)h->n_lat), make_fastdiv(m.blocks), (const uint32_t *)h->d_thr,
                           make_round_keys(h->d.seed), (uint32_t)sweep0, (uint32_t)cover);
   return cover;
@@ -412,8 +438,8 @@ cudaError_t planes_res_sweeps(spin_lattice *h, int64_t at, int64_t n, int from, 
   s.step = call.step;
   s.accepted = (long long *)call.accepted;
   s.labels = call.labels;
-  return launch_dependent(m.dim == 3 ? planes_res_kernel<3> : planes_res_kernel<2>, dim3((unsigned)h->n_lat),
-                          dim3((4 * m.blocks + 31) / 32 * 32), places(h, m).sweeps, h->stream,
+  return launch_dependent(res_kernel(h, n), dim3((unsigned)h->n_lat),
+                          dim3((4 * m.blocks + 31) / 32 * 32), places(h, m, at, n).sweeps, h->stream,
                           (const uint64_t *)(call.bytes_in ? h->spins : nullptr),
                           (uint64_t *)(call.bytes_out ? h->spins : nullptr), (const uint32_t *)(p + (size_t)from * buf),
                           p + (size_t)(from ^ 1) * buf, (const uint32_t *)tape, m, h->g, (int)n, s, pt_tables(h),

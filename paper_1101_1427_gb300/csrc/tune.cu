@@ -73,7 +73,7 @@ extern "C" int spin_tune(spin_lattice *h, const void *couplings, const double *b
     }
     const std::pair<int, int> unset(h->default_variant + kAuto, h->order_tile);
     apply(unset);
-    if (spin::planes_form(h, n_sweeps, 0) != spin::PlanesForm::none) cand.push_back(unset);
+    if (spin::planes_form(h, n_sweeps, 0, 0) != spin::PlanesForm::none) cand.push_back(unset);
     apply(start);
   } else {
     cand.push_back(start);

@@ -58,3 +58,20 @@ def test_conversions_pay(L, n_lat, n):
     for lat in lats:
         lat.sync()
         lat.close()
+
+
+@pytest.mark.parametrize("dim,L,n_lat", [(3, 32, 200), (3, 24, 600), (2, 128, 1216)])
+def test_measuring_after_every_sweep_costs_little(dim, L, n_lat):
+    """Large lattices, too many for the masks of many sweeps: a call that measures
+    often still takes the form that measures in place."""
+    lat = sp.Lattice(B.SPIN_ISING, dim, L, B.SPIN_I8, n_real=n_lat, seed=1)
+    series = lat.series_buffers(30)
+
+    def run(every):
+        B.spin_run(lat.h, None, [0.3], 30, every, 0, *((series["E"], series["M"]) if every else (None, None)), None, None,
+                   None, None, None)
+
+    plain, measured = us(lambda: run(0)), us(lambda: run(1))
+    assert measured < 1.6 * plain, (plain, measured)
+    lat.sync()
+    lat.close()
