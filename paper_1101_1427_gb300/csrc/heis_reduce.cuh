@@ -14,18 +14,18 @@
 // product is split without error into its rounded value and the remainder
 // (one FMA), and each addition passes its rounding error (Knuth's two-sum)
 // to the next term.  The expansion carries 72 bits, more than a double, and
-// becomes a double once per thread: about 40 us, and a call of 20 sweeps and
-// one measurement at L = 128 went from 601 to 388 us.  Sums whose spins are far from unit
-// length, where an FP32 product could overflow or vanish, are formed in FP64.
+// becomes a double once per thread: about 36 us, and a call of 20 sweeps and one
+// measurement at L = 128 went from 601 to 384 us.  Sums whose spins are far from
+// unit length, where an FP32 product could overflow or vanish, are formed in FP64.
 //
 // A lattice has kHeisParts partials whatever its size; large lattices take a
 // cluster of 2, 4 or 8 CTAs per partial, whose sums rank 0 adds in rank order,
 // so that up to 512 CTAs share the work.  The rule depends on the lattice size
 // alone, so that the sums do not depend on how many lattices a call takes.  It
 // keeps 16 sites and more per thread, since the FP64 additions of the tree cost a
-// thread as much as several sites: with 8 CTAs per
-// partial, 8 lattices of L = 64 took 123 us and 4 of L = 80 68 us, with one 37
-// and 39; one of L = 80 26 against 33, of L = 100 30 against 55.
+// thread as much as several sites: with 8 CTAs per partial, 8 lattices of L = 64
+// took 123 us and 4 of L = 80 68 us, with one 37 and 39; one of L = 80 26 against
+// 33, of L = 100 30 against 55.
 #pragma once
 #include <cooperative_groups.h>
 #include <stdint.h>

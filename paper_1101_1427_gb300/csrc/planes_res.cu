@@ -13,8 +13,8 @@
 // exchange step is folded into the start of the next launch: each CTA decides
 // its pair from the energies the last launch left and loads its partner's
 // planes instead of its own where the exchange is accepted.  One L = 64, 1000
-// sweeps with E and M after each 1335 -> 265 us; 20 x L = 64, 100 sweeps and 10
-// exchanges 181 -> 55 us; 20 x 3D L = 16, 256 sweeps 234 -> 63 us.
+// sweeps with E and M after each 1335 -> 256 us; 20 x L = 64, 100 sweeps and 10
+// exchanges 181 -> 54 us; 20 x 3D L = 16, 256 sweeps 234 -> 63 us.
 #include <algorithm>
 #include <type_traits>
 
@@ -103,9 +103,10 @@ constexpr int kResRows = 32;  // measurement rows kept in shared memory before t
 // exchange, the partner's) to bytes_out (the last launch) or the planes `dst`.
 // Thread i holds word i (4 block + plane) of both colours in registers and
 // publishes them in shared memory for its neighbours.  Grid: lattices; at
-// least `words` threads.  Bound by latency: about 76 instructions per phase in
-// a chain of shared-memory loads, logic and a barrier (0.10 us per phase of
-// L = 64, 0.13 us of L = 128 and of L = 64 measured after every sweep).
+// least `words` threads.  Bound by latency: about 61 instructions per phase, a
+// measurement included, in a chain of shared-memory loads, logic and a barrier
+// (0.10 us per phase of L = 64, 0.13 us of L = 128 and of L = 64 measured after
+// every sweep).
 // kLong: long launches run a copy of the loop that does not look for the end (1000
 // sweeps of one L = 64 measured after each 265 -> 254 us; not in 3D, where the two
 // copies need over 96 registers).

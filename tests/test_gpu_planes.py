@@ -1,7 +1,9 @@
 """Longer calls of int8 ferromagnets on bit planes (one or several rows per
 block, pieces and row groups whose last is smaller, one to three lattices per
 thread) against twin handles held to the in-place colour phases: lattices,
-series, exchanges and labels, over calls of several lengths and schedules."""
+series, exchanges and labels, over calls of several lengths and schedules.  (2D
+handles of few sites stay on bytes; test_gpu_planes_routes.py has the narrow
+planes of those sizes, with more lattices.)"""
 import pytest
 
 torch = pytest.importorskip("torch")
