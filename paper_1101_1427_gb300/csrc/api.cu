@@ -352,8 +352,9 @@ int spin_run(spin_lattice *h, const void *couplings, const double *betas, int64_
   if (!h || n_sweeps < 0) return SPIN_EINVAL;
   if (pt_every > 0 && h->d.model == SPIN_HEISENBERG) return SPIN_EINVAL;
   const bool measuring = measure_every > 0 && (E_series || M_series || Q_series || Ef_series || Mf_series);
-  const PlanesForm wanted =
-      Q_series || Ef_series || Mf_series ? PlanesForm::none : planes_form(h, n_sweeps, measuring ? measure_every : 0, pt_every);
+  const PlanesForm wanted = Q_series || Ef_series || Mf_series
+                                ? PlanesForm::none
+                                : planes_form(h, n_sweeps, measuring ? measure_every : 0, pt_every);
   if (wanted != PlanesForm::none) {
     const int rc = upload_thresholds(h, betas);
     if (rc) return rc;

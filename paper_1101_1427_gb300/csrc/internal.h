@@ -184,8 +184,8 @@ PlanesForm planes_form(const spin_lattice *h, int64_t n_sweeps, int32_t measure_
 // memory, or a capture that must not allocate)
 PlanesForm planes_ready(spin_lattice *h, PlanesForm form, int64_t n_sweeps);
 // the call (SPIN_* status), spin_run without Q; counters advanced
-int planes_run(spin_lattice *h, PlanesForm form, const double *betas, int64_t n_sweeps, int32_t measure_every, int32_t pt_every,
-               int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels);
+int planes_run(spin_lattice *h, PlanesForm form, const double *betas, int64_t n_sweeps, int32_t measure_every,
+               int32_t pt_every, int64_t *E_series, int64_t *M_series, int64_t *accepted, int32_t *labels);
 
 // planes_res.cu: the same for lattices small enough for one CTA each
 struct PlanesResCall {

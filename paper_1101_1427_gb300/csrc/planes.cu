@@ -416,8 +416,8 @@ bool resident_pays(const spin_lattice *h, int32_t measure_every, int32_t pt_ever
 
 // The conversions of a call cost about what planes save in a few sweeps of the
 // byte kernels.  Us per call, planes / bytes.  Against the fused pass, 4
-// sweeps: one 2D L = 144 21 / 33, 20 x L = 512 30 / 49, three L = 8000 619 / 893
-// (it saves from 2 sweeps on, but for odd numbers of sweeps at least).
+// sweeps: one 2D L = 144 21 / 33, 20 x L = 512 30 / 49, three L = 8000 619 / 893;
+// 2 sweeps 13 / 17, 21 / 25, 381 / 446: the line could lie lower.
 constexpr int64_t kFusedMinSweeps = 4;
 // Against the colour phases in three dimensions, 2 sweeps: one L = 40 14 / 26,
 // three L = 264 198 / 202, one L = 512 293 / 409.

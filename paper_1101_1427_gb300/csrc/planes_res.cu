@@ -14,7 +14,7 @@
 // its pair from the energies the last launch left and loads its partner's
 // planes instead of its own where the exchange is accepted.  One L = 64, 1000
 // sweeps with E and M after each 1335 -> 256 us; 20 x L = 64, 100 sweeps and 10
-// exchanges 181 -> 54 us; 20 x 3D L = 16, 256 sweeps 234 -> 63 us.
+// exchanges 181 -> 55 us; 20 x 3D L = 16, 256 sweeps 234 -> 63 us.
 #include <algorithm>
 #include <type_traits>
 
@@ -400,8 +400,9 @@ bool planes_res_reserve(spin_lattice *h, int64_t n_sweeps) {
   if (!h->res_smem_set) {
     h->res_smem_set = true;
     for (int64_t n : {1, 32})  // short and long launches
-      h->res_smem_set = h->res_smem_set && cudaFuncSetAttribute(res_kernel(h, n), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                                kResSpread) == cudaSuccess;
+      h->res_smem_set =
+          h->res_smem_set && cudaFuncSetAttribute(res_kernel(h, n), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  kResSpread) == cudaSuccess;
   }
   return h->res_smem_set;
 }
