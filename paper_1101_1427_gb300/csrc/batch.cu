@@ -895,7 +895,8 @@ struct Tuned {
 };
 static std::map<std::vector<long long>, Tuned> g_tuned;  // autotuner cache, by batch signature
 
-static constexpr double kEaFixedUs = 13.0, kLatticeUs = 0.45, kQuadUs = 1.0e-3, kSiteUs = 2.0e-3, kUnstaged = 1.6;
+static constexpr double kEaFixedUs = 13.0, kLatticeUs = 0.45, kQuadUs = 1.0e-3, kSiteUs = 2.0e-3;
+static constexpr double kQuadUnstaged = 1.6, kSiteUnstaged = 1.1;
 
 // Time of one sweep of a unit with a team of P CTAs, with measurement and
 // exchange every sweep, in us (fitted to the times at which the units of the
@@ -910,7 +911,9 @@ static double unit_time(const BatchUnit &U, int P, double ising_scale, double ea
   if (U.kind == 0) {
     const int W = U.n_T * U.n_sets;
     const int owned = P <= U.n_T ? (U.n_T + P - 1) / P * U.n_sets : (W + P - 1) / P;
-    const double per_site = (U.L % 8 != 0 ? kSiteUs : kQuadUs) * (3u * U.N > 12288u ? kUnstaged : 1.0);
+    const bool unstaged = 3u * U.N > 12288u;
+    const double per_site = U.L % 8 != 0 ? kSiteUs * (unstaged ? kSiteUnstaged : 1.0)
+                                           : kQuadUs * (unstaged ? kQuadUnstaged : 1.0);
     return kEaFixedUs + owned * (kLatticeUs + per_site * ((double)U.N + ea_n0));
   }
   const double rows = (U.L + P - 1) / P;

@@ -342,8 +342,16 @@ __device__ __forceinline__ Flip ea_site_flip(const EaSiteW &x, const EaSiteJ &c,
 
 // One colour phase of the chunks [c0, c1) (128 consecutive colour indices
 // each) of one 3D word-lattice by a warp: lane l draws the call of quad l of a
-// chunk, and sites 32 s + l take their words from lane 8 s + l / 4.  add(f, on) receives each site's Flip and whether the lane has
-// a site.
+// chunk, and sites 32 s + l take their words from lane 8 s + l / 4.  add(f, on)
+// receives each site's Flip and whether the lane has a site.
+//   Bound by the latency of the loads (words in L2, couplings there too from
+// L = 18 on): two sites at a time, all fourteen words and their couplings
+// before the first store.  The words of four sites first and then the
+// couplings of each waits for L2 five times a chunk, and four sites with
+// couplings spill.  Us per 8 sweeps, groups x slots of two sets (four sites'
+// words first / two sites): L = 28 64 x 8 2052 / 1341, 2 x 8 313 / 218; L = 30
+// 16 x 31 2108 / 1588; L = 20 64 x 8 599 / 513; couplings staged: L = 12 32 x 8
+// 89 / 87, L = 14 16 x 32 199 / 194.
 template <typename AddFn>
 __device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, int colour,
                                                uint32_t L, uint32_t N, const FastDiv &fL, const RoundKeys &rk,
@@ -352,29 +360,29 @@ __device__ __forceinline__ void ea_sites_phase(uint32_t *__restrict__ w, const u
   const uint32_t half = N >> 1, lane = threadIdx.x & 31u, wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
   const uint32_t end = min(128u * c1, half);
   for (uint32_t base = 128u * c0; base < end; base += 128u) {
-    // the words of the four sites first, so that their latencies overlap
-    EaSite e[4];
-    EaSiteW x[4];
-#pragma unroll
-    for (uint32_t s = 0; s < 4; ++s) {
-      e[s] = ea_site<3>(min(base + 32u * s + lane, half - 1), colour, L, fL);
-      x[s] = ea_site_words<3>(w, e[s], colour, N);
-    }
     const uint4 v = philox(make_uint4((base >> 2) + lane, sweep, lid, wctr), rk);
 #pragma unroll
-    for (uint32_t s = 0; s < 4; ++s) {
-      const uint32_t from = 8u * s + (lane >> 2);
-      const uint32_t r0 = __shfl_sync(0xffffffffu, v.x, from), r1 = __shfl_sync(0xffffffffu, v.y, from);
-      const uint32_t r2 = __shfl_sync(0xffffffffu, v.z, from), r3 = __shfl_sync(0xffffffffu, v.w, from);
-      const uint32_t r = (lane & 2u) ? ((lane & 1u) ? r3 : r2) : ((lane & 1u) ? r1 : r0);
-      const uint32_t j = base + 32u * s + lane;
-      const bool on = j < half;
-      Flip f = {};
-      if (on) {
-        f = ea_site_flip<3>(x[s], ea_site_couplings<3>(J, e[s], colour, N), r, t4, t8, t12);
-        w[(uint32_t)colour * half + j] = x[s].S ^ f.F;
+    for (uint32_t s0 = 0; s0 < 4; s0 += 2) {
+      EaSiteW x[2];
+      EaSiteJ c[2];
+#pragma unroll
+      for (uint32_t k = 0; k < 2; ++k) {
+        const EaSite e = ea_site<3>(min(base + 32u * (s0 + k) + lane, half - 1), colour, L, fL);
+        x[k] = ea_site_words<3>(w, e, colour, N);
+        c[k] = ea_site_couplings<3>(J, e, colour, N);
       }
-      add(f, on);
+#pragma unroll
+      for (uint32_t k = 0; k < 2; ++k) {
+        const uint32_t s = s0 + k, from = 8u * s + (lane >> 2);
+        const uint32_t r0 = __shfl_sync(0xffffffffu, v.x, from), r1 = __shfl_sync(0xffffffffu, v.y, from);
+        const uint32_t r2 = __shfl_sync(0xffffffffu, v.z, from), r3 = __shfl_sync(0xffffffffu, v.w, from);
+        const uint32_t r = (lane & 2u) ? ((lane & 1u) ? r3 : r2) : ((lane & 1u) ? r1 : r0);
+        const uint32_t j = base + 32u * s + lane;
+        const bool on = j < half;
+        const Flip f = ea_site_flip<3>(x[k], c[k], r, t4, t8, t12);
+        if (on) w[(uint32_t)colour * half + j] = x[k].S ^ f.F;
+        add(f, on);
+      }
     }
   }
 }

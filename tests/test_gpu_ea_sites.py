@@ -41,6 +41,23 @@ def test_batched_sites_equal_per_handle_runs(L, n_real, T):
         lat.close()
 
 
+# last chunks of 128 sites that hold 100, 76, 84 and 60, couplings not staged
+@pytest.mark.parametrize("L", [18, 22, 26, 30])
+def test_batched_sites_with_couplings_in_l2_equal_per_handle_runs(L):
+    lats = [sp.Lattice(B.SPIN_EA, 3, L, B.SPIN_MSC1, n_real=64, n_temps=3, n_sets=2, seed=5) for _ in range(2)]
+    betas = [0.5, 0.8, 1.1]
+    for n, me, pt in ((2, 0, 0), (3, 1, 1)):
+        ref = lats[0].run(betas, n, measure_every=me, pt_every=pt)
+        ser = lats[1].series_buffers(3) if me else None
+        sp.batch_run([lats[1].batch_item(betas, ser)], n, me, pt)
+        for key in ref:
+            assert torch.equal(ref[key], ser[key]), key
+        assert torch.equal(lats[0].spins, lats[1].spins)
+    for lat in lats:
+        lat.sync()
+        lat.close()
+
+
 @pytest.mark.parametrize("dim,L,n_real,T", [(2, 6, 32, 3), (2, 16, 64, 2), (2, 50, 32, 2), (2, 90, 32, 1), (3, 4, 32, 2),
                                             (3, 8, 32, 2), (3, 12, 64, 3), (3, 18, 32, 2), (3, 26, 32, 1)])
 def test_counts_and_bytes_equal_bytes(dim, L, n_real, T):
