@@ -1137,9 +1137,20 @@ constexpr int kResidentSmem = 212 * 1024;
 // those loads at 16 warps per SM.  For batches of EA units alone whose
 // word-lattices are small enough that most of a CTA's fit (32 KB at L = 20),
 // and whose units are large enough for three CTAs and more each (a unit takes
-// whole CTAs) but have no more CTAs than slots.  1024 x 32 x 2 of L = 16, 8
-// sweeps with E, M, Q and an exchange after each: 523 -> 485 us.  A batch whose
-// least teams need more CTAs than there are SMs only fits two to an SM.
+// whole CTAs) but have no more CTAs than slots.  A batch whose least teams need
+// more CTAs than there are SMs only fits two to an SM.  Otherwise the form with
+// less work on its fullest SM: word-sites of the CTA with the most slots and
+// what the barriers of one CTA leave idle (as much as 2100 of them), 0.87 (0.91
+// from L = 18 on) of the time per word-site of two CTAs, of which one has the
+// most slots and one an average share.  Us per 8 sweeps with E, M, Q and an
+// exchange after each, one / two CTAs per SM, groups x slots of two sets:
+//   L = 8   20 x 60 231 / 171, 40 x 32 234 / 205, 48 x 33 239 / 248
+//   L = 10  12 x 32 202 / 178, 28 x 60 414 / 444
+//   L = 12  28 x 16 251 / 227, 28 x 60 556 / 608, 40 x 32 512 / 483
+//   L = 16  32 x 32 474 / 520, 40 x 32 655 / 624, 48 x 33 664 / 803
+//   L = 20  28 x 16 678 / 609, 12 x 32 558 / 611, 40 x 60 3446 / 3028
+// Of 112 shapes with 8 <= L <= 20 it takes the slower one by more than 3 % in
+// five, 7 % at most.
 static bool resident_preferred(const BatchParams &prm, int sms) {
   double total = 0.0;
   int least = 0;
@@ -1150,12 +1161,19 @@ static bool resident_preferred(const BatchParams &prm, int sms) {
     least += least_team(U);
   }
   if (least > sms) return false;
+  double one = 0.0, two = 0.0;  // work of the fullest SM with one, with two CTAs
   for (int u = 0; u < prm.n_units; ++u) {
     const BatchUnit &U = prm.units[u];
-    const double share = sms * (double)U.n_sets * U.n_T * U.N / total;
+    const int W = U.n_sets * U.n_T;
+    const double share = sms * (double)W * U.N / total, slot = (double)U.n_sets * U.N;
     if (share < 3.0 || share > (double)U.n_T) return false;
+    const int P1 = (int)share, P2 = std::min((int)(2.0 * share), W);
+    const int m1 = (U.n_T + P1 - 1) / P1;
+    const double m2 = P2 <= U.n_T ? (U.n_T + P2 - 1) / P2 : (double)((W + P2 - 1) / P2) / U.n_sets;
+    one = std::max(one, (U.N <= 4096u ? 0.87 : 0.91) * (m1 * slot + 2100.0));
+    two = std::max(two, (m2 + (double)U.n_T / P2) * slot);
   }
-  return true;
+  return one < two;
 }
 
 static bool resident(const BatchParams &prm) { return prm.smem_words > prm.staged_words; }

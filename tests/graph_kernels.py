@@ -1,6 +1,7 @@
 """Names of the kernels that a call enqueues, in order of first appearance: the
 call is captured into a CUDA graph (which runs nothing) and the graph is
 written out as text."""
+import gc
 import re
 import warnings
 
@@ -11,8 +12,13 @@ def kernels(torch, stream, call, path):
     g = torch.cuda.CUDAGraph(keep_graph=True)
     g.enable_debug_mode()
     torch.cuda.synchronize()
-    with torch.cuda.graph(g, stream=stream):
-        call()
+    gc.collect()  # lattices of earlier tests free their buffers, which ends a capture
+    gc.disable()
+    try:
+        with torch.cuda.graph(g, stream=stream):
+            call()
+    finally:
+        gc.enable()
     with warnings.catch_warnings():
         warnings.simplefilter("ignore")
         g.debug_dump(str(path))
