@@ -490,11 +490,20 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
   }
   // EA coded words: parts of kRowThreads (or kRowThreadsFew) threads per
   // word-lattice, at most kRowItems groups of four sites per thread; with one
-  // part per word-lattice the counts are stored, not added, and need no zeroing
+  // part per word-lattice the counts are stored, not added, and need no zeroing.
+  // kRowThreads leave no thread idle up to 1024 sites, and beyond that fill the
+  // GPU from about five word-lattices per SM on, except where one part of
+  // kRowThreadsFew holds the lattice and kRowThreads need several.  E, M and Q
+  // in us, 64 / 256 threads, L x word-lattices: 8 x 2048 6.6 / 9.0, 12 x 512
+  // 10.8 / 10.1, 12 x 1024 13.2 / 16.2, 18 x 1536 55.8 / 48.8, 28 x 1024 123 /
+  // 132.  A lattice of several parts has as many as give two CTAs to an SM: 28 x
+  // 4 in 2 parts 21.6, in 22 parts 9.1; at 128 word-lattices 2 parts are best.
   const int64_t n_wl = (int64_t)g.n_sets * (g.n_real / 32) * g.n_temps;
-  const bool few = n_wl < 152 * 10;
-  const int per_part = (few ? kRowThreadsFew : kRowThreads) * kRowItems;
-  const unsigned gx = (unsigned)((g.N / 4 + per_part - 1) / per_part);
+  const bool few = g.N > 1024 && (n_wl < 5 * h->sms || (g.N > 4096 && g.N <= 4 * kRowThreadsFew * kRowItems));
+  const int threads = few ? kRowThreadsFew : kRowThreads;
+  int64_t parts = (g.N / 4 + threads * kRowItems - 1) / (threads * kRowItems);
+  if (parts > 1) parts = std::max(parts, std::min((g.N / 4 + threads - 1) / threads, 2 * h->sms / n_wl));
+  const unsigned gx = (unsigned)parts;
   const bool coded_direct = h->d.layout == SPIN_MSC1 && gx == 1;
   if (!coded_direct) {
     if (E) cudaMemsetAsync(E, 0, sizeof(int64_t) * nl, st);
@@ -535,8 +544,8 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
       {{measure_msc_rows_kernel<3, false, kRowThreads>, measure_msc_rows_kernel<3, false, kRowThreadsFew>},
        {measure_msc_rows_kernel<3, true, kRowThreads>, measure_msc_rows_kernel<3, true, kRowThreadsFew>}}};
   const Kern kern = kerns[g.dim == 3][quads][few];
-  return launch_dependent(kern, dim3(gx, (unsigned)n_wl), dim3(few ? kRowThreadsFew : kRowThreads), 0, st, (const uint32_t *)h->spins,
-                          (const uint32_t *)J, g, (long long *)E, (long long *)M,
+  return launch_dependent(kern, dim3(gx, (unsigned)n_wl), dim3((unsigned)threads), 0, st,
+                          (const uint32_t *)h->spins, (const uint32_t *)J, g, (long long *)E, (long long *)M,
                           (g.n_sets >= 2) ? (long long *)Q : nullptr);
 }
 
