@@ -95,12 +95,14 @@ __device__ __forceinline__ EaItem ea_item(const Geom &g, uint32_t k, const FastD
 // uniforms, keyed by q.  ftb divides by the number of slot blocks.  Register
 // bound: two CTAs per SM (the coupling words stay live across the slots).
 // The geometry does not depend on the previous phase and comes before
-// griddep_wait().
+// griddep_wait(); the next phase starts only then, since the CTAs of several
+// phases that wait at once lie unevenly on the SMs.  10 sweeps in us, release
+// first / here: 3D L = 8 32 groups x 33 slots x 2 (0.95 CTAs per SM) 95 / 68, 2D
+// L = 40 14 x 33 (1.3) 89 / 65; 4 CTAs per SM and more are equal.
 template <int kDim, bool kPair>
 __global__ void __launch_bounds__(256, 2)
     msc_phase_kernel(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, Geom g, uint32_t total,
                      FastDiv ftb, const uint32_t *__restrict__ thr, RoundKeys rk, uint32_t sweep, int colour) {
-  griddep_release();
   const uint32_t N = (uint32_t)g.N, wctr = ctr_w(TAG_UPDATE, (uint32_t)colour, 0);
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= total) return;
@@ -109,6 +111,7 @@ __global__ void __launch_bounds__(256, 2)
   uint32_t *ws = w + (size_t)x.st * (uint32_t)g.n_temps * N;  // slot t of (a, grp) is word-lattice st T + t
   const EaQuadGeom q = ea_quad_geom<kDim>(x.j4, colour, (uint32_t)g.L, g.fL);
   griddep_wait();
+  griddep_release();
   const EaQuadJ c = ea_quad_couplings<kDim>(J + (size_t)x.grp * kDim * N, q, colour, N);
 #pragma unroll 1
   for (uint32_t t = x.t0; t < x.t1; ++t) {
@@ -126,12 +129,12 @@ __global__ void __launch_bounds__(256, 2)
 // A thread per quad and slot read its words four apart from the next lane's and
 // looked up each site's geometry and couplings again for every slot: 10 sweeps
 // of 256 x 30 x 2 lattices of L = 12 with 2 measurements and exchanges took 151
-// us, 135 here.
+// us, 135 here.  Draws before griddep_wait(), the next phase after it (10 sweeps
+// in us, next phase first / here: 3D L = 18 20 x 4 x 2, 1.5 CTAs per SM, 73 / 49).
 template <int kDim, bool kPair>
 __global__ void __launch_bounds__(256)
     msc_site_phase_kernel(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, Geom g, uint32_t total,
                           FastDiv ftb, const uint32_t *__restrict__ thr, RoundKeys rk, uint32_t sweep, int colour) {
-  griddep_release();
   const uint32_t N = (uint32_t)g.N;
   const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x, lane4 = id & 3u;
   const EaItem x = ea_item(g, min(id >> 2, total - 1), ftb);  // (lanes beyond the end draw the last quad again)
@@ -151,6 +154,7 @@ __global__ void __launch_bounds__(256)
   const EaSite e = ea_site<kDim>(j, colour, (uint32_t)g.L, g.fL);
   uint32_t *ws = w + (size_t)x.st * (uint32_t)g.n_temps * N;
   griddep_wait();
+  griddep_release();
   const EaSiteJ c = ea_site_couplings<kDim>(J + (size_t)x.grp * kDim * N, e, colour, N);
   // all slots' words first, so that their latencies overlap
   EaSiteW v[kSlots];
@@ -173,14 +177,16 @@ __global__ void __launch_bounds__(256)
 // instead of a launch.  Items, draws and updates are those of the phase kernels.
 // Bound by the latency of a phase in one CTA (L = 12: 1.9 us for two sites per
 // thread in four slots, 3.6 with a launch per phase): 10 sweeps of 256 x 30 x 2
-// lattices of L = 12 with 2 measurements and exchanges 116 -> 100 us.
+// lattices of L = 12 with 2 measurements and exchanges 116 -> 100 us.  The next
+// kernel starts after griddep_wait(): CTAs of several calls that wait at once
+// pile up on some SMs (10 sweeps of 50 x 4 x 2 lattices of 2D L = 60 100 us, 70
+// here).
 template <int kDim, bool kPair, bool kRow>
 __global__ void __launch_bounds__(kResThreads)
     msc_res_kernel(uint32_t *__restrict__ w, const uint32_t *__restrict__ J, Geom g, FastDiv ftb,
                    const uint32_t *__restrict__ thr, RoundKeys rk, uint32_t sweep0, uint32_t n_sweeps) {
   extern __shared__ uint4 msc_res_smem[];
   __shared__ uint32_t s_thr[kSlots][4];
-  griddep_release();
   const uint32_t N = (uint32_t)g.N, half = N / 2, quads = (half + 3) / 4, lane4 = threadIdx.x & 3u;
   const uint32_t G = (uint32_t)g.n_real / 32, T = (uint32_t)g.n_temps, TB = (T + kSlots - 1) / kSlots;
   const uint32_t st = fdiv(blockIdx.x, ftb), a = fdiv(st, g.fgrp), grp = st - a * G;
@@ -190,6 +196,7 @@ __global__ void __launch_bounds__(kResThreads)
   uint32_t *ws = w + ((size_t)st * T + t0) * N;
   const uint32_t *gJ = J + (size_t)grp * kDim * N;
   griddep_wait();
+  griddep_release();
 #pragma unroll 8
   for (uint32_t i = threadIdx.x; i < n_slots * N; i += blockDim.x) sw[i] = ws[i];
 #pragma unroll 8
