@@ -63,6 +63,7 @@ struct NoAdd {
 constexpr int kResThreads = 512;    // at most, msc_res_kernel
 constexpr int64_t kResSweeps = 1024;  // sweeps per launch
 constexpr size_t kResSmem = 227 * 1024 - 64;  // beside its thresholds
+constexpr int kSmSmem = 228 * 1024;           // of an SM, 1 KB of it per CTA the system's
 constexpr uint32_t kSlots = 4;  // slots of one (set, group) per thread of a colour phase
 
 // Place of thread item k: (a, grp) and the first slot of its block, with the
@@ -324,6 +325,15 @@ cudaError_t launch_couplings_msc(spin_lattice *h) {
 }
 
 namespace {
+// Shared memory that a grid asks for so that at most ceil(ctas / sms) of its
+// CTAs fit on an SM (to 16 of them): a kernel that starts while another one
+// still runs fills the free places first, and several of its CTAs would share
+// one SM while others idle.
+size_t spread_smem(int64_t ctas, int sms) {
+  const int64_t per_sm = (ctas + sms - 1) / sms;
+  return per_sm <= 16 ? (size_t)(kSmSmem / (per_sm + 1) - 1024 + 128) : 0;
+}
+
 using ResKern = decltype(&msc_res_kernel<3, false, false>);
 
 // Sweeps of a call with the lattices in shared memory (msc_res_kernel): CTAs,
@@ -347,8 +357,7 @@ MscRes msc_res_plan(const spin_lattice *h, int64_t n_sweeps) {
   MscRes p;
   const size_t smem = (size_t)(kSlots + (uint32_t)g.dim) * (size_t)g.N * 4;
   if (n_sweeps < 3 || smem > kResSmem) return p;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = h->sms;
   const bool row = g.L % 8 == 0;
   const uint32_t quads = (uint32_t)((g.N / 2 + 3) / 4), items = row ? quads : 4 * quads;
   const uint32_t rounds = (items + kResThreads - 1) / kResThreads;
@@ -360,11 +369,11 @@ MscRes msc_res_plan(const spin_lattice *h, int64_t n_sweeps) {
   const double here = 7.0 + 0.17 * (double)smem / 4.0 / threads * per_sm +
                       n * sweep * std::max(1.0, per_sm * threads / 448.0);
   const double lat = row ? 2.0 + 1.1 * std::min(kSlots, T) : 3.3;
-  const double words = (row ? 3.35e-6 : 5.3e-6) * d * (double)st * T * (double)g.N;
+  const double words = (row ? 3.6e-6 : 4.8e-6) * d * (double)st * T * (double)g.N;
   if (here > 0.95 * (3.5 + n * (std::max(lat, words) + 0.5 * std::min(lat, words)))) return p;
   p.grid = st * TB;
   p.threads = threads;
-  p.smem = smem;
+  p.smem = std::min(std::max(smem, spread_smem(p.grid, sms)), kResSmem);
   return p;
 }
 }  // namespace
@@ -398,10 +407,21 @@ cudaError_t launch_sweeps_msc_ea(spin_lattice *h, const uint32_t *J, int64_t n_s
     return e;
   }
   const int64_t threads = row_quads ? work : 4 * (int64_t)work;  // < 2^30: fewer than 2^27 words
+  const int grid = (int)grid_for(threads, 256);
+  // Up to two CTAs per SM one more on some SMs counts; beyond, three and four
+  // at a time are faster.  10 sweeps in us with an exchange and E, M, Q after every
+  // second, as they fall / spread: 2D L = 40, 33 slots, 0.9 CTAs per SM 156 / 143,
+  // 1.7 206 / 178; 3D L = 16, 32 slots, 0.8 169 / 149, 1.9 197 / 197; L = 12, 33 slots, 2.0
+  // 138 / 122; 2D L = 64, 4 slots, 1.1 140 / 144, 1.9 186 / 165.
+  const size_t smem = grid <= 2 * h->sms ? spread_smem(grid, h->sms) : 0;
+  if (smem) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
+    if (e != cudaSuccess) return e;
+  }
   for (int64_t k = 0; k < n_sweeps; ++k) {
     const uint32_t sweep = (uint32_t)(h->sweeps_done + k);
     for (int colour = 0; colour < 2; ++colour) {
-      const cudaError_t e = launch_dependent(kern, dim3(grid_for(threads, 256)), dim3(256), 0, h->stream,
+      const cudaError_t e = launch_dependent(kern, dim3(grid), dim3(256), smem, h->stream,
                                              (uint32_t *)h->spins, J, g, work, ftb, (const uint32_t *)h->d_thr,
                                              rk, sweep, colour);
       if (e != cudaSuccess) return e;

@@ -11,7 +11,8 @@ from paper_1101_1427_gb300 import _binding as B  # noqa: E402
 
 
 @pytest.mark.parametrize("dim,L,groups,T", [(3, 8, 2, 33), (2, 40, 4, 16), (3, 16, 2, 5), (3, 10, 3, 6), (3, 18, 4, 4),
-                                            (2, 30, 8, 5), (2, 60, 6, 3), (2, 16, 40, 5)])
+                                            (2, 30, 8, 5), (2, 60, 6, 3), (2, 16, 40, 5), (2, 32, 6, 33),
+                                            (2, 40, 18, 33), (3, 12, 5, 33), (3, 16, 9, 16), (3, 16, 10, 16)])
 def test_calls_back_to_back_equal_bytes(dim, L, groups, T):
     betas = [0.3 + 0.05 * t for t in range(T)]
     lats = [sp.Lattice(B.SPIN_EA, dim, L, layout, n_real=32 * groups, n_temps=T, n_sets=2, seed=6)
