@@ -491,18 +491,23 @@ cudaError_t launch_measure(spin_lattice *h, const void *J, int64_t *E, int64_t *
   // EA coded words: parts of kRowThreads (or kRowThreadsFew) threads per
   // word-lattice, at most kRowItems groups of four sites per thread; with one
   // part per word-lattice the counts are stored, not added, and need no zeroing.
-  // kRowThreads leave no thread idle up to 1024 sites, and beyond that fill the
-  // GPU from about five word-lattices per SM on, except where one part of
-  // kRowThreadsFew holds the lattice and kRowThreads need several.  E, M and Q
-  // in us, 64 / 256 threads, L x word-lattices: 8 x 2048 6.6 / 9.0, 12 x 512
-  // 10.8 / 10.1, 12 x 1024 13.2 / 16.2, 18 x 1536 55.8 / 48.8, 28 x 1024 123 /
-  // 132.  A lattice of several parts has as many as give two CTAs to an SM: 28 x
-  // 4 in 2 parts 21.6, in 22 parts 9.1; at 128 word-lattices 2 parts are best.
+  // More threads for few word-lattices of more than 512 sites, and where one part
+  // of them holds the lattice and kRowThreads need several.  4 sweeps in us with E,
+  // M, Q after each, 64 / 256 threads, L x word-lattices: 2D 20 x 1024 54 / 63, 28 x
+  // 768 61 / 61, 28 x 1280 76 / 88, 3D 12 x 768 101 / 96, 12 x 1024 116 / 114, 16 x 1280
+  // 174 / 169, 12 x 2048 165 / 208, 18 x 2048 529 / 507, 26 x 1024 764 / 779.
+  // A lattice of several parts has as many as give two CTAs to an SM (E, M and Q
+  // alone of 28 x 4 in 2 parts 21.6, in 22 parts 9.1), and so has a lattice of one
+  // part where its latency outweighs the zeroing: 4 sweeps with an exchange
+  // after each, one / several parts, 20 x 4 69 / 47, 20 x 96 109 / 87, 16 x 96 66 / 73;
+  // with E, M, Q after each 22 x 96 125 / 113, 20 x 96 100 / 104, 24 x 96 89 / 113.
   const int64_t n_wl = (int64_t)g.n_sets * (g.n_real / 32) * g.n_temps;
-  const bool few = g.N > 1024 && (n_wl < 5 * h->sms || (g.N > 4096 && g.N <= 4 * kRowThreadsFew * kRowItems));
+  const bool one = g.N <= 4 * kRowThreadsFew * kRowItems;
+  const bool few = g.N > 512 && (g.N > 4096 && one ? true : n_wl < (g.N > 1024 && one ? 8 : 5) * h->sms);
   const int threads = few ? kRowThreadsFew : kRowThreads;
   int64_t parts = (g.N / 4 + threads * kRowItems - 1) / (threads * kRowItems);
-  if (parts > 1) parts = std::max(parts, std::min((g.N / 4 + threads - 1) / threads, 2 * h->sms / n_wl));
+  if (parts > 1 || (g.N > 4096 && !M && !Q) || (g.N > 8192 && g.L % 8 != 0))
+    parts = std::max(parts, std::min((g.N / 4 + threads - 1) / threads, 2 * h->sms / n_wl));
   const unsigned gx = (unsigned)parts;
   const bool coded_direct = h->d.layout == SPIN_MSC1 && gx == 1;
   if (!coded_direct) {
