@@ -392,14 +392,28 @@ cudaError_t launch_sweeps_msc_ea(spin_lattice *h, const uint32_t *J, int64_t n_s
                                {{msc_site_phase_kernel<3, false>, msc_phase_kernel<3, false>},
                                 {msc_site_phase_kernel<3, true>, msc_phase_kernel<3, true>}}};
   const Kern kern = kerns[g.dim == 3][pair][row_quads];
+  const ResKern res_kerns[2][2][2] = {{{msc_res_kernel<2, false, false>, msc_res_kernel<2, false, true>},
+                                       {msc_res_kernel<2, true, false>, msc_res_kernel<2, true, true>}},
+                                      {{msc_res_kernel<3, false, false>, msc_res_kernel<3, false, true>},
+                                       {msc_res_kernel<3, true, false>, msc_res_kernel<3, true, true>}}};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  static OncePerDevice limits;
+  if (!limits.done(dev)) {
+    for (int k = 0; k < 8; ++k) {
+      cudaError_t e = cudaFuncSetAttribute(kerns[k >> 2][k >> 1 & 1][k & 1],
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(res_kerns[k >> 2][k >> 1 & 1][k & 1], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kResSmem);
+      if (e != cudaSuccess) return e;
+    }
+    limits.mark(dev);
+  }
   const MscRes res = msc_res_plan(h, n_sweeps);
   if (res.grid) {
-    const ResKern res_kerns[2][2][2] = {{{msc_res_kernel<2, false, false>, msc_res_kernel<2, false, true>},
-                                         {msc_res_kernel<2, true, false>, msc_res_kernel<2, true, true>}},
-                                        {{msc_res_kernel<3, false, false>, msc_res_kernel<3, false, true>},
-                                         {msc_res_kernel<3, true, false>, msc_res_kernel<3, true, true>}}};
     const ResKern kern = res_kerns[g.dim == 3][pair][row_quads];
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
+    cudaError_t e = cudaSuccess;
     for (int64_t k = 0; e == cudaSuccess && k < n_sweeps; k += kResSweeps)
       e = launch_dependent(kern, dim3(res.grid), dim3(res.threads), res.smem, h->stream, (uint32_t *)h->spins, J, g,
                            ftb, (const uint32_t *)h->d_thr, rk, (uint32_t)(h->sweeps_done + k),
@@ -414,10 +428,6 @@ cudaError_t launch_sweeps_msc_ea(spin_lattice *h, const uint32_t *J, int64_t n_s
   // 1.7 206 / 178; 3D L = 16, 32 slots, 0.8 169 / 149, 1.9 197 / 197; L = 12, 33 slots, 2.0
   // 138 / 122; 2D L = 64, 4 slots, 1.1 140 / 144, 1.9 186 / 165.
   const size_t smem = grid <= 2 * h->sms ? spread_smem(grid, h->sms) : 0;
-  if (smem) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
-    if (e != cudaSuccess) return e;
-  }
   for (int64_t k = 0; k < n_sweeps; ++k) {
     const uint32_t sweep = (uint32_t)(h->sweeps_done + k);
     for (int colour = 0; colour < 2; ++colour) {
