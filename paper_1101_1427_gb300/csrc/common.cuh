@@ -286,7 +286,7 @@ __host__ __device__ __forceinline__ int slot_of(const Geom &g, int64_t lat) {
 // may start while the previous kernel of its stream is finishing: it calls
 // griddep_wait() before touching memory, which returns once that kernel has
 // completed and its writes are visible.  griddep_release() lets the next
-// such kernel's CTAs be scheduled once every CTA of this grid has started
+// such kernel's CTAs be scheduled once every CTA of this grid has called it or ended
 // (they wait in griddep_wait() until this grid is done).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_release() { asm volatile("griddepcontrol.launch_dependents;"); }

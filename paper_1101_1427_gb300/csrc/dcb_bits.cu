@@ -205,7 +205,19 @@ cudaError_t launch_t(spin_lattice *h, int coarse, uint32_t sweep0) {
   const int B = h->g.L / kT;
   const int64_t threads = (int64_t)B * B / 2 * BitTile<kT, kR>::kLanes;
   const dim3 grid((unsigned)((threads + kBitThreads - 1) / kBitThreads), (unsigned)h->n_lat);
-  return launch_dependent(dcb_bits_kernel<kT, kR, kS>, grid, dim3(kBitThreads), 0, h->stream, (int8_t *)h->spins,
+  // even shares of grids that fit at once (us for 100 hits on three L = 1440, as
+  // the CTAs fall / spread: T = 8 619 / 537, T = 16 668 / 584)
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  static OncePerDevice limit;
+  if (!limit.done(dev)) {
+    const cudaError_t e = cudaFuncSetAttribute(dcb_bits_kernel<kT, kR, kS>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)spread_smem(1, 1));
+    if (e != cudaSuccess) return e;
+    limit.mark(dev);
+  }
+  const size_t smem = spread_smem((int64_t)grid.x * grid.y, h->sms);
+  return launch_dependent(dcb_bits_kernel<kT, kR, kS>, grid, dim3(kBitThreads), smem, h->stream, (int8_t *)h->spins,
                           h->g.L, coarse, sweep0, h->order_hits, (const uint32_t *)h->d_thr, h->g,
                           make_round_keys(h->d.seed));
 }
@@ -218,13 +230,16 @@ cudaError_t launch_t(spin_lattice *h, int coarse, uint32_t sweep0) {
 // byte form 387 / 444 / 1275 / 1869 / 4833, 4 rows per thread 413 / 413 /
 // 1116 / 1468 / 3711, 16 rows 784 / 783 / 1210 / 1505 / 3496; T = 8 (8 rows)
 // at 2048 / 6144 / 8192: byte form 158 / 391 / 453, here 229 / 366 / 367.
-// T = 64: 2 rows beat 4 up to 98304 units (3527 against 3727).
+// T = 64: 2 rows beat 4 up to 98304 units (3527 against 3727); byte form and
+// here at 9600 / 11616 / 13824 / 16224 units 514 / 499, 629 / 732, 743 / 732, 858 /
+// 734.
 namespace {
 int64_t units(const spin_lattice *h) { return h->n_lat * (h->g.N / 512); }
 }  // namespace
 
 bool dcb_bits_preferred(const spin_lattice *h) {
-  return h->g.dim == 2 && h->order_tile <= 64 && units(h) >= (h->order_tile == 8 ? 6144 : 8192);
+  const int64_t least = h->order_tile == 8 ? 6144 : h->order_tile == 64 ? 13500 : 8192;
+  return h->g.dim == 2 && h->order_tile <= 64 && units(h) >= least;
 }
 
 cudaError_t launch_dcb_bits(spin_lattice *h, int coarse, uint32_t sweep0) {

@@ -241,6 +241,15 @@ cudaError_t launch_dcb_bits(spin_lattice *h, int coarse, uint32_t sweep0);
 // batch.cu: load the batch kernel's device counters from the host counters
 int sync_device_counters(spin_lattice *h, cudaStream_t st);
 
+// Dynamic shared memory that a grid asks for so that at most ceil(ctas / sms) of
+// its CTAs fit on an SM (to 16 of them): a kernel that starts while another one
+// still runs fills the free places first, and several of its CTAs would share one
+// SM while others idle.  An SM has 228 KB, 1 KB of it per CTA the system's.
+inline size_t spread_smem(int64_t ctas, int sms) {
+  const int64_t per_sm = (ctas + sms - 1) / sms;
+  return per_sm <= 16 ? (size_t)(228 * 1024 / (per_sm + 1) - 1024 + 128) : 0;
+}
+
 inline unsigned grid_for(int64_t n, int block) {
   int64_t g = (n + block - 1) / block;
   return (unsigned)(g < 1 ? 1 : g);

@@ -231,7 +231,7 @@ __device__ __forceinline__ int warp_count(const uint32_t (&C)[kRP]) {
   return cnt;
 }
 
-// grid: (blocks per word-lattice, word-lattices), kRowThreads threads; the
+// grid: (blocks per word-lattice, word-lattices), kThreads threads; the
 // register bound lets 14 blocks share an SM.
 template <int kDim, bool kQuads, int kThreads>
 __global__ void __launch_bounds__(kThreads, 896 / kThreads) measure_msc_rows_kernel(const uint32_t *__restrict__ w,

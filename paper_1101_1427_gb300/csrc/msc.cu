@@ -63,7 +63,6 @@ struct NoAdd {
 constexpr int kResThreads = 512;    // at most, msc_res_kernel
 constexpr int64_t kResSweeps = 1024;  // sweeps per launch
 constexpr size_t kResSmem = 227 * 1024 - 64;  // beside its thresholds
-constexpr int kSmSmem = 228 * 1024;           // of an SM, 1 KB of it per CTA the system's
 constexpr uint32_t kSlots = 4;  // slots of one (set, group) per thread of a colour phase
 
 // Place of thread item k: (a, grp) and the first slot of its block, with the
@@ -325,15 +324,6 @@ cudaError_t launch_couplings_msc(spin_lattice *h) {
 }
 
 namespace {
-// Shared memory that a grid asks for so that at most ceil(ctas / sms) of its
-// CTAs fit on an SM (to 16 of them): a kernel that starts while another one
-// still runs fills the free places first, and several of its CTAs would share
-// one SM while others idle.
-size_t spread_smem(int64_t ctas, int sms) {
-  const int64_t per_sm = (ctas + sms - 1) / sms;
-  return per_sm <= 16 ? (size_t)(kSmSmem / (per_sm + 1) - 1024 + 128) : 0;
-}
-
 using ResKern = decltype(&msc_res_kernel<3, false, false>);
 
 // Sweeps of a call with the lattices in shared memory (msc_res_kernel): CTAs,

@@ -12,6 +12,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 import paper_1101_1427_gb300 as sp  # noqa: E402
+from graph_kernels import kernels  # noqa: E402
 from paper_1101_1427_gb300 import _binding as B  # noqa: E402
 
 
@@ -35,3 +36,24 @@ def test_bit_tiles_equal_the_oracle(T, L, n_lat, hits, order):
         oracle.dcb_sweeps(L, s, betas[t], 17, lid, 0, 2 * hits, T, hits, symmetric=order == B.SPIN_ORDER_DCB_SYMMETRIC)
         assert np.array_equal(got[t], s.ravel()), t
     lat.close()
+
+
+# n_lat L^2 / 512 on both sides of 6144, 8192 and 13500
+@pytest.mark.parametrize("T,L,n_lat,bits", [(8, 256, 47, False), (8, 256, 48, True), (16, 256, 63, False),
+                                            (32, 256, 64, True), (64, 384, 46, False), (64, 384, 47, True)])
+def test_form_and_equal_to_the_oracle_at_the_line(T, L, n_lat, bits, tmp_path):
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        lat = sp.Lattice(B.SPIN_ISING, 2, L, B.SPIN_I8, n_temps=n_lat, seed=19)
+        lat.set_update_order(B.SPIN_ORDER_DCB, T, 2)
+        betas = [0.4407] * n_lat
+        lat.sweep(betas, 2)
+        lat.sync()
+        got = lat.spins.cpu().numpy().reshape(n_lat, -1)[n_lat - 1]
+        lid = oracle.lattice_id(0, 0, n_lat - 1)
+        s = oracle.ising_init(2, L, 19, lid)
+        oracle.dcb_sweeps(L, s, 0.4407, 19, lid, 0, 2, T, 2, symmetric=False)
+        assert np.array_equal(got, s.ravel())
+        names = kernels(torch, stream, lambda: lat.sweep(betas, 2), tmp_path / "graph.dot")
+        assert any("dcb_bits" in name for name in names) == bits, names
+        lat.close()
