@@ -245,7 +245,8 @@ def config_rooflines(side, i8_value, sms, mhz):
         out[name] = line(side.get(key), heis, f"{HEIS_WIDE_MULS_PER_FLIP} wide multiplies (one Philox call)",
                          mul_basis, "heis_resident_kernel (100-sweep calls)")
     out["3d_ea_L16_sweep"] = line(side.get("ea_L16_w32_sweep_flips_per_ns"), ea_sweep,
-                                  f"{EA_SWEEP_ALU_PER_WORD}/32 logic ops", alu_basis, "msc_phase_kernel")
+                                  f"{EA_SWEEP_ALU_PER_WORD}/32 logic ops", alu_basis,
+                                  "msc_res_kernel (calls of 40 sweeps)")
     out["3d_ea_L16_pt_per_handle"] = line(side.get("ea_L16_pt_plain_flips_per_ns"), ea_pt,
                                           f"{EA_PT_ALU_PER_WORD}/32 logic ops", alu_basis,
                                           "msc_phase_kernel + measure_msc_rows_kernel + pt kernels")
